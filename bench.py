@@ -41,11 +41,11 @@ import p3m_synth as S  # noqa: E402
 METRIC = "P3M particle-updates/s"
 UNIT = "particle-updates/s"
 # algorithmic FP32 flops per accepted pair of the short-range sum: the FP32 arithmetic of the
-# FP32 kernel's accepted-pair sequence, FMA = 2: d 3 FADD; r^2 3 FFMA; r^2 + eps^2 FADD;
-# s^3 = rsqrt * rcp FMUL; r^3 = r^2 sqrt(r^2) FMUL; tau FFMA; the degree-8 Horner chain 8 FFMA;
-# g = 1 + r^3 p FFMA; f = g s^3 FMUL; a += f d 3 FFMA  ->  16 FFMA + 7 FADD/FMUL = 39 flops
-# (sqrt, rsqrt and rcp run on the MUFU pipe and are not counted)
-FLOPS_PER_PAIR = 39
+# FP32 kernel's accepted-pair sequence, FMA = 2: d 3 FADD; r^2 + eps^2 3 FFMA; s + b FADD; the
+# (1 - t)/r^2 term FFMA; s^2 FMUL; its product and the constant FFMA; the cubic in t 3 FFMA;
+# a += f d 3 FFMA  ->  11 FFMA + 5 FADD/FMUL = 27 flops (rsqrt and ex2 run on the MUFU pipe and
+# are not counted)
+FLOPS_PER_PAIR = 27
 # the same for the FP64 kernel: d 6 DADD (difference plus image); r^2 DMUL + 2 DFMA; r^2 + eps^2
 # DADD; r^3 = r^2 (r^2 rsqrt(r^2)) 2 DMUL; tau DFMA; the degree-18 Horner chain 18 DFMA;
 # g DFMA; s^3 and g s^3 3 DMUL; a += f d 3 DFMA  ->  25 DFMA + 13 DADD/DMUL = 63 flops

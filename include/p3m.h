@@ -100,12 +100,13 @@ typedef struct {
     uint64_t launches;    /* kernels this library launched on the stream since p3m_init
                              (cuFFT's own kernels not included)                             */
     uint64_t pair_warp_j[3]; /* pair kernel work since p3m_init, in warp-iterations over one
-                             j particle (32 pair slots each): [0] in chunks entirely inside
-                             r_c of every i of the warp, [1] in chunks tested pair by pair,
-                             [2] tested ones that some i accepted                          */
+                             j particle (32 pair slots each).  FP64 mode: [0] in chunks entirely
+                             inside r_c of every i of the warp, [1] in chunks tested pair by
+                             pair, [2] tested ones that some i accepted.  FP32 mode: [0] 0, [1] j's
+                             tested against the box of a group of i's, [2] those evaluated    */
     uint64_t pair_blocks_culled; /* 32-particle j blocks skipped by the bounding-box test     */
-    uint64_t pair_tiles[2];  /* j tiles streamed through shared memory; [1] of them entirely
-                                culled                                                       */
+    uint64_t pair_tiles[2];  /* FP64 mode: j tiles streamed through shared memory; [1] of them
+                                entirely culled.  FP32 mode: j lists evaluated; 0              */
     int64_t n;            /* number of particles                                            */
     int32_t n_cells_side; /* chaining cells per side n_c                                    */
     int32_t max_cell_count; /* most particles in one chaining cell (last sort)              */
@@ -245,10 +246,10 @@ int p3m_ensemble_set_batched(p3m_ensemble *ens, int enable);
 int p3m_ensemble_set_fft_groups(p3m_ensemble *ens, int enable);
 
 /*
- * Autotuner of the sort key's Hilbert depth and of the FP32 pair kernel's tile length: times two
+ * Autotuner of the sort key's Hilbert depth and of the FP32 pair kernel's list length: times two
  * force evaluations of the current particles for each sub_bits in 0..3 whose key fits in 32 bits
  * (ms_out[b], nullable; NaN when skipped), keeps the fastest (*sub_bits_out), then (FP32 P3M
- * contexts) times tiles of 3 and 5 blocks of 32 j particles at that depth and keeps the faster,
+ * contexts) times lists of 3 and 5 blocks of 32 j particles at that depth and keeps the faster,
  * and leaves valid forces.  The cells, and hence which pairs interact, do not depend on either
  * choice; the forces agree up to the FP32 rounding of a different summation order.
  * p3m_get_tuning reports the current choices (tile_blocks: 3 or 5; 5 by default).

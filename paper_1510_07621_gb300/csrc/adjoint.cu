@@ -399,14 +399,6 @@ __global__ void __launch_bounds__(32)
 constexpr float kVjpTiny = 1e-20f;
 constexpr int kVjpBlocksPerTile = 3;
 
-// 2^x (MUFU); here x in [-7.3, 0], no denormal results
-__device__ __forceinline__ float ex2_approx(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 struct VjpConst2 {
     f2 c[P3M_SPLIT_DEG + 1];
     f2 c11, m1, one, eps2, tiny, ex2arg, c1, m3;

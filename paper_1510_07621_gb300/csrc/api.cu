@@ -154,6 +154,119 @@ void fit_split_poly64(double cutoff_in_rs, double r_s, double *out)
     out[P3M_SPLIT_DEG64 + 1] = 2.0 / (uc * r_s * r_s);
 }
 
+// ---------------------------------------------------------------- FP32 pair factor fit
+// g - 1 = r^3 Q with (lengths in r_s, u = r^2, t = exp(-kappa u))
+//   Q ~ alpha (1 - t)/u + c0 + c1 t + c2 t^2 + c3 t^3,
+// whose first term carries Q's slow tail.  At kappa = 0.0757 this follows Q to 6e-9 of the force
+// scale up to the cutoff 4.5 (2.8e-8 at 4.8, 3.6e-7 at 6), where the degree-8 polynomial in u had
+// 2.5e-7 (6.4e-7, 1.2e-5), needs one MUFU operation beside s = (u + eps^2)^-1/2 and no
+// cancelling terms.  (The general form below takes one more power of t, at kappa = 0.0574: a large
+// softening damps the force at small r, and with it the scale that the error is compared with.)  The
+// error that counts in the force is |df| r; beside it a relative error of f
+// itself counts.  Least squares with the weights raised where the error is largest; a few kappa
+// around the quoted ones are tried, the best kept.
+// Additive form: with w = u + eps^2 in place of u,
+//   g w^-3/2 = w^-3/2 + b/w + alpha (1 - t)/w + c0 + c1 t + c2 t^2 + c3 t^3,
+// b/w = -3/2 eps^2 Q(0)/w the leading softening term of Q(u) (u/w)^3/2.  What it leaves out, of
+// order eps^4/w^2, is a relative error of f of at most 0.046 (eps/r_s)^3, reached at r ~ eps.
+PairFactor fit_pair_factor(double cutoff_in_rs, const P3MGeom &g)
+{
+    constexpr int kMax = 6, kN = 48;
+    const double xc = cutoff_in_rs, r0 = xc < 1.0 ? 0.1 * xc : 0.4;
+    const double eps = g.eps / g.r_s;
+    // 0.046 eps^3 <= 1.6e-6: at r ~ eps the FP32 rounding of the pair distance is larger
+    const bool additive = eps <= 0.0326 && xc >= 2.0;  // (shorter cutoffs leave the fit ill-conditioned)
+    const int kM = additive ? 5 : 6;  // alpha, c0 .. c3 (general form: .. c4)
+    const double soft = additive ? eps * eps : 0.0;
+    const double bw = 1.5 * soft * 0.094031597257959381;  // Q(0) = -1/(6 sqrt(pi))
+    double w[kN], tgt[kN], wt[kN], best[kMax] = {}, best_err = 1e300, kappa = 0.0;
+    for (int i = 0; i < kN; ++i) {
+        const double r = r0 + 0.5 * (xc - r0) * (1.0 - cos(M_PI * (i + 0.5) / kN)), u = r * r;
+        const double q = split_q(u), g = 1.0 + u * r * q;
+        w[i] = u + soft;
+        const double ratio = u / w[i];
+        tgt[i] = q * ratio * sqrt(ratio) - bw / w[i];
+        // (general form: df = dQ r^3 s^3, which a large softening damps at small r)
+        const double s2 = u + eps * eps, rs = sqrt(u / s2);
+        wt[i] = (additive ? 1.0 : rs * rs * rs) / (1.0 / r + 2.0 * g / (s2 * sqrt(s2)));
+    }
+    for (int ik = 0; ik < 12; ++ik) {  // the value quoted above, then steps of 0.3 % to both sides
+        const double k = (additive ? 0.0757 : 0.0574) * (1.0 + 0.003 * ((ik + 1) / 2) * (ik & 1 ? 1 : -1));
+        double v[kN][kMax], lw[kN], x[kMax], emax = 0.0;
+        for (int i = 0; i < kN; ++i) {
+            const double t = exp(-k * w[i]);
+            v[i][0] = -expm1(-k * w[i]) / w[i];
+            v[i][1] = 1.0;
+            for (int q = 2; q < kM; ++q) v[i][q] = v[i][q - 1] * t;
+            lw[i] = 1.0;
+        }
+        for (int it = 0; it < 12; ++it) {
+            // weighted least squares by Householder reflections (the columns are nearly dependent
+            // for small cutoffs, so no normal equations)
+            double a[kN][kMax + 1];
+            for (int i = 0; i < kN; ++i) {
+                const double s = wt[i] * sqrt(lw[i]);
+                for (int q = 0; q < kM; ++q) a[i][q] = s * v[i][q];
+                a[i][kM] = s * tgt[i];
+            }
+            for (int q = 0; q < kM; ++q) {
+                double nrm = 0.0;
+                for (int i = q; i < kN; ++i) nrm += a[i][q] * a[i][q];
+                nrm = a[q][q] > 0.0 ? -sqrt(nrm) : sqrt(nrm);
+                double h[kN], hh = 0.0;
+                for (int i = q; i < kN; ++i) {
+                    h[i] = a[i][q] - (i == q ? nrm : 0.0);
+                    hh += h[i] * h[i];
+                }
+                for (int c = q; c <= kM && hh > 0.0; ++c) {
+                    double dot = 0.0;
+                    for (int i = q; i < kN; ++i) dot += h[i] * a[i][c];
+                    dot *= 2.0 / hh;
+                    for (int i = q; i < kN; ++i) a[i][c] -= dot * h[i];
+                }
+            }
+            for (int q = kM - 1; q >= 0; --q) {
+                x[q] = a[q][kM];
+                for (int c = q + 1; c < kM; ++c) x[q] -= a[q][c] * x[c];
+                x[q] /= a[q][q];
+            }
+            double err[kN];
+            emax = 0.0;
+            for (int i = 0; i < kN; ++i) {
+                err[i] = -tgt[i];
+                for (int q = 0; q < kM; ++q) err[i] += x[q] * v[i][q];
+                err[i] = fabs(err[i]) * wt[i];
+                emax = fmax(emax, err[i]);
+            }
+            if (!(emax > 1e-12)) break;
+            for (int i = 0; i < kN; ++i) lw[i] *= err[i] / emax + 1e-3;
+        }
+        if (!(emax < best_err)) continue;
+        best_err = emax;
+        kappa = k;
+        memcpy(best, x, sizeof(best));
+        if (emax < 1e-8) break;  // far below the FP32 rounding
+    }
+    const double rho = sqrt(kappa * 1.4426950408889634);  // scaled lengths per r_s: t = 2^-w
+    PairFactor p;
+    memset(&p, 0, sizeof(p));
+    for (int k = 0; k + 1 < kM; ++k) p.c[k] = (float)(best[k + 1] / (rho * rho * rho));
+    p.na = (float)(-best[0] / rho);
+    p.ab = (float)((best[0] + bw) / rho);
+    const double e2 = eps * eps * rho * rho, rc2 = xc * xc * rho * rho;
+    p.e2 = (float)(additive ? fmax(e2, 1e-24) : e2);  // (r = 0 pairs stay finite)
+    p.rc2 = (float)(additive ? rc2 + e2 : rc2);
+    p.rlist2 = (float)(rc2 * (1.0 + 2e-5));
+    p.length = (float)(g.r_s / rho);
+    p.lambda = (float)(ldexp(g.cs, -kFixBits) * rho / g.r_s);
+    p.cell = (float)g.cs;
+    // (accelerations scale with length^-2; lambda's FP32 rounding is the unit that the kernel uses)
+    const double len = ldexp(g.cs, -kFixBits) / (double)p.lambda;
+    p.scale = g.gm / (len * len);
+    p.additive = additive ? 1 : 0;
+    return p;
+}
+
 // ---------------------------------------------------------------- phase timing
 
 void harvest(p3m_ctx *c)
@@ -185,7 +298,7 @@ void release(p3m_ctx *c)
                     c->tab_one,   c->ps_acc,   c->fac_table,    c->step_idx, c->cur_fac,
                     c->tab_origin,
                     c->adj_u,     c->adj_vfx,  c->adj_vs,       c->adj_out,  c->kself,
-                    c->li,        c->relx,     c->sort_status,  c->sort_hist,
+                    c->li,        c->relx,     c->relq,     c->sort_status,  c->sort_hist,
                     c->rho_fix,   c->fix_exp,  c->ps_part,     c->sort_probe};
     for (void *p : bufs)
         if (p) cudaFree(p);
@@ -600,6 +713,7 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
             {(void **)&c->rel, 4 * real * N}, {(void **)&c->keys, 4 * N},
             {(void **)&c->block_box, 32 * ((N + 31) / 32)},
             {(void **)&c->relx, opt.precision == P3M_PREC_MIXED ? 384 * ((N + 31) / 32) : 16},
+            {(void **)&c->relq, opt.precision == P3M_PREC_MIXED ? 384 * ((N + 31) / 32) : 16},
             {(void **)&c->keys_alt, 4 * N},   {(void **)&c->vals, 4 * N},
             {(void **)&c->vals_alt, 4 * N},   {(void **)&c->digit_counts, 4 * 256 * (size_t)c->n_tiles},
             {(void **)&c->scan_aux, 4 * (scan_n / P3M_SORT_TILE + 4)},
@@ -665,6 +779,7 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
         }
         c->green_const = -4.0 * M_PI * (g.gm / (h * h * h)) / ((double)M3);
         fit_split_poly(cutoff_in_rs, g.r_s, c->gpoly);
+        c->pair_factor = fit_pair_factor(cutoff_in_rs, g);
         fit_split_poly64(cutoff_in_rs, g.r_s, c->gpoly64);
         if (c->precision == P3M_PREC_MIXED) {
             std::vector<float> f(M);

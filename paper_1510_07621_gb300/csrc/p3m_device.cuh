@@ -87,6 +87,14 @@ __device__ __forceinline__ float rsqrt_approx(float x)
     return y;
 }
 
+// 2^x (MUFU)
+__device__ __forceinline__ float ex2_approx(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // Packed two-lane FP32 values (f32x2) through the compiler's own float2 builtins, so that
 // register pairs and scheduling are the compiler's to choose.
 typedef float2 f2;

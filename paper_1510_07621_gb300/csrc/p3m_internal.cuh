@@ -17,6 +17,26 @@
 // 4e-14 relative (at r_c), far below the FP64 mode's 1e-12 parity bar.
 #define P3M_SPLIT_DEG64 18
 
+// Fixed-point coordinates of the FP32 pair kernels: 2^-kFixBits of a chaining cell, modulo 2^32
+// (8 cells), so that differences of particles in neighbouring cells are exact integers.
+constexpr int kFixBits = 29;
+constexpr float kFixUnit = 0x1p-29f;
+
+// The FP32 pair factor f(r) = g(r/r_s) (r^2 + eps^2)^-3/2 in scaled lengths (see fit_pair_factor):
+// one unit is `length`, chosen so that t = 2^-w is the exponential of the fit, w the squared
+// scaled distance.  With s = (w + softening)^-1/2 and P(t) = c[0] + c[1] t + c[2] t^2 + c[3] t^3:
+//   additive:  w includes the softening (e2): f = s^3 + (ab + na t) s^2 + P(t); rc2 bounds w
+//   otherwise: f = s^3 (1 + r (ab + na t + r^2 P(t))), r without the softening; rc2 bounds r^2
+struct PairFactor {
+    float c[5];
+    float na, ab, e2, rc2;
+    float rlist2;        // squared radius of the candidate test (a little above the cutoff)
+    float lambda;        // scaled lengths per fixed-point unit
+    float cell, length;  // side of a chaining cell; one scaled length
+    double scale;        // accelerations = scale * sum f d
+    int additive;
+};
+
 // Chaining-cell geometry, mesh constants and the per-evaluation scalars every kernel needs.
 struct P3MGeom {
     double box;       // L
@@ -71,7 +91,8 @@ struct p3m_ctx {
     void *rel;  // float4 (mixed) or double4_16a (fp64): position relative to its cell origin
     float4 *block_box;  // per 32-slot block of the sorted order: lo, hi (FP32, absolute)
     float *relx;        // FP32 mode: rel as block-SoA, per 32-slot block x[32] y[32] z[32]
-    int tile_blocks;    // FP32 pair kernel: 32-slot blocks per shared-memory tile (3 or 5)
+    uint32_t *relq;     // FP32 mode: fixed-point coordinates (kFixBits), per 32-slot block x[32] y[32] z[32]
+    int tile_blocks;    // FP32 pair kernel: its list is evaluated every 32 tile_blocks entries (3 or 5)
 
     // sort
     uint32_t *keys, *keys_alt, *vals, *vals_alt;
@@ -111,6 +132,7 @@ struct p3m_ctx {
     double green_const;
     float gpoly[12];  // FP32 split factor: g = 1 + r^3 Q(tau), Q = sum gpoly[k] tau^k
                       // (k <= P3M_SPLIT_DEG), tau = r^2 gpoly[11] - 1
+    PairFactor pair_factor;  // of the FP32 force kernel
     double gpoly64[P3M_SPLIT_DEG64 + 2];  // the same in FP64 (degree P3M_SPLIT_DEG64); the
                                           // last entry is tau's scale
     cufftHandle plan_r2c, plan_c2r, plan_c2r_one;  // R2C, batched 3 x C2R, single C2R
@@ -177,6 +199,8 @@ enum {
 #define P3M_MAX_GRAPH_STEPS 4096  // steps per p3m_run_steps / p3m_ensemble_run call
 #define P3M_SORT_TILE 4096   // keys per radix-sort tile (256 threads x 16)
 #define P3M_PAIR_TI 32       // i-particles per pair work item (one per lane of a warp)
+#define P3M_PAIR_GROUP 16    // particles of a work item that share one list (FP32 kernel)
+#define P3M_PAIR_CTAS 18     // one-warp CTAs per SM that the FP32 kernel's registers leave room for
 #define P3M_PAIR_TJ 128      // j-particles per shared-memory tile (4 blocks of 32)
 #define P3M_FLAG_TIMEOUT 1u  // counters[1] bit: a bounded wait gave up
 
@@ -185,9 +209,7 @@ enum {
 // kfac, or *kfac_dev when that is set).  Passed by value for one context, or as a device array
 // indexed by simulation in the batched ensemble launch.
 struct PairArgs {
-    const float *relx;
-    const float4 *rel;
-    const double *pos;
+    const uint32_t *relq;
     const float4 *block_box;
     const uint32_t *cell_start;
     const uint32_t *work;
@@ -199,8 +221,8 @@ struct PairArgs {
     unsigned long long *pair_count;
     double kfac;
     P3MGeom g;
-    float gpoly[12];
-    float rcull2, rin2;
+    PairFactor fac;
+    float rcull2, pad;
 };
 
 // A neighbour cell of a pair work item, for the FP32 pair kernels: the shift between the two

@@ -481,6 +481,7 @@ __global__ void __launch_bounds__(256, 6) k_permute(const uint32_t *__restrict__
                           double *__restrict__ pos_out, double *__restrict__ mom_out,
                           uint32_t *__restrict__ pid_out, R4 *__restrict__ rel,
                           float4 *__restrict__ block_box, float *__restrict__ relx,
+                          uint32_t *__restrict__ relq, double fix_scale,
                           const double *__restrict__ origin)
 {
     // one warp per 32-slot block of the sorted order; the warp also writes the block's
@@ -518,6 +519,11 @@ __global__ void __launch_bounds__(256, 6) k_permute(const uint32_t *__restrict__
             dst[lane] = (float)rv.x;
             dst[32 + lane] = (float)rv.y;
             dst[64 + lane] = (float)rv.z;
+            // fixed point: 1.5 * 2^52 rounds x * scale to an integer in the low word (modulo 2^32)
+            uint32_t *fix = relq + blk * 96;
+            fix[lane] = (uint32_t)__double_as_longlong(fma(x, fix_scale, 0x1.8p52));
+            fix[32 + lane] = (uint32_t)__double_as_longlong(fma(y, fix_scale, 0x1.8p52));
+            fix[64 + lane] = (uint32_t)__double_as_longlong(fma(z, fix_scale, 0x1.8p52));
         }
         float lx = (float)x, ly = (float)y, lz = (float)z, hx = lx, hy = ly, hz = lz;
 #pragma unroll
@@ -730,13 +736,14 @@ cudaError_t launch_permute_and_cells(p3m_ctx *c)
     if (c->precision == P3M_PREC_MIXED)
         k_permute<float4><<<gb, 256, 0, c->stream>>>(c->vals, c->keys, c->g, c->pos, c->mom,
                                                      c->pid, c->pos_alt, c->mom_alt, c->pid_alt,
-                                                     (float4 *)c->rel, c->block_box, c->relx,
+                                                     (float4 *)c->rel, c->block_box, c->relx, c->relq,
+                                                     ldexp((double)c->g.n_c, kFixBits) / c->g.box,
                                                      c->tab_origin);
     else
         k_permute<double4_16a><<<gb, 256, 0, c->stream>>>(c->vals, c->keys, c->g, c->pos, c->mom,
                                                       c->pid, c->pos_alt, c->mom_alt,
                                                       c->pid_alt, (double4_16a *)c->rel, c->block_box,
-                                                      nullptr, c->tab_origin);
+                                                      nullptr, nullptr, 0.0, c->tab_origin);
     double *t = c->pos;
     c->pos = c->pos_alt;
     c->pos_alt = t;

@@ -1,0 +1,61 @@
+"""The FP32 pair kernel's lists at the sizes where they can go wrong: groups of 16 particles with
+one more or one less, cells around a whole work item, rows of cells that wrap, lists longer than one
+chunk and one FP64 flush, both forms of the split factor (a softening small or large against r_s, a
+short and a long cutoff) and both list lengths.
+
+Bars: the short-range accelerations within 1e-5 relative RMS of the oracle (the FP32 bar), and the
+accepted pairs within the pairs whose distance lies within 1e-6 of the cutoff."""
+
+import math
+
+import numpy as np
+import pytest
+
+import p3m_synth as S
+from oracle import p3m_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+def _set(kind, n, box, seed):
+    x = S.uniform_random(n, box, seed)
+    if kind == "cell":  # half of them inside one small region of one cell
+        m = n // 2
+        x[:, :m] = 0.45 * box + 0.02 * box * S.uniform_random(m, 1.0, seed + 1)
+    return np.mod(x, box)
+
+
+@pytest.mark.parametrize("kind,n,mesh,cutoff,softening", [
+    ("uniform", 2, 20, 4.5, 0.02), ("cell", 30, 20, 4.5, 0.0), ("cell", 32, 26, 4.5, 0.02),
+    ("cell", 34, 32, 4.5, 0.02), ("cell", 62, 20, 4.5, 0.5), ("cell", 66, 32, 4.5, 0.02),
+    ("cell", 1500, 20, 4.5, 0.02), ("cell", 1500, 24, 4.5, 0.3), ("cell", 6001, 32, 4.5, 0.02),
+    ("uniform", 4097, 24, 1.5, 0.02), ("uniform", 4097, 48, 6.0, 0.02), ("uniform", 4097, 48, 6.0, 1.0),
+])
+@pytest.mark.parametrize("tile_blocks", [5, 3])
+def test_pair_lists(kind, n, mesh, cutoff, softening, tile_blocks):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1510_07621_gb300 import P3M, build
+    build.build()
+    box = 50.0
+    x = _set(kind, n, box, 1000 + n + mesh)
+    p = O.Params(box, n, mesh, 1.25, cutoff, softening)
+    ref, pairs = O.sr_accel(O.wrap(x, box), p)
+    with P3M(box, n, mesh, 1.25, cutoff, softening=softening) as sim:
+        sim.set_particles(x, np.zeros_like(x), a=1.0)
+        if tile_blocks == 3:  # the autotuner times both lengths; which one it keeps does not matter
+            sim.autotune()
+        _, sr = sim.forces_split()
+        got = sim.diagnostics()["pairs"]
+    # (no pair within the cutoff: the force is exactly zero)
+    assert math.sqrt(float(np.sum((sr - ref) ** 2))) <= 1e-5 * math.sqrt(float(np.sum(ref ** 2)))
+    d = x[:, :, None] - x[:, None, :] if n <= 1500 else None
+    if d is not None:
+        d -= box * np.round(d / box)
+        r = np.sqrt((d ** 2).sum(0))
+        rc = cutoff * 1.25 * box / mesh
+        near = int((np.abs(r - rc) < 1e-6 * rc).sum())
+        assert abs(got - pairs) <= near
+    else:
+        assert abs(got - pairs) <= max(4, int(2e-6 * pairs))
