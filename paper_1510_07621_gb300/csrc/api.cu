@@ -143,15 +143,37 @@ void fit_split_poly(double cutoff_in_rs, double r_s, float out[12])
     out[11] = (float)(2.0 / (uc * r_s * r_s));
 }
 
-// FP64 coefficients (degree P3M_SPLIT_DEG64, largest error in g about 4e-14 relative) into
-// out[0..P3M_SPLIT_DEG64], tau's scale into out[P3M_SPLIT_DEG64 + 1].
-void fit_split_poly64(double cutoff_in_rs, double r_s, double *out)
+// g on kSplitTab64 equal intervals of r in [0, r_c]: row k holds the coefficients of a degree-7
+// polynomial in t = (2 kSplitTab64 / r_c) r - (2 k + 1), interpolated at 8 Chebyshev nodes (its
+// error is below 1e-16 up to the cutoff 6), and -(2 k + 1).
+void fit_split_table(double cutoff_in_rs, double *tab)
 {
-    double mono[P3M_SPLIT_DEG64 + 1];
-    fit_split_mono(cutoff_in_rs, P3M_SPLIT_DEG64, 64, mono);
-    const double uc = cutoff_in_rs * cutoff_in_rs, inv_rs3 = 1.0 / (r_s * r_s * r_s);
-    for (int i = 0; i <= P3M_SPLIT_DEG64; ++i) out[i] = mono[i] * inv_rs3;
-    out[P3M_SPLIT_DEG64 + 1] = 2.0 / (uc * r_s * r_s);
+    constexpr int kN = 8;
+    auto split_g = [](double x) {
+        return x < 1.0 ? 1.0 + x * x * x * split_q(x * x)
+                       : erfc(0.5 * x) + x * 0.56418958354775628695 * exp(-0.25 * x * x);
+    };
+    for (int k = 0; k < kSplitTab64; ++k) {
+        double *c = tab + (size_t)k * kSplitRow64;
+        // (the difference from the centre's value: the sums over the nodes then stay small)
+        const double g0 = split_g((k + 0.5) * cutoff_in_rs / kSplitTab64);
+        double cheb[kN] = {}, prev[kN] = {1.0}, cur[kN] = {0.0, 1.0}, next[kN];
+        for (int j = 0; j < kN; ++j) {
+            const double th = M_PI * (j + 0.5) / kN, x = (k + 0.5 * (cos(th) + 1.0)) * cutoff_in_rs / kSplitTab64;
+            const double g = split_g(x) - g0;
+            for (int q = 0; q < kN; ++q) cheb[q] += g * cos(q * th) * (q == 0 ? 1.0 : 2.0) / kN;
+        }
+        for (int i = 0; i < kSplitRow64; ++i) c[i] = 0.0;
+        c[0] = cheb[0];
+        for (int q = 1; q < kN; ++q) {  // Chebyshev series -> monomials
+            for (int i = 0; i < kN; ++i) c[i] += cheb[q] * cur[i];
+            for (int i = 0; i < kN; ++i) next[i] = 2.0 * (i > 0 ? cur[i - 1] : 0.0) - prev[i];
+            memcpy(prev, cur, sizeof(cur));
+            memcpy(cur, next, sizeof(cur));
+        }
+        c[0] += g0;
+        c[8] = -(2.0 * k + 1.0);
+    }
 }
 
 // ---------------------------------------------------------------- FP32 pair factor fit
@@ -299,7 +321,7 @@ void release(p3m_ctx *c)
                     c->tab_origin,
                     c->adj_u,     c->adj_vfx,  c->adj_vs,       c->adj_out,  c->kself,
                     c->li,        c->relx,     c->relq,     c->sort_status,  c->sort_hist,
-                    c->rho_fix,   c->fix_exp,  c->ps_part,     c->sort_probe};
+                    c->rho_fix,   c->fix_exp,  c->ps_part,     c->sort_probe, c->split_tab};
     for (void *p : bufs)
         if (p) cudaFree(p);
     if (c->plans_made) {
@@ -713,7 +735,7 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
             {(void **)&c->rel, 4 * real * N}, {(void **)&c->keys, 4 * N},
             {(void **)&c->block_box, 32 * ((N + 31) / 32)},
             {(void **)&c->relx, opt.precision == P3M_PREC_MIXED ? 384 * ((N + 31) / 32) : 16},
-            {(void **)&c->relq, opt.precision == P3M_PREC_MIXED ? 384 * ((N + 31) / 32) : 16},
+            {(void **)&c->relq, 384 * ((N + 31) / 32)},
             {(void **)&c->keys_alt, 4 * N},   {(void **)&c->vals, 4 * N},
             {(void **)&c->vals_alt, 4 * N},   {(void **)&c->digit_counts, 4 * 256 * (size_t)c->n_tiles},
             {(void **)&c->scan_aux, 4 * (scan_n / P3M_SORT_TILE + 4)},
@@ -738,6 +760,7 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
             {(void **)&c->kself, 8 * 27},     {(void **)&c->li, 8 * 4},
             {(void **)&c->adj_u, 3 * real * M3}, {(void **)&c->adj_vfx, opt.precision == P3M_PREC_MIXED ? 384 * ((N + 31) / 32) : 16},
             {(void **)&c->adj_vs, 24 * N},    {(void **)&c->adj_out, 24 * N},
+            {(void **)&c->split_tab, opt.precision == P3M_PREC_FP64 ? 8 * kSplitTab64 * kSplitRow64 : 16},
         };
         int idx = 0;
         for (auto &a : allocs) {
@@ -780,7 +803,6 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
         c->green_const = -4.0 * M_PI * (g.gm / (h * h * h)) / ((double)M3);
         fit_split_poly(cutoff_in_rs, g.r_s, c->gpoly);
         c->pair_factor = fit_pair_factor(cutoff_in_rs, g);
-        fit_split_poly64(cutoff_in_rs, g.r_s, c->gpoly64);
         if (c->precision == P3M_PREC_MIXED) {
             std::vector<float> f(M);
             const std::vector<double> *src[3] = {&tk, &tkg, &tg};
@@ -794,6 +816,11 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
             e = cudaMemcpy(c->tab_k, tk.data(), 8 * M, cudaMemcpyHostToDevice);
             if (e == cudaSuccess) e = cudaMemcpy(c->tab_kg, tkg.data(), 8 * M, cudaMemcpyHostToDevice);
             if (e == cudaSuccess) e = cudaMemcpy(c->tab_g, tg.data(), 8 * M, cudaMemcpyHostToDevice);
+        }
+        if (e == cudaSuccess && c->precision == P3M_PREC_FP64) {
+            std::vector<double> tab(kSplitTab64 * kSplitRow64);
+            fit_split_table(cutoff_in_rs, tab.data());
+            e = cudaMemcpy(c->split_tab, tab.data(), 8 * tab.size(), cudaMemcpyHostToDevice);
         }
         if (e == cudaSuccess) {
             std::vector<double> w2(M), one(M, 1.0);

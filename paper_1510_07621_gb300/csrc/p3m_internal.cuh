@@ -13,11 +13,11 @@
 // degree 10, 1.8e-5 at degree 7: the FP32 rounding of nearly cancelling pair sums dominates)
 // and by 1.7e-6 on a clustered state.
 #define P3M_SPLIT_DEG 8
-// Degree of the FP64 split factor of the FP64 pair kernel: its largest error in g is about
-// 4e-14 relative (at r_c), far below the FP64 mode's 1e-12 parity bar.
-#define P3M_SPLIT_DEG64 18
+// The FP64 pair kernel's table of g (fit_split_table): intervals of [0, r_c], and doubles per row
+// (8 coefficients, the interval's centre, one of padding against bank conflicts).
+constexpr int kSplitTab64 = 64, kSplitRow64 = 10;
 
-// Fixed-point coordinates of the FP32 pair kernels: 2^-kFixBits of a chaining cell, modulo 2^32
+// Fixed-point coordinates of the pair kernels: 2^-kFixBits of a chaining cell, modulo 2^32
 // (8 cells), so that differences of particles in neighbouring cells are exact integers.
 constexpr int kFixBits = 29;
 constexpr float kFixUnit = 0x1p-29f;
@@ -91,7 +91,7 @@ struct p3m_ctx {
     void *rel;  // float4 (mixed) or double4_16a (fp64): position relative to its cell origin
     float4 *block_box;  // per 32-slot block of the sorted order: lo, hi (FP32, absolute)
     float *relx;        // FP32 mode: rel as block-SoA, per 32-slot block x[32] y[32] z[32]
-    uint32_t *relq;     // FP32 mode: fixed-point coordinates (kFixBits), per 32-slot block x[32] y[32] z[32]
+    uint32_t *relq;     // fixed-point coordinates (kFixBits), per 32-slot block x[32] y[32] z[32]
     int tile_blocks;    // FP32 pair kernel: its list is evaluated every 32 tile_blocks entries (3 or 5)
 
     // sort
@@ -133,8 +133,7 @@ struct p3m_ctx {
     float gpoly[12];  // FP32 split factor: g = 1 + r^3 Q(tau), Q = sum gpoly[k] tau^k
                       // (k <= P3M_SPLIT_DEG), tau = r^2 gpoly[11] - 1
     PairFactor pair_factor;  // of the FP32 force kernel
-    double gpoly64[P3M_SPLIT_DEG64 + 2];  // the same in FP64 (degree P3M_SPLIT_DEG64); the
-                                          // last entry is tau's scale
+    double *split_tab;  // FP64 mode: the table of g (kSplitTab64 rows)
     cufftHandle plan_r2c, plan_c2r, plan_c2r_one;  // R2C, batched 3 x C2R, single C2R
     bool plans_made;
 
@@ -201,7 +200,6 @@ enum {
 #define P3M_PAIR_TI 32       // i-particles per pair work item (one per lane of a warp)
 #define P3M_PAIR_GROUP 16    // particles of a work item that share one list (FP32 kernel)
 #define P3M_PAIR_CTAS 18     // one-warp CTAs per SM that the FP32 kernel's registers leave room for
-#define P3M_PAIR_TJ 128      // j-particles per shared-memory tile (4 blocks of 32)
 #define P3M_FLAG_TIMEOUT 1u  // counters[1] bit: a bounded wait gave up
 
 // Everything the FP32 pair kernel needs from one context: its arrays, geometry, fitted split

@@ -17,253 +17,223 @@
 
 #include "p3m_device.cuh"
 #include "p3m_internal.cuh"
+#include "pair_walk.cuh"
 
 namespace {
 
-constexpr int kTJ = P3M_PAIR_TJ;  // 128
-constexpr int kBlocksPerTile = kTJ / 32;
 constexpr int kLongChunk = 5;   // FP32 kernel: the list is evaluated every 160 entries
 constexpr int kShortChunk = 3;  // the autotuner's other choice
 constexpr int kGroup = P3M_PAIR_GROUP;
 
-// Coefficients of the FP64 split factor (the context's gpoly64): g = 1 + r^3 sum_k c[k] tau^k
-// (k <= P3M_SPLIT_DEG64), tau = r^2 c[P3M_SPLIT_DEG64 + 1] - 1.
-struct GPoly64 {
-    double c[P3M_SPLIT_DEG64 + 2];
-};
-
-// g(r/r_s) (r^2 + eps^2)^-3/2 for one pair in FP64, g from the FP64 fit (largest error about
-// 4e-14 relative): rsqrt and a Horner chain instead of sqrt, a division, erfc and exp, which
-// all run on GB300's narrow FP64 pipe.  For r2 = 0 the result is not finite; callers select
-// such pairs out.
-__device__ __forceinline__ double pair_factor64(double r2, double eps2, const GPoly64 &gp)
+// x^-1/2: the hardware's approximation (relative error e0 / 2 below 2^-20) and one step of the
+// third-order iteration y (1 + e/2 + 3 e^2/8), e = 1 - x y^2, whose error 5/16 e^3 is below 2^-58.
+__device__ __forceinline__ double rsqrt64(double x)
 {
-    const double s = rsqrt(r2 + eps2);
-    const double r3 = r2 * (r2 * rsqrt(r2));
-    const double tau = fma(r2, gp.c[P3M_SPLIT_DEG64 + 1], -1.0);
-    double p = gp.c[P3M_SPLIT_DEG64];
-#pragma unroll
-    for (int k = P3M_SPLIT_DEG64 - 1; k >= 0; --k) p = fma(p, tau, gp.c[k]);
-    const double gval = fma(r3, p, 1.0);
-    return gval * (s * s * s);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
 }
 
-// The FP64 kernel.  A lane holds one particle of the work item; the warp streams the j particles of
-// the 27 neighbour cells through shared memory in tiles of up to four 32-slot blocks of the sorted
-// order, copied by the bulk-copy (TMA) engine into two alternating buffers (the next tile in
-// flight while the current one is used; one mbarrier per buffer; every wait bounded).  It skips a
-// block when no lane's particle is within r_c of the block's bounding box, evaluates it without
-// per-pair tests when the box lies within r_c of every lane's particle, and otherwise tests each
-// pair, skipping j's that no lane accepts.  Absolute coordinates: d = (x_j - x_i) + image, like a
-// plain minimum-image difference.
-struct Neighbour {
-    uint32_t start, end;
-    double imx, imy, imz;  // periodic image of the neighbour cell
-};
+// g(r/r_s) (r^2 + eps^2)^-3/2 for one pair in FP64.  g comes from the context's table (tab: 64
+// intervals of r in [0, r_c], a degree-7 polynomial in t in [-1, 1] each, see fit_split_table): 7
+// FP64 operations per pair, where one polynomial over the whole range takes 18 and two to form r^3.
+// The interval index needs no FP64 operation: r truncated to FP32 by its bits; at an interval's end it
+// may be one off, and t then exceeds 1 by 1e-5.  For r2 = 0 the result is not finite, beyond r_c it is
+// extrapolated; callers select such pairs out.
+__device__ __forceinline__ double pair_factor64(double r2, double eps2, float scale_f, double scale,
+                                                const double *tab)
+{
+    const double ri = rsqrt64(r2), s = eps2 == 0.0 ? ri : rsqrt64(r2 + eps2);
+    const double r = r2 * ri;
+    const int hi = __double2hiint(r), e = (hi >> 20 & 0x7FF) - 1023 + 127;
+    const float rf = e >= 1 && e <= 254 ? __int_as_float((e << 23) | (hi & 0xFFFFF) << 3) : 0.0f;
+    const int k = min((int)(rf * scale_f), kSplitTab64 - 1);
+    const double *c = tab + k * kSplitRow64;
+    const double t = fma(r, scale, c[8]);  // (c[8] = -(2 k + 1))
+    double p = fma(c[7], t, c[6]);
+#pragma unroll
+    for (int q = 5; q >= 0; --q) p = fma(p, t, c[q]);
+    return p * (s * s * s);
+}
+
+// The FP64 kernel.  GB300's FP64 pipe issues one warp instruction in 16 cycles per SM, 64 times fewer
+// than the FP32 pipes, so that everything but the accepted pairs' arithmetic is kept off it.  A
+// one-warp CTA takes 8 particles of a work item at a time, four lanes to a particle:
+//   1. For up to kEntries32 surviving 32-slot blocks (pair_walk.cuh) it tests every (particle, slot)
+//      in FP32 on the fixed-point coordinates, with a radius padded by more than their rounding, and
+//      keeps one 32-bit mask per particle and block in shared memory.
+//   2. Lane q of a particle then takes the pairs number q, q + 4, q + 8, ... of its masks: every step
+//      evaluates 32 different pairs in FP64 (d = (x_j - x_i) + image, like a plain minimum-image
+//      difference, and the exact test 0 < r < r_c), whatever blocks they lie in.
+// Before, a lane held one particle and all lanes met the same j, tested in FP64: 0.37 of the
+// evaluated and 0.2 of the tested lane slots held an accepted pair, and 32^3 particles gave too few
+// warps to hide the FP64 latency.  One step (two evaluations) of 32^3 particles: 38.9 -> 4.6 ms, of
+// the clustered 48^3 set 2.9 to 5 times less (more, the more clustered).  What bounds it: the 32 FP64
+// operations of a pair (45 before the table of g, 2.0 instead of 2.8 ms per evaluation at 32^3);
+// at the measured FP64 rate they take 1.5 ms there.
+constexpr int kEntries64 = 96;  // blocks per round (about what a group of 8 has in all at 200 per cell)
 
 __global__ void __launch_bounds__(32)
-    k_pairs64(const double4_16a *__restrict__ rel, const double *__restrict__ pos,
-            const float4 *__restrict__ block_box, const uint32_t *__restrict__ cell_start,
-            const uint32_t *__restrict__ work, const uint32_t *__restrict__ order,
-            const uint32_t *__restrict__ n_work_ptr, P3MGeom g, GPoly64 gp, float rcull2, float rin2,
-            const double *__restrict__ acc_in, double *__restrict__ acc_out,
-            double *__restrict__ mom, double kfac, const double *__restrict__ kfac_dev,
-            uint32_t *__restrict__ counters, unsigned long long *__restrict__ pair_count)
+    k_pairs64(const uint32_t *__restrict__ relq, const double *__restrict__ pos,
+              const float4 *__restrict__ block_box, const uint32_t *__restrict__ cell_start,
+              const uint32_t *__restrict__ work, const uint32_t *__restrict__ order,
+              const uint32_t *__restrict__ n_work_ptr, P3MGeom g, const double *__restrict__ split, float rcull2, float rlist2,
+              const double *__restrict__ acc_in, double *__restrict__ acc_out,
+              double *__restrict__ mom, double kfac, const double *__restrict__ kfac_dev,
+              uint32_t *__restrict__ cursor, unsigned long long *__restrict__ pair_count)
 {
+    constexpr int kG = 8, kSub = P3M_PAIR_TI / kG;
     if (kfac_dev) kfac = *kfac_dev;  // graph-replayed steps read the factor from the device
-    __shared__ __align__(128) double4_16a sj[2][kTJ];
-    __shared__ __align__(8) uint64_t bar[2];
-    __shared__ Neighbour nbr[27];
-
-    const int lane = threadIdx.x;
-    const int64_t n = g.n;
-    const uint32_t n_work = *n_work_ptr;
-    const double rc2 = g.r_c * g.r_c;
-    const double eps2 = g.eps * g.eps;
-    const int nc = g.n_c;
-
-    if (lane == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-        mbar_fence_init();
-    }
+    __shared__ uint32_t mask[kEntries64][kG];
+    __shared__ uint32_t entry[kEntries64];
+    __shared__ __align__(16) float sj[3][32];
+    __shared__ PairSeg seg[kPairSegs];
+    __shared__ uint32_t live[32];
+    __shared__ __align__(16) double tab[kSplitTab64 * kSplitRow64];
+    for (int t = threadIdx.x; t < kSplitTab64 * kSplitRow64; t += 32) tab[t] = split[t];
     __syncwarp();
-    uint32_t parity = 0u;  // bit b: parity of the next phase of bar[b]
-    unsigned long long my_pairs = 0, st_fast = 0, st_tested = 0, st_eval = 0, st_culled = 0,
-                       st_tiles = 0, st_empty_tiles = 0;
-    bool timed_out = false;
+
+    const int lane = threadIdx.x, pi = lane & 7, q = lane >> 3;  // particle of the group, its lane
+    const int64_t n = g.n;
+    const uint32_t n_units = *n_work_ptr * kSub;
+    const long long rc2 = __double_as_longlong(g.r_c * g.r_c);
+    const double eps2 = g.eps * g.eps, tscale = 2.0 * kSplitTab64 / g.r_c;
+    const float kscale = (float)(kSplitTab64 / g.r_c);
+    const int nc = g.n_c;
+    const float cell_f = (float)g.cs;
+    unsigned long long st_pairs = 0, st_tested = 0, st_steps = 0, st_culled = 0, st_rounds = 0;
 
     for (;;) {
-        uint32_t slot = 0;
-        if (lane == 0) slot = atomicAdd(&counters[0], 1u);
-        slot = __shfl_sync(0xffffffffu, slot, 0);
-        if (slot >= n_work) break;
-        const uint32_t item = order[slot];
+        uint32_t unit = 0;
+        if (lane == 0) unit = atomicAdd(cursor, 1u);
+        unit = __shfl_sync(0xffffffffu, unit, 0);
+        if (unit >= n_units) break;
+        const uint32_t item = order[unit / kSub];
         const uint32_t cell = work[2 * (size_t)item];
-        const uint32_t first = work[2 * (size_t)item + 1];
+        const uint32_t first = work[2 * (size_t)item + 1] + (unit % kSub) * kG;
         const uint32_t cend = cell_start[cell + 1];
+        if (first >= cend) continue;
         const int cx = (int)(cell % nc), cy = (int)((cell / nc) % nc), cz = (int)(cell / (nc * nc));
-        if (lane < 27) {
-            const int ox = lane % 3 - 1, oy = (lane / 3) % 3 - 1, oz = lane / 9 - 1;
-            const int ux = cx + ox, uy = cy + oy, uz = cz + oz;  // unwrapped neighbour index
-            const int wx = (ux + nc) % nc, wy = (uy + nc) % nc, wz = (uz + nc) % nc;
-            const uint32_t nb = ((uint32_t)wz * nc + wy) * nc + wx;
-            Neighbour q;
-            q.start = cell_start[nb];
-            q.end = cell_start[nb + 1];
-            if (q.start == q.end) q.start = q.end = 0;  // empty: the tile walk skips it
-            const double L = g.box;
-            q.imx = ux < 0 ? -L : (ux >= nc ? L : 0.0);
-            q.imy = uy < 0 ? -L : (uy >= nc ? L : 0.0);
-            q.imz = uz < 0 ? -L : (uz >= nc ? L : 0.0);
-            nbr[lane] = q;
-        }
-        __syncwarp();
-
-        const uint32_t i = first + lane;
-        const bool valid = i < cend;
-        const uint32_t ii = valid ? i : first;
-        const double4_16a xi = rel[ii];
-        const double xa = pos[ii], ya = pos[n + ii], za = pos[2 * n + ii];  // absolute, FP64
+        // FP32 frame in cell sides
+        const GroupFrame fr = group_frame<kG>(relq, first, cend, cx, cy, cz, kFixUnit, cell_f);
+        const uint2 blocks = group_ranges(seg, cell_start, g, cx, cy, cz, fr, cell_f);
+        const uint32_t i = min(first + pi, cend - 1);
+        const bool valid = first + pi < cend;
+        const uint32_t *qi = fix_coords(relq, i);
+        const float fx = (float)(int)(__ldg(qi) - fr.ctr[0]) * kFixUnit,
+                    fy = (float)(int)(__ldg(qi + 32) - fr.ctr[1]) * kFixUnit,
+                    fz = (float)(int)(__ldg(qi + 64) - fr.ctr[2]) * kFixUnit;
+        const double xi = pos[i], yi = pos[n + i], zi = pos[2 * n + i];
         double ax = 0.0, ay = 0.0, az = 0.0;
+        uint32_t pairs = 0, steps = 0, rounds = 0, n_live = 0;
 
-        // Tile sequence over (neighbour nb, first block b); a tile is the blocks [b, b + 4)
-        // clipped to the neighbour's range of slots; nb == 27 ends the sequence.
-        auto next_tile = [&](int &nb, uint32_t &b) {
-            while (nb < 27 && b * 32u >= nbr[nb].end) {
-                ++nb;
-                if (nb < 27) b = nbr[nb].start >> 5;
-            }
-        };
-        auto issue = [&](int nb, uint32_t b, int to) {
-            const uint32_t bend = min(b + kBlocksPerTile, (nbr[nb].end + 31) >> 5);
-            const uint32_t j0 = b * 32;
-            const uint32_t j1 = min((uint32_t)n, bend * 32);
-            const uint32_t bytes = (j1 - j0) * (uint32_t)sizeof(double4_16a);
-            mbar_expect_tx(&bar[to], bytes);
-            bulk_load(&sj[to][0], rel + j0, bytes, &bar[to]);
-        };
-
-        int nb_c = 0;
-        uint32_t b_c = nbr[0].start >> 5;
-        next_tile(nb_c, b_c);
-        int buf = 0;
-        if (nb_c < 27 && lane == 0) issue(nb_c, b_c, 0);
-        while (nb_c < 27) {
-            const uint32_t nstart = nbr[nb_c].start, nend = nbr[nb_c].end;
-            const uint32_t bend = min(b_c + kBlocksPerTile, (nend + 31) >> 5);
-            int nb_n = nb_c;
-            uint32_t b_n = bend;
-            next_tile(nb_n, b_n);
-            __syncwarp();  // every lane is done with sj[buf ^ 1] before it is refilled
-            if (nb_n < 27 && lane == 0) issue(nb_n, b_n, buf ^ 1);
-            const bool ok = mbar_wait_bounded(&bar[buf], (parity >> buf) & 1u);
-            parity ^= 1u << buf;
-            if (__any_sync(0xffffffffu, !ok)) {
-                timed_out = true;
-                if (nb_n < 27) mbar_wait_bounded(&bar[buf ^ 1], (parity >> (buf ^ 1)) & 1u);
-                break;
-            }
-            const Neighbour &q = nbr[nb_c];
-            // d = (x_j - x_i) + image, like a plain minimum-image difference
-            const double xs = xi.x, ys = xi.y, zs = xi.z;
-            const double ix = q.imx, iy = q.imy, iz = q.imz;
-            // particle i in the frame of the block boxes (absolute, image removed)
-            const float cxs = (float)(xa - q.imx), cys = (float)(ya - q.imy), czs = (float)(za - q.imz);
-            const double4_16a *tile = sj[buf];
-            double px = 0, py = 0, pz = 0;
-            uint32_t cnt = 0, n_fast = 0, n_tested = 0, n_eval = 0, n_culled = 0;
-            for (uint32_t b = b_c; b < bend; ++b) {
-                const float4 lo = __ldg(block_box + 2 * b), hi = __ldg(block_box + 2 * b + 1);
-                const float ex = fmaxf(fmaxf(lo.x - cxs, cxs - hi.x), 0.0f);
-                const float ey = fmaxf(fmaxf(lo.y - cys, cys - hi.y), 0.0f);
-                const float ez = fmaxf(fmaxf(lo.z - czs, czs - hi.z), 0.0f);
-                const bool near = valid && ex * ex + ey * ey + ez * ez < rcull2;
-                if (!__any_sync(0xffffffffu, near)) {
-                    ++n_culled;
-                    continue;
-                }
-                // the block's slots that belong to the neighbour cell, as tile offsets
-                const uint32_t j0 = max(b * 32, nstart) - b_c * 32;
-                const uint32_t j1 = min(b * 32 + 32, nend) - b_c * 32;
-                const float fx = fmaxf(cxs - lo.x, hi.x - cxs);
-                const float fy = fmaxf(cys - lo.y, hi.y - cys);
-                const float fz = fmaxf(czs - lo.z, hi.z - czs);
-                if (__all_sync(0xffffffffu, !valid || fx * fx + fy * fy + fz * fz < rin2)) {
-                    // the block lies within r_c of every particle of the warp
-                    n_fast += j1 - j0;
-#pragma unroll 2
-                    for (uint32_t j = j0; j < j1; ++j) {
-                        const double4_16a qj = tile[j];
-                        const double dx = (qj.x - xs) + ix, dy = (qj.y - ys) + iy, dz = (qj.z - zs) + iz;
-                        const double r2 = dx * dx + dy * dy + dz * dz;
-                        const bool in = valid && r2 > 0.0;
-                        double f = pair_factor64(r2, eps2, gp);
-                        f = in ? f : 0.0;
-                        px += f * dx;
-                        py += f * dy;
-                        pz += f * dz;
-                        cnt += in ? 1u : 0u;
+        for (uint32_t base = 0; base < blocks.y;) {
+            int ne = 0;
+            for (; base < blocks.y && ne + 32 <= kEntries64; base += 32) {
+                const int nl = live_blocks(base + lane, blocks.y, seg, block_box, fr, cell_f, rcull2, live);
+                n_live += nl;
+                for (int k = 0; k < nl; ++k) {
+                    const uint32_t w = live[k];
+                    const PairSeg &S = seg[w >> 26];
+                    const uint32_t b = w & 0x3FFFFFFu;
+                    const uint32_t *qj = fix_coords(relq, b * 32 + lane);
+                    const uint32_t jx = __ldg(qj), jy = __ldg(qj + 32), jz = __ldg(qj + 64);
+                    // the slots of the block that belong to the range
+                    const uint32_t in = __ballot_sync(0xffffffffu, b * 32 + lane - S.start < S.end - S.start);
+                    __syncwarp();  // every lane is done with the previous block's coordinates
+                    sj[0][lane] = (float)(int)(jx - S.cx) * kFixUnit;
+                    sj[1][lane] = (float)(int)(jy - S.cy) * kFixUnit;
+                    sj[2][lane] = (float)(int)(jz - S.cz) * kFixUnit;
+                    __syncwarp();
+                    uint32_t m = 0;  // slots 8 q .. 8 q + 7 against particle pi
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float4 X = *(const float4 *)&sj[0][8 * q + 4 * h], Y = *(const float4 *)&sj[1][8 * q + 4 * h],
+                                     Z = *(const float4 *)&sj[2][8 * q + 4 * h];
+                        const float xs[4] = {X.x, X.y, X.z, X.w}, ys[4] = {Y.x, Y.y, Y.z, Y.w}, zs[4] = {Z.x, Z.y, Z.z, Z.w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const float dx = xs[e] - fx, dy = ys[e] - fy, dz = zs[e] - fz;
+                            if (dx * dx + dy * dy + dz * dz < rlist2) m |= 1u << (4 * h + e);
+                        }
                     }
-                    continue;
+                    m <<= 8 * q;
+                    m |= __shfl_xor_sync(0xffffffffu, m, 8);
+                    m |= __shfl_xor_sync(0xffffffffu, m, 16);
+                    if (q == 0) mask[ne + k][pi] = valid ? m & in : 0u;
+                    if (lane == 0) entry[ne + k] = w;
                 }
-                n_tested += j1 - j0;
-                for (uint32_t j = j0; j < j1; ++j) {
-                    const double4_16a qj = tile[j];
-                    const double dx = (qj.x - xs) + ix, dy = (qj.y - ys) + iy, dz = (qj.z - zs) + iz;
-                    const double r2 = dx * dx + dy * dy + dz * dz;
-                    const bool in = valid && r2 < rc2 && r2 > 0.0;
-                    if (!__any_sync(0xffffffffu, in)) continue;
-                    ++n_eval;
-                    double f = pair_factor64(r2, eps2, gp);
-                    f = in ? f : 0.0;
-                    px += f * dx;
-                    py += f * dy;
-                    pz += f * dz;
-                    cnt += in ? 1u : 0u;
+                ne += nl;
+            }
+            __syncwarp();
+            // this lane's pairs: number q, q + 4, ... of the particle's masks
+            int k = 0, skip = q;
+            uint32_t m = 0, w = 0;
+            for (;;) {
+                while (__popc(m) <= skip && k < ne) {
+                    skip -= __popc(m);
+                    m = mask[k][pi];
+                    w = entry[k++];
                 }
+                const bool have = __popc(m) > skip;
+                if (!__any_sync(0xffffffffu, have)) break;
+                for (; skip > 0; --skip) m &= m - 1;
+                const uint32_t j = have ? (w & 0x3FFFFFFu) * 32 + (uint32_t)__ffs(m) - 1 : i;
+                m &= m - 1;
+                skip = have ? 3 : 0;
+                double dx = pos[j] - xi, dy = pos[n + j] - yi, dz = pos[2 * n + j] - zi;
+                const uint32_t img = have ? seg[w >> 26].image : 0x15u;
+                if (__any_sync(0xffffffffu, img != 0x15u)) {  // some pair crosses the boundary
+                    const double L = g.box;
+                    dx += (img & 3u) == 1u ? 0.0 : ((img & 3u) == 0u ? -L : L);
+                    dy += (img >> 2 & 3u) == 1u ? 0.0 : ((img >> 2 & 3u) == 0u ? -L : L);
+                    dz += (img >> 4) == 1u ? 0.0 : ((img >> 4) == 0u ? -L : L);
+                }
+                const double r2 = dx * dx + dy * dy + dz * dz;
+                // 0 < r2 < r_c^2 on the bit patterns (non-negative doubles order like integers)
+                const long long rb = __double_as_longlong(r2);
+                const bool acc = have && rb != 0 && rb < rc2;
+                double f = pair_factor64(r2, eps2, kscale, tscale, tab);
+                f = acc ? f : 0.0;
+                ax = fma(f, dx, ax);
+                ay = fma(f, dy, ay);
+                az = fma(f, dz, az);
+                pairs += acc ? 1u : 0u;
+                ++steps;
             }
-            ax += (double)px;
-            ay += (double)py;
-            az += (double)pz;
-            my_pairs += cnt;
-            st_fast += n_fast;
-            st_tested += n_tested;
-            st_eval += n_eval;
-            st_culled += n_culled;
-            ++st_tiles;
-            if (n_culled == bend - b_c) ++st_empty_tiles;
-            buf ^= 1;
-            nb_c = nb_n;
-            b_c = b_n;
+            ++rounds;
+            __syncwarp();  // the masks are rewritten by the next round
         }
-        if (timed_out) break;
-        if (valid) {
-            const double a3[3] = {g.gm * ax, g.gm * ay, g.gm * az};
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                const double tot = (acc_in ? acc_in[d * n + i] : 0.0) + a3[d];
-                acc_out[d * n + i] = tot;
-                if (kfac != 0.0) mom[d * n + i] = __dadd_rn(mom[d * n + i], __dmul_rn(kfac, tot));
-            }
+        // the four lanes of a particle, always in the same order
+        ax += __shfl_xor_sync(0xffffffffu, ax, 8);
+        ay += __shfl_xor_sync(0xffffffffu, ay, 8);
+        az += __shfl_xor_sync(0xffffffffu, az, 8);
+        ax += __shfl_xor_sync(0xffffffffu, ax, 16);
+        ay += __shfl_xor_sync(0xffffffffu, ay, 16);
+        az += __shfl_xor_sync(0xffffffffu, az, 16);
+        if (valid && q < 3) {  // lane q of a particle writes component q
+            const size_t o = (size_t)q * n + i;
+            const double a = g.gm * (q == 0 ? ax : (q == 1 ? ay : az));
+            const double tot = (acc_in ? acc_in[o] : 0.0) + a;
+            acc_out[o] = tot;
+            if (kfac != 0.0) mom[o] = __dadd_rn(mom[o], __dmul_rn(kfac, tot));
         }
-        __syncwarp();  // nbr is rewritten by the next item
+        st_pairs += __reduce_add_sync(0xffffffffu, pairs);
+        st_tested += n_live * kG;
+        st_steps += steps;
+        st_culled += blocks.y - n_live;
+        st_rounds += rounds;
     }
-    if (timed_out && lane == 0) atomicOr(&counters[1], P3M_FLAG_TIMEOUT);
-    // pair count: warp sum, one atomic per warp
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) my_pairs += __shfl_down_sync(0xffffffffu, my_pairs, o);
     if (lane == 0) {
-        if (my_pairs) {
-            atomicAdd(pair_count, my_pairs);
-            atomicAdd(pair_count + 1, my_pairs);
+        if (st_pairs) {
+            atomicAdd(pair_count, st_pairs);
+            atomicAdd(pair_count + 1, st_pairs);
         }
-        if (st_fast) atomicAdd(pair_count + 2, st_fast);
         if (st_tested) atomicAdd(pair_count + 3, st_tested);
-        if (st_eval) atomicAdd(pair_count + 4, st_eval);
+        if (st_steps) atomicAdd(pair_count + 4, st_steps);
         if (st_culled) atomicAdd(pair_count + 5, st_culled);
-        if (st_tiles) atomicAdd(pair_count + 6, st_tiles);
-        if (st_empty_tiles) atomicAdd(pair_count + 7, st_empty_tiles);
+        if (st_rounds) atomicAdd(pair_count + 6, st_rounds);
     }
 }
 
@@ -299,19 +269,9 @@ __global__ void __launch_bounds__(32)
 // kTinyQ when there is no softening) and contributes exactly f * 0.  Only the row of the own cell
 // can hold such pairs; there (kOwn) a pair counts only if one of its differences is non-zero.
 
-constexpr int kPairSegs = 18;           // 9 rows of neighbour cells, each at most two ranges
 constexpr int kFlushTerms = 80;         // FP32 terms per partial sum before it joins the FP64 sum
 constexpr float kTinyQ = 1e-24f;        // far below the smallest non-zero scaled r^2
 constexpr float kFarQ = 1e6f;           // scaled coordinate of a padding entry: outside every cutoff
-
-// One range of neighbour slots of a group: its slots, the group's centre in the range's periodic
-// image (fixed point, and absolute FP32 for the block boxes), and the number of blocks before it.
-struct __align__(16) PairSeg {
-    uint32_t start, end, cx, cy;
-    uint32_t cz, first_block;
-    float ax, ay;
-    float az, pad[3];
-};
 
 struct PairConstQ {
     f2 c[5];
@@ -425,69 +385,11 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
         if (first >= cend) continue;
         const int cx = (int)(cell % nc), cy = (int)((cell / nc) % nc), cz = (int)(cell / (nc * nc));
 
-        // the group's bounding box around an integer centre; lane l < kG holds particle l
-        uint32_t ctr[3];
-        float half[3], actr[3];
-        {
-            const uint32_t i = min(first + min(lane, kG - 1), cend - 1);
-            const uint32_t *q = A.relq + (size_t)(i >> 5) * 96 + (i & 31);
-            const int c3[3] = {cx, cy, cz};
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                const uint32_t x = __ldg(q + 32 * d), x0 = __shfl_sync(0xffffffffu, x, 0);
-                const int lo = __reduce_min_sync(0xffffffffu, (int)(x - x0));
-                const int hi = __reduce_max_sync(0xffffffffu, (int)(x - x0));
-                const int mid = lo + ((hi - lo) >> 1);
-                ctr[d] = x0 + (uint32_t)mid;
-                half[d] = (float)(max(hi - mid, mid - lo)) * (1.0f + 0x1p-20f) * A.fac.lambda;
-                // absolute FP32 centre: cell index and offset inside the cell, in cell sides
-                actr[d] = ((float)c3[d] + (float)(int)(ctr[d] - ((uint32_t)c3[d] << kFixBits)) * kFixUnit) *
-                          A.fac.cell;
-            }
-        }
-        __syncwarp();  // the previous group is done with seg
-        uint32_t nblk = 0;
-        if (lane < kPairSegs) {
-            const int row = ((lane >> 1) + 4) % 9;  // the own row (4) comes first
-            const int uy = cy + row % 3 - 1, uz = cz + row / 3 - 1;
-            const int wy = uy < 0 ? uy + nc : (uy >= nc ? uy - nc : uy);
-            const int wz = uz < 0 ? uz + nc : (uz >= nc ? uz - nc : uz);
-            const int iy = uy < 0 ? -1 : (uy >= nc ? 1 : 0), iz = uz < 0 ? -1 : (uz >= nc ? 1 : 0);
-            int x0 = max(cx - 1, 0), x1 = min(cx + 1, nc - 1), ix = 0;
-            if (lane & 1) {  // the wrapped end of the row, if any
-                ix = cx == 0 ? -1 : (cx == nc - 1 ? 1 : 0);
-                x0 = x1 = cx == 0 ? nc - 1 : 0;
-            }
-            const uint32_t base = ((uint32_t)wz * nc + wy) * nc;
-            uint32_t s = A.cell_start[base + x0], e = A.cell_start[base + x1 + 1];
-            if (!p3m_in_bounds(s <= e && e <= (uint32_t)n, g.flags)) e = s;
-            if ((lane & 1) && ix == 0) e = s;
-            PairSeg q;
-            q.start = s;
-            q.end = e;
-            const uint32_t box = (uint32_t)nc << kFixBits;  // the box side modulo 2^32
-            q.cx = ctr[0] - (uint32_t)ix * box;
-            q.cy = ctr[1] - (uint32_t)iy * box;
-            q.cz = ctr[2] - (uint32_t)iz * box;
-            q.ax = actr[0] - (float)(ix * nc) * A.fac.cell;
-            q.ay = actr[1] - (float)(iy * nc) * A.fac.cell;
-            q.az = actr[2] - (float)(iz * nc) * A.fac.cell;
-            nblk = e > s ? ((e - 1) >> 5) - (s >> 5) + 1 : 0;
-            uint32_t incl = nblk;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync((1u << kPairSegs) - 1u, incl, o);
-                if (lane >= o) incl += y;
-            }
-            q.first_block = incl - nblk;
-            seg[lane] = q;
-            nblk = incl;
-        }
+        const GroupFrame fr = group_frame<kG>(A.relq, first, cend, cx, cy, cz, A.fac.lambda, A.fac.cell);
+        const uint2 blocks = group_ranges(seg, A.cell_start, g, cx, cy, cz, fr, A.fac.cell);
+        const float hx = fr.half[0], hy = fr.half[1], hz = fr.half[2];
 #pragma unroll
         for (int q = 0; q < 6; ++q) sum[q][lane] = 0.0;
-        __syncwarp();
-        const uint32_t own_blocks = __shfl_sync(0xffffffffu, nblk, 1);
-        const uint32_t all_blocks = __shfl_sync(0xffffffffu, nblk, kPairSegs - 1);
 
         // the lane's two particles, relative to the centre and negated
         const float lambda = A.fac.lambda;
@@ -496,10 +398,10 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const uint32_t i = min(first + ip + u * kPairsI, cend - 1);
-            const uint32_t *q = A.relq + (size_t)(i >> 5) * 96 + (i & 31);
-            const float x = (float)(int)(__ldg(q) - ctr[0]) * -lambda,
-                        y = (float)(int)(__ldg(q + 32) - ctr[1]) * -lambda,
-                        z = (float)(int)(__ldg(q + 64) - ctr[2]) * -lambda;
+            const uint32_t *q = fix_coords(A.relq, i);
+            const float x = (float)(int)(__ldg(q) - fr.ctr[0]) * -lambda,
+                        y = (float)(int)(__ldg(q + 32) - fr.ctr[1]) * -lambda,
+                        z = (float)(int)(__ldg(q + 64) - fr.ctr[2]) * -lambda;
             nx[u] = f2_pack(x, x);
             ny[u] = f2_pack(y, y);
             nz[u] = f2_pack(z, z);
@@ -563,27 +465,7 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
         // the blocks [t0, t1) of the ranges in sequence
         auto walk = [&](auto own, uint32_t t0, uint32_t t1) {
             for (uint32_t base = t0; base < t1; base += 32) {
-                const uint32_t t = base + lane;
-                bool keep = false;
-                uint32_t word = 0;
-                if (t < t1) {
-                    int s = 0;  // the last range that starts at or before block t
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1)
-                        if (s + o < kPairSegs && seg[s + o].first_block <= t) s += o;
-                    const uint32_t b = (seg[s].start >> 5) + (t - seg[s].first_block);
-                    const float4 lo = __ldg(A.block_box + 2 * (size_t)b), hi = __ldg(A.block_box + 2 * (size_t)b + 1);
-                    const float hx = half[0] * A.fac.length, hy = half[1] * A.fac.length, hz = half[2] * A.fac.length;
-                    const float ex = fmaxf(fmaxf(lo.x - seg[s].ax, seg[s].ax - hi.x) - hx, 0.0f);
-                    const float ey = fmaxf(fmaxf(lo.y - seg[s].ay, seg[s].ay - hi.y) - hy, 0.0f);
-                    const float ez = fmaxf(fmaxf(lo.z - seg[s].az, seg[s].az - hi.z) - hz, 0.0f);
-                    keep = ex * ex + ey * ey + ez * ez < A.rcull2;
-                    word = ((uint32_t)s << 26) | b;
-                }
-                const uint32_t m = __ballot_sync(0xffffffffu, keep);
-                if (keep) live[__popc(m & lt)] = word;
-                __syncwarp();
-                const int nl = __popc(m);
+                const int nl = live_blocks(base + lane, t1, seg, A.block_box, fr, A.fac.length, A.rcull2, live);
                 n_live += nl;
                 // the next block's coordinates are loaded while the current one is tested
                 uint32_t word_n = 0, xn = 0, yn = 0, zn = 0;
@@ -603,8 +485,8 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
                                 z = (float)(int)(zn - S.cz) * lambda;
                     const bool mine = slot - S.start < S.end - S.start;
                     if (k + 1 < nl) fetch(k + 1);
-                    const float ex = fmaxf(fabsf(x) - half[0], 0.0f), ey = fmaxf(fabsf(y) - half[1], 0.0f),
-                                ez = fmaxf(fabsf(z) - half[2], 0.0f);
+                    const float ex = fmaxf(fabsf(x) - hx, 0.0f), ey = fmaxf(fabsf(y) - hy, 0.0f),
+                                ez = fmaxf(fabsf(z) - hz, 0.0f);
                     const bool in = mine && ex * ex + ey * ey + ez * ez < rlist2;
                     const uint32_t mm = __ballot_sync(0xffffffffu, in);
                     if (in) {
@@ -628,7 +510,6 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
                         if (++n_chunks % kFlushChunks == 0) flush();
                     }
                 }
-                __syncwarp();  // live is rewritten by the next 32 blocks
             }
             // the rest of the list, padded to whole steps with far entries
             const int count = (fill + kStride - 1) / kStride * kStride;
@@ -640,8 +521,8 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
             n_list += fill;
             fill = 0;
         };
-        walk(std::true_type{}, 0u, own_blocks);
-        walk(std::false_type{}, own_blocks, all_blocks);
+        walk(std::true_type{}, 0u, blocks.x);
+        walk(std::false_type{}, blocks.x, blocks.y);
         __syncwarp();
 
         // particle t of the group: the sums of the 32/kPairsI lanes that shared it, in lane order
@@ -666,7 +547,7 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
             stat[0] += pairs;
             stat[1] += (n_live * kG);              // j's tested against the group's box, in slots of 32
             stat[2] += (n_list * kG + 16) / 32;    // list entries evaluated, the same
-            stat[3] += all_blocks - n_live;
+            stat[3] += blocks.y - n_live;
             stat[4] += n_chunks + 2;
         }
         __syncwarp();
@@ -684,18 +565,15 @@ cudaError_t pairs64_impl(p3m_ctx *c, const double *acc_in, double *acc_out, doub
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     const int grid = c->num_sms * per_sm;
-    GPoly64 gp;
-    for (int k = 0; k < P3M_SPLIT_DEG64 + 2; ++k) gp.c[k] = c->gpoly64[k];
-    // culling radii: r_c widened (narrowed) by more than the FP32 rounding of absolute
-    // coordinates up to the box size
-    const double rcull = c->g.r_c * (1.0 + 1e-4) + c->g.box * 1e-6;
-    const double rin = c->g.r_c * (1.0 - 1e-4) - c->g.box * 1e-6;
+    // culling radius: r_c widened by more than the FP32 rounding of absolute coordinates up to the
+    // box size; candidate radius (in cell sides): by more than the FP32 rounding of differences of up
+    // to two cells
+    const double rcull = c->g.r_c * (1.0 + 1e-4) + c->g.box * 1e-6, rlist = c->g.r_c / c->g.cs + 2e-6;
     c->launches += 1;
-    k_pairs64<<<grid, 32, 0, c->stream>>>(
-        (const double4_16a *)c->rel, c->pos, c->block_box, c->cell_start, c->work,
-        c->work_order, c->work_off + c->g.n_cells, c->g, gp, (float)(rcull * rcull),
-        rin > 0.0 ? (float)(rin * rin) : 0.0f, acc_in, acc_out, c->mom, kfac, kfac_dev,
-        c->counters, c->pair_count);
+    k_pairs64<<<grid, 32, 0, c->stream>>>(c->relq, c->pos, c->block_box, c->cell_start, c->work,
+                                          c->work_order, c->work_off + c->g.n_cells, c->g, c->split_tab,
+                                          (float)(rcull * rcull), (float)(rlist * rlist), acc_in, acc_out,
+                                          c->mom, kfac, kfac_dev, c->counters, c->pair_count);
     return cudaGetLastError();
 }
 

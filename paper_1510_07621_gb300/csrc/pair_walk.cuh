@@ -1,0 +1,138 @@
+// The walk over the neighbourhood of a group of particles that the pair kernels share.  A group is up
+// to 32 consecutive particles of one chaining cell, handled by one warp.  Its neighbour cells form 9
+// rows of 3 along x, each a contiguous range of sorted slots (two ranges where a row wraps); the
+// ranges' 32-slot blocks are tested 32 at a time, one per lane, against the group's bounding box.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "p3m_internal.cuh"
+
+namespace {
+
+constexpr int kPairSegs = 18;  // 9 rows of neighbour cells, each at most two ranges
+
+// The group's bounding box around an integer centre (fixed-point coordinates, kFixBits): centre,
+// half extents (scaled by lambda, rounded up), and the centre in absolute FP32 coordinates.
+struct GroupFrame {
+    uint32_t ctr[3];
+    float half[3], actr[3];
+};
+
+// One range of neighbour slots of a group: its slots, the group's centre in the range's periodic
+// image (fixed point, and absolute FP32 for the block boxes), the number of blocks before it and
+// the image as 3 x 2 bits (image index + 1).
+struct __align__(16) PairSeg {
+    uint32_t start, end, cx, cy;
+    uint32_t cz, first_block;
+    float ax, ay;
+    float az;
+    uint32_t image, pad[2];
+};
+
+__device__ __forceinline__ const uint32_t *fix_coords(const uint32_t *relq, uint32_t i)
+{
+    return relq + (size_t)(i >> 5) * 96 + (i & 31);
+}
+
+// Frame of the particles [first, min(first + kG, cend)) of cell (cx, cy, cz).
+template <int kG>
+__device__ __forceinline__ GroupFrame group_frame(const uint32_t *relq, uint32_t first, uint32_t cend,
+                                                  int cx, int cy, int cz, float lambda, float cell)
+{
+    GroupFrame f;
+    const int lane = threadIdx.x & 31;
+    const uint32_t *q = fix_coords(relq, min(first + min(lane, kG - 1), cend - 1));
+    const int c3[3] = {cx, cy, cz};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const uint32_t x = __ldg(q + 32 * d), x0 = __shfl_sync(0xffffffffu, x, 0);
+        const int lo = __reduce_min_sync(0xffffffffu, (int)(x - x0));
+        const int hi = __reduce_max_sync(0xffffffffu, (int)(x - x0));
+        const int mid = lo + ((hi - lo) >> 1);
+        f.ctr[d] = x0 + (uint32_t)mid;
+        f.half[d] = (float)(max(hi - mid, mid - lo)) * (1.0f + 0x1p-20f) * lambda;
+        // cell index and offset inside the cell, in cell sides
+        f.actr[d] = ((float)c3[d] + (float)(int)(f.ctr[d] - ((uint32_t)c3[d] << kFixBits)) * kFixUnit) * cell;
+    }
+    return f;
+}
+
+// Fills seg (the own row's two ranges first); returns the number of blocks of the own row and of all.
+__device__ __forceinline__ uint2 group_ranges(PairSeg *seg, const uint32_t *cell_start, const P3MGeom &g,
+                                              int cx, int cy, int cz, const GroupFrame &f, float cell)
+{
+    const int lane = threadIdx.x & 31, nc = g.n_c;
+    __syncwarp();  // the previous group is done with seg
+    uint32_t blocks = 0;
+    if (lane < kPairSegs) {
+        const int row = ((lane >> 1) + 4) % 9;  // the own row (4) comes first
+        const int uy = cy + row % 3 - 1, uz = cz + row / 3 - 1;
+        const int iy = uy < 0 ? -1 : (uy >= nc ? 1 : 0), iz = uz < 0 ? -1 : (uz >= nc ? 1 : 0);
+        int x0 = max(cx - 1, 0), x1 = min(cx + 1, nc - 1), ix = 0;
+        if (lane & 1) {  // the wrapped end of the row, if any
+            ix = cx == 0 ? -1 : (cx == nc - 1 ? 1 : 0);
+            x0 = x1 = cx == 0 ? nc - 1 : 0;
+        }
+        const uint32_t base = ((uint32_t)(uz - iz * nc) * nc + (uint32_t)(uy - iy * nc)) * nc;
+        uint32_t s = cell_start[base + x0], e = cell_start[base + x1 + 1];
+        if (!p3m_in_bounds(s <= e && e <= (uint32_t)g.n, g.flags)) e = s;
+        if ((lane & 1) && ix == 0) e = s;
+        PairSeg q;
+        q.start = s;
+        q.end = e;
+        const uint32_t box = (uint32_t)nc << kFixBits;  // the box side modulo 2^32
+        q.cx = f.ctr[0] - (uint32_t)ix * box;
+        q.cy = f.ctr[1] - (uint32_t)iy * box;
+        q.cz = f.ctr[2] - (uint32_t)iz * box;
+        q.ax = f.actr[0] - (float)(ix * nc) * cell;
+        q.ay = f.actr[1] - (float)(iy * nc) * cell;
+        q.az = f.actr[2] - (float)(iz * nc) * cell;
+        q.image = (uint32_t)(ix + 1) | (uint32_t)(iy + 1) << 2 | (uint32_t)(iz + 1) << 4;
+        q.pad[0] = q.pad[1] = 0;
+        const uint32_t mine = e > s ? ((e - 1) >> 5) - (s >> 5) + 1 : 0;
+        blocks = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync((1u << kPairSegs) - 1u, blocks, o);
+            if (lane >= o) blocks += y;
+        }
+        q.first_block = blocks - mine;
+        seg[lane] = q;
+    }
+    __syncwarp();
+    return make_uint2(__shfl_sync(0xffffffffu, blocks, 1), __shfl_sync(0xffffffffu, blocks, kPairSegs - 1));
+}
+
+// Tests block t of the ranges in sequence (t >= t1: none) against the group's box; the survivors of
+// the warp's 32 blocks go to live[0 ..] in order, coded (range << 26) | block.  Returns their number.
+// length: one scaled length (as in f.half); rcull2: the squared cutoff, padded by more than the FP32
+// rounding of absolute coordinates.
+__device__ __forceinline__ int live_blocks(uint32_t t, uint32_t t1, const PairSeg *seg,
+                                           const float4 *block_box, const GroupFrame &f, float length,
+                                           float rcull2, uint32_t *live)
+{
+    const int lane = threadIdx.x & 31;
+    bool keep = false;
+    uint32_t word = 0;
+    if (t < t1) {
+        int s = 0;  // the last range that starts at or before block t
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            if (s + o < kPairSegs && seg[s + o].first_block <= t) s += o;
+        const uint32_t b = (seg[s].start >> 5) + (t - seg[s].first_block);
+        const float4 lo = __ldg(block_box + 2 * (size_t)b), hi = __ldg(block_box + 2 * (size_t)b + 1);
+        const float ex = fmaxf(fmaxf(lo.x - seg[s].ax, seg[s].ax - hi.x) - f.half[0] * length, 0.0f);
+        const float ey = fmaxf(fmaxf(lo.y - seg[s].ay, seg[s].ay - hi.y) - f.half[1] * length, 0.0f);
+        const float ez = fmaxf(fmaxf(lo.z - seg[s].az, seg[s].az - hi.z) - f.half[2] * length, 0.0f);
+        keep = ex * ex + ey * ey + ez * ez < rcull2;
+        word = ((uint32_t)s << 26) | b;
+    }
+    const uint32_t m = __ballot_sync(0xffffffffu, keep);
+    __syncwarp();  // every lane is done with the previous survivors
+    if (keep) live[__popc(m & ((1u << lane) - 1u))] = word;
+    __syncwarp();
+    return __popc(m);
+}
+
+}  // namespace

@@ -519,7 +519,8 @@ __global__ void __launch_bounds__(256, 6) k_permute(const uint32_t *__restrict__
             dst[lane] = (float)rv.x;
             dst[32 + lane] = (float)rv.y;
             dst[64 + lane] = (float)rv.z;
-            // fixed point: 1.5 * 2^52 rounds x * scale to an integer in the low word (modulo 2^32)
+        }
+        {  // fixed point: 1.5 * 2^52 rounds x * scale to an integer in the low word (modulo 2^32)
             uint32_t *fix = relq + blk * 96;
             fix[lane] = (uint32_t)__double_as_longlong(fma(x, fix_scale, 0x1.8p52));
             fix[32 + lane] = (uint32_t)__double_as_longlong(fma(y, fix_scale, 0x1.8p52));
@@ -732,18 +733,19 @@ cudaError_t launch_permute_and_cells(p3m_ctx *c)
 {
     const int64_t n = c->g.n;
     const int gb = grid_for(n, 256, c->num_sms);
+    const double fix_scale = ldexp((double)c->g.n_c, kFixBits) / c->g.box;
     c->launches += 7;  // permute, cell_start, work_count, 3 scan kernels, work_fill
     if (c->precision == P3M_PREC_MIXED)
         k_permute<float4><<<gb, 256, 0, c->stream>>>(c->vals, c->keys, c->g, c->pos, c->mom,
                                                      c->pid, c->pos_alt, c->mom_alt, c->pid_alt,
                                                      (float4 *)c->rel, c->block_box, c->relx, c->relq,
-                                                     ldexp((double)c->g.n_c, kFixBits) / c->g.box,
+                                                     fix_scale,
                                                      c->tab_origin);
     else
         k_permute<double4_16a><<<gb, 256, 0, c->stream>>>(c->vals, c->keys, c->g, c->pos, c->mom,
                                                       c->pid, c->pos_alt, c->mom_alt,
                                                       c->pid_alt, (double4_16a *)c->rel, c->block_box,
-                                                      nullptr, nullptr, 0.0, c->tab_origin);
+                                                      nullptr, c->relq, fix_scale, c->tab_origin);
     double *t = c->pos;
     c->pos = c->pos_alt;
     c->pos_alt = t;

@@ -1,10 +1,15 @@
-"""The FP32 pair kernel's lists at the sizes where they can go wrong: groups of 16 particles with
+"""The pair kernels' lists.
+
+FP32: at the sizes where they can go wrong: groups of 16 particles with
 one more or one less, cells around a whole work item, rows of cells that wrap, lists longer than one
 chunk and one FP64 flush, both forms of the split factor (a softening small or large against r_s, a
-short and a long cutoff) and both list lengths.
+short and a long cutoff) and both list lengths.  Bars: the short-range accelerations within 1e-5
+relative RMS of the oracle (the FP32 bar), and the accepted pairs within the pairs whose distance
+lies within 1e-6 of the cutoff.
 
-Bars: the short-range accelerations within 1e-5 relative RMS of the oracle (the FP32 bar), and the
-accepted pairs within the pairs whose distance lies within 1e-6 of the cutoff."""
+FP64: groups of 8 particles with one more or one less, more candidate blocks than one round of masks
+holds, and a table of the split factor that covers a short or a long range.  Bars: 1e-12 relative RMS
+(the FP64 bar) and the same number of pairs."""
 
 import math
 
@@ -59,3 +64,26 @@ def test_pair_lists(kind, n, mesh, cutoff, softening, tile_blocks):
         assert abs(got - pairs) <= near
     else:
         assert abs(got - pairs) <= max(4, int(2e-6 * pairs))
+
+
+@pytest.mark.parametrize("kind,n,mesh,cutoff,softening", [
+    ("uniform", 2, 20, 4.5, 0.02), ("cell", 14, 20, 4.5, 0.0), ("cell", 16, 26, 4.5, 0.02),
+    ("cell", 18, 20, 4.5, 0.5), ("cell", 1500, 20, 4.5, 0.02), ("cell", 6001, 32, 4.5, 0.0),
+    ("uniform", 4097, 24, 1.5, 0.02), ("uniform", 4097, 48, 6.0, 1.0),
+])
+def test_pair_masks_fp64(kind, n, mesh, cutoff, softening):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1510_07621_gb300 import P3M, build
+    build.build()
+    box = 50.0
+    x = _set(kind, n, box, 2000 + n + mesh)
+    p = O.Params(box, n, mesh, 1.25, cutoff, softening)
+    ref, pairs = O.sr_accel(O.wrap(x, box), p)
+    with P3M(box, n, mesh, 1.25, cutoff, softening=softening, precision="fp64") as sim:
+        sim.set_particles(x, np.zeros_like(x), a=1.0)
+        _, sr = sim.forces_split()
+        got = sim.diagnostics()["pairs"]
+    assert math.sqrt(float(np.sum((sr - ref) ** 2))) <= 1e-12 * math.sqrt(float(np.sum(ref ** 2)))
+    assert got == pairs
