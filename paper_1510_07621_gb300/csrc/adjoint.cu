@@ -18,6 +18,7 @@
 
 #include "p3m_device.cuh"
 #include "p3m_internal.cuh"
+#include "pair_walk.cuh"
 
 namespace {
 
@@ -262,11 +263,6 @@ __global__ void k_sum_parts(double *part, int nb, double *out)
 
 // ------------------------------------------------------------------ pair part
 
-// Coefficients of the FP32 split factor (the context's fitted polynomial, see p3m_ctx::gpoly).
-struct GPolyA {
-    float c[12];
-};
-
 // h(r)/Gm and h'(r)/(Gm r) for one pair in FP64, g and g' in closed form.
 __device__ __forceinline__ void pair_jac(double r2, double eps2, double inv_rs, double &h,
                                          double &hr)
@@ -385,276 +381,245 @@ __global__ void __launch_bounds__(32)
     }
 }
 
-// FP32 mode: the force kernel's traversal and arithmetic style (one-warp persistent CTAs,
-// bulk-copy tiles of the block-SoA coordinates and v, block culling, the all-inside fast path,
-// two j particles per lane in packed f32x2, per-tile FP32 sums added in FP64), for
-//   out_k += Gm sum_j [h(r) w + (h'(r)/r)(d.w) d],  w = v_j - v_k,
-//   h = g s^3, h'/r = -(r e / (2 sqrt(pi) r_s^3)) s^3 - 3 h s^2,  s = (r^2 + eps^2)^-1/2,
-//   e = exp(-r^2 / (4 r_s^2)),
-// g from the fitted polynomial (g'(x) = -x^2 exp(-x^2/4) / (2 sqrt(pi)) in closed form).  r^2
-// starts at kVjpTiny = 1e-20 like in the force kernel; r = 0 pairs are selected out (their w need
-// not vanish for coincident particles).  r^2 = kVjpTiny can only occur in the work item's own
-// cell (the particle itself, coincident particles), so only the own cell tests r^2 > kVjpTiny.
-// Tiles of 3 blocks of coordinates and v (4.5 KB for both buffers) keep 32 CTAs per SM.
-constexpr float kVjpTiny = 1e-20f;
-constexpr int kVjpBlocksPerTile = 3;
+// FP32 mode: the force kernel's lists (k_pairs_list in pair.cu: groups of 16 particles, candidates
+// tested one per lane against the group's box, the accepted ones compacted into a list, two particles
+// and two list entries per lane in packed f32x2 arithmetic), here with v beside the coordinates, for
+//   out_k += Gm sum_j [h w + (h'/r) (d.w) d],  w = v_j - v_k,
+// where h is the force kernel's fitted factor and h'/r, in the additive form, twice the derivative of
+// that fit with respect to w = r^2 + eps^2 (scaled lengths, q = s + ab + na t, k = ln 2):
+//   h = q s^2 + P(t),  h'/r = t (2 k (-na) s^2 - 2 k P'(t)) - (2 q + s) s^4,
+// as accurate as the closed form (1.9e-7 against 3.8e-7 of the force derivative at the cutoff 4.5) and
+// without a second exponential.  The general form takes g' = -x^2 exp(-x^2/4)/(2 sqrt(pi)) closed.
+// s^4 is never formed: (2 q + s) s^2 times s^2 (d.w) stays finite for close pairs without softening.
+// r = 0 pairs are selected out (their w need not vanish for coincident particles); only the row of the
+// own cell can hold them.  Before, all 32 lanes met every j of a tested block with 40 FP32 operations
+// and three 8-cycle MUFU operations per pair (34 and one here).  128^3 near-uniform, one call with the
+// mesh part: 9.35 -> 7.13 ms, the pair part 7.6 -> 5.4.  What bounds it: of 137 cycles per 32 accepted
+// pairs and scheduler, 110 are the evaluation (52 per 32 slots, 47 % of them accepted).  8 or 32
+// particles per group, 18 or 20 CTAs per SM and lists of 192 are within 2 % or slower.
+constexpr int kVjpGroup = 16, kVjpChunk = 128, kVjpFlush = 5;  // (16 FP32 terms per chunk and sum)
+constexpr float kVjpTiny = 1e-24f, kVjpFar = 1e6f;
 
 struct VjpConst2 {
-    f2 c[P3M_SPLIT_DEG + 1];
-    f2 c11, m1, one, eps2, tiny, ex2arg, c1, m3;
+    f2 c[5], d[3];  // P, and -2 k P' as d[0] + d[1] t + d[2] t^2 (additive form)
+    f2 na, ab, e2, na2, two;
 };
 
-// h and h'/r of both halves of r2 (r2 includes kVjpTiny)
-__device__ __forceinline__ void pair_jac2(f2 r2, const VjpConst2 &k, f2 &h, f2 &hr)
+// h, and (h'/r) dw as *c, for both halves of w (see PairFactor)
+template <bool kAdditive>
+__device__ __forceinline__ f2 pair_jac2(f2 w, f2 dw, const VjpConst2 &k, f2 *c)
 {
-    float r2l, r2h, s2l, s2h, al, ah;
-    const f2 s2 = f2_add(r2, k.eps2);
-    f2_unpack(r2, r2l, r2h);
-    f2_unpack(s2, s2l, s2h);
-    const f2 s = f2_pack(rsqrt_approx(s2l), rsqrt_approx(s2h));
-    const f2 r = f2_pack(sqrt_approx(r2l), sqrt_approx(r2h));
-    const f2 tau = f2_fma(r2, k.c11, k.m1);
-    f2 p = k.c[P3M_SPLIT_DEG];
-#pragma unroll
-    for (int q = P3M_SPLIT_DEG - 1; q >= 0; --q) p = f2_fma(p, tau, k.c[q]);
-    const f2 gval = f2_fma(f2_mul(r2, r), p, k.one);
-    const f2 ss = f2_mul(s, s);
-    const f2 s3 = f2_mul(ss, s);
-    h = f2_mul(gval, s3);
-    f2_unpack(f2_mul(r2, k.ex2arg), al, ah);  // -r^2 log2(e) / (4 r_s^2)
-    const f2 e = f2_pack(ex2_approx(al), ex2_approx(ah));
-    const f2 res3 = f2_mul(f2_mul(r, e), s3);
-    hr = f2_fma(res3, k.c1, f2_mul(f2_mul(h, ss), k.m3));  // c1 = -1/(2 sqrt(pi) r_s^3), m3 = -3
+    const f2 t = f2_pack(ex2_approx(-w.x), ex2_approx(-w.y));
+    const f2 rw = f2_pack(rsqrt_approx(w.x), rsqrt_approx(w.y));
+    f2 p = kAdditive ? k.c[3] : f2_fma(k.c[4], t, k.c[3]);
+    p = f2_fma(p, t, k.c[2]);
+    p = f2_fma(p, t, k.c[1]);
+    if (kAdditive) {
+        const f2 q = f2_add(rw, f2_fma(k.na, t, k.ab)), s2 = f2_mul(rw, rw);
+        const f2 h = f2_fma(p, t, f2_fma(q, s2, k.c[0]));
+        const f2 dp = f2_fma(f2_fma(k.d[2], t, k.d[1]), t, k.d[0]);
+        const f2 inner = f2_mul(t, f2_fma(k.na2, s2, dp));
+        const f2 m = f2_mul(f2_fma(k.two, q, rw), s2);
+        *c = f2_fma(inner, dw, f2_neg(f2_mul(m, f2_mul(s2, dw))));
+        return h;
+    }
+    // d[0]: exponent of exp(-r^2/(4 r_s^2)) over t's, d[1]: -1/(2 sqrt(pi)) in scaled lengths, d[2]: -3
+    p = f2_fma(p, t, k.c[0]);
+    const f2 su = f2_add(w, k.e2), eu = f2_mul(w, k.d[0]);
+    const f2 s = f2_pack(rsqrt_approx(su.x), rsqrt_approx(su.y));
+    const f2 e = f2_pack(ex2_approx(-eu.x), ex2_approx(-eu.y));
+    const f2 r = f2_mul(w, rw), s2 = f2_mul(s, s), s3 = f2_mul(s2, s);
+    const f2 gv = f2_fma(r, f2_fma(w, p, f2_fma(k.na, t, k.ab)), f2_pack(1.0f, 1.0f));
+    const f2 h = f2_mul(gv, s3);
+    *c = f2_fma(f2_mul(f2_mul(r, e), f2_mul(s3, k.d[1])), dw, f2_mul(f2_mul(h, k.d[2]), f2_mul(s2, dw)));
+    return h;
 }
 
-__global__ void __launch_bounds__(32, 32)
-    k_pairs_vjp_x2(const float *__restrict__ relx, const float *__restrict__ vfx,
-                   const float4 *__restrict__ rel, const double *__restrict__ pos,
-                   const float4 *__restrict__ block_box, const uint32_t *__restrict__ cell_start,
-                   const uint32_t *__restrict__ work, const uint32_t *__restrict__ order,
-                   const uint32_t *__restrict__ n_work_ptr, P3MGeom g, GPolyA gp, float rcull2,
-                   float rin2, uint32_t *__restrict__ cursor, uint32_t *__restrict__ flags,
-                   double *__restrict__ out)
+template <bool kAdditive>
+__global__ void __launch_bounds__(32, 16)
+    k_pairs_vjp_list(const uint32_t *__restrict__ relq, const float *__restrict__ vfx,
+                     const float4 *__restrict__ block_box, const uint32_t *__restrict__ cell_start,
+                     const uint32_t *__restrict__ work, const uint32_t *__restrict__ order,
+                     const uint32_t *__restrict__ n_work_ptr, P3MGeom g, PairFactor fac, double scale,
+                     float rcull2, uint32_t *__restrict__ cursor, double *__restrict__ out)
 {
-    constexpr int kBlockFloats = 96;
-    __shared__ __align__(128) float sj[2][kVjpBlocksPerTile * kBlockFloats];
-    __shared__ __align__(128) float sv[2][kVjpBlocksPerTile * kBlockFloats];
-    __shared__ __align__(16) float4 sbox[2][2 * kVjpBlocksPerTile];  // the tile's block boxes
-    __shared__ __align__(8) uint64_t bar[2];
-    __shared__ NeighbourF nbr[27];
+    constexpr int kG = kVjpGroup, kPairsI = kG / 2, kStride = 2 * (32 / kPairsI), kSub = P3M_PAIR_TI / kG;
+    __shared__ __align__(16) float list[6][kVjpChunk + 32];  // x, y, z, vx, vy, vz
+    __shared__ double sum[6][32];
+    __shared__ PairSeg seg[kPairSegs];
+    __shared__ uint32_t live[32];
 
-    const int lane = threadIdx.x;
+    const int lane = threadIdx.x, ip = lane % kPairsI, js = lane / kPairsI;
+    const uint32_t lt = (1u << lane) - 1u;
     const int64_t n = g.n;
-    const uint32_t n_work = *n_work_ptr;
-    const float rc2 = (float)(g.r_c * g.r_c);
+    const uint32_t n_units = *n_work_ptr * kSub;
     const int nc = g.n_c;
+    const float lambda = fac.lambda, rc2 = fac.rc2, rlist2 = fac.rlist2;
     VjpConst2 kc;
 #pragma unroll
-    for (int q = 0; q <= P3M_SPLIT_DEG; ++q) kc.c[q] = f2_pack(gp.c[q], gp.c[q]);
-    kc.c11 = f2_pack(gp.c[11], gp.c[11]);
-    kc.m1 = f2_pack(-1.0f, -1.0f);
-    kc.one = f2_pack(1.0f, 1.0f);
-    const float e2 = (float)(g.eps * g.eps);
-    kc.eps2 = f2_pack(e2, e2);
-    kc.tiny = f2_pack(kVjpTiny, kVjpTiny);
-    const float xa_ = (float)(-1.4426950408889634 / (4.0 * g.r_s * g.r_s));
-    kc.ex2arg = f2_pack(xa_, xa_);
-    const float c1 = (float)(-0.28209479177387814347 / (g.r_s * g.r_s * g.r_s));
-    kc.c1 = f2_pack(c1, c1);
-    kc.m3 = f2_pack(-3.0f, -3.0f);
-
-    if (lane == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-        mbar_fence_init();
+    for (int q = 0; q < 5; ++q) kc.c[q] = f2_pack(fac.c[q], fac.c[q]);
+    kc.na = f2_pack(fac.na, fac.na);
+    kc.ab = f2_pack(fac.ab, fac.ab);
+    kc.e2 = f2_pack(fac.e2, fac.e2);
+    const float k2 = 2.0f * 0.69314718055994531f;
+    kc.na2 = f2_pack(-k2 * fac.na, -k2 * fac.na);
+    kc.two = f2_pack(2.0f, 2.0f);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const float d = kAdditive ? -k2 * (float)(q + 1) * fac.c[q + 1] : fac.grad[q];
+        kc.d[q] = f2_pack(d, d);
     }
-    __syncwarp();
-    uint32_t parity = 0u;
-    bool timed_out = false;
+    const f2 w0 = kAdditive ? kc.e2 : f2_pack(kVjpTiny, kVjpTiny);
 
     for (;;) {
-        uint32_t slot = 0;
-        if (lane == 0) slot = atomicAdd(cursor, 1u);
-        slot = __shfl_sync(0xffffffffu, slot, 0);
-        if (slot >= n_work) break;
-        const uint32_t item = order[slot];
+        uint32_t unit = 0;
+        if (lane == 0) unit = atomicAdd(cursor, 1u);
+        unit = __shfl_sync(0xffffffffu, unit, 0);
+        if (unit >= n_units) break;
+        const uint32_t item = order[unit / kSub];
         const uint32_t cell = work[2 * (size_t)item];
-        const uint32_t first = work[2 * (size_t)item + 1];
+        const uint32_t first = work[2 * (size_t)item + 1] + (unit % kSub) * kG;
         const uint32_t cend = cell_start[cell + 1];
+        if (first >= cend) continue;
         const int cx = (int)(cell % nc), cy = (int)((cell / nc) % nc), cz = (int)(cell / (nc * nc));
-        __syncwarp();  // the previous item is done with nbr
-        if (lane < 27) nbr[lane] = make_neighbour(g, cell_start, cx, cy, cz, lane);
+        const GroupFrame fr = group_frame<kG>(relq, first, cend, cx, cy, cz, lambda, fac.cell);
+        const uint2 blocks = group_ranges(seg, cell_start, g, cx, cy, cz, fr, fac.cell);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) sum[q][lane] = 0.0;
+
+        // the lane's two particles, coordinates and v negated
+        f2 nx[2][3], nv[2][3], o[2][3];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const uint32_t i = min(first + ip + u * kPairsI, cend - 1);
+            const uint32_t *q = fix_coords(relq, i);
+            const float *v = vfx + (size_t)(i >> 5) * 96 + (i & 31);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const float x = (float)(int)(__ldg(q + 32 * d) - fr.ctr[d]) * -lambda, y = -__ldg(v + 32 * d);
+                nx[u][d] = f2_pack(x, x);
+                nv[u][d] = f2_pack(y, y);
+                o[u][d] = f2_pack(0.0f, 0.0f);
+            }
+        }
+        auto flush = [&]() {
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    sum[3 * u + d][lane] += (double)(o[u][d].x + o[u][d].y);
+                    o[u][d] = f2_pack(0.0f, 0.0f);
+                }
+        };
+        // list entries [0, count), count a multiple of kStride
+        auto eval = [&](auto own, int count) {
+#pragma unroll 1
+            for (int k = 2 * js; k < count; k += kStride) {
+                f2 X[3], V[3];
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    X[d] = *(const f2 *)&list[d][k];
+                    V[d] = *(const f2 *)&list[3 + d][k];
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    f2 dx[3], wv[3];
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        dx[d] = f2_add(X[d], nx[u][d]);
+                        wv[d] = f2_add(V[d], nv[u][d]);
+                    }
+                    const f2 w = f2_fma(dx[2], dx[2], f2_fma(dx[1], dx[1], f2_fma(dx[0], dx[0], w0)));
+                    const f2 dw = f2_fma(dx[2], wv[2], f2_fma(dx[1], wv[1], f2_mul(dx[0], wv[0])));
+                    f2 c, h = pair_jac2<kAdditive>(w, dw, kc, &c);
+                    bool lo = w.x < rc2, hi = w.y < rc2;
+                    if (decltype(own)::value) {
+                        lo = lo && (__float_as_uint(dx[0].x) | __float_as_uint(dx[1].x) | __float_as_uint(dx[2].x)) != 0u;
+                        hi = hi && (__float_as_uint(dx[0].y) | __float_as_uint(dx[1].y) | __float_as_uint(dx[2].y)) != 0u;
+                    }
+                    h = f2_pack(lo ? h.x : 0.0f, hi ? h.y : 0.0f);
+                    c = f2_pack(lo ? c.x : 0.0f, hi ? c.y : 0.0f);
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) o[u][d] = f2_fma(h, wv[d], f2_fma(c, dx[d], o[u][d]));
+                }
+            }
+        };
+
+        int fill = 0, chunks = 0;
+        auto walk = [&](auto own, uint32_t t0, uint32_t t1) {
+            for (uint32_t base = t0; base < t1; base += 32) {
+                const int nl = live_blocks(base + lane, t1, seg, block_box, fr, fac.length, rcull2, live);
+                // the next block's data are loaded while the current one is tested
+                uint32_t word_n = 0, qn[3];
+                float vn[3];
+                auto fetch = [&](int k) {
+                    word_n = live[k];
+                    const size_t at = (size_t)(word_n & 0x3FFFFFFu) * 96 + lane;
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        qn[d] = __ldg(relq + at + 32 * d);
+                        vn[d] = __ldg(vfx + at + 32 * d);
+                    }
+                };
+                if (nl) fetch(0);
+#pragma unroll 1
+                for (int k = 0; k < nl; ++k) {
+                    const PairSeg &S = seg[word_n >> 26];
+                    const uint32_t slot = (word_n & 0x3FFFFFFu) * 32 + lane;
+                    const float x = (float)(int)(qn[0] - S.cx) * lambda, y = (float)(int)(qn[1] - S.cy) * lambda,
+                                z = (float)(int)(qn[2] - S.cz) * lambda;
+                    const float vx = vn[0], vy = vn[1], vz = vn[2];
+                    const bool mine = slot - S.start < S.end - S.start;
+                    if (k + 1 < nl) fetch(k + 1);
+                    const float ex = fmaxf(fabsf(x) - fr.half[0], 0.0f), ey = fmaxf(fabsf(y) - fr.half[1], 0.0f),
+                                ez = fmaxf(fabsf(z) - fr.half[2], 0.0f);
+                    const bool in = mine && ex * ex + ey * ey + ez * ez < rlist2;
+                    const uint32_t mm = __ballot_sync(0xffffffffu, in);
+                    if (in) {
+                        const int p = fill + __popc(mm & lt);
+                        list[0][p] = x;
+                        list[1][p] = y;
+                        list[2][p] = z;
+                        list[3][p] = vx;
+                        list[4][p] = vy;
+                        list[5][p] = vz;
+                    }
+                    fill += __popc(mm);
+                    if (fill >= kVjpChunk) {
+                        __syncwarp();
+                        eval(own, kVjpChunk);
+                        __syncwarp();
+                        fill -= kVjpChunk;
+                        if (lane < fill)  // (fill < 32 <= kVjpChunk: no overlap)
+                            for (int d = 0; d < 6; ++d) list[d][lane] = list[d][kVjpChunk + lane];
+                        if (++chunks % kVjpFlush == 0) flush();
+                    }
+                }
+            }
+            // the rest of the list, padded to whole steps with far entries
+            const int count = (fill + kStride - 1) / kStride * kStride;
+            if (lane < count - fill)
+                for (int d = 0; d < 6; ++d) list[d][fill + lane] = d < 3 ? kVjpFar : 0.0f;
+            __syncwarp();
+            eval(own, count);
+            __syncwarp();
+            flush();
+            fill = 0;
+        };
+        walk(std::true_type{}, 0u, blocks.x);
+        walk(std::false_type{}, blocks.x, blocks.y);
         __syncwarp();
-
-        const uint32_t i = first + lane;
-        const bool valid = i < cend;
-        const uint32_t ii = valid ? i : first;
-        const float4 xi = rel[ii];
-        const float xa = (float)pos[ii], ya = (float)pos[n + ii], za = (float)pos[2 * n + ii];
-        const float *vi = vfx + (ii >> 5) * kBlockFloats + (ii & 31);
-        const f2 vix2 = f2_pack(vi[0], vi[0]), viy2 = f2_pack(vi[32], vi[32]),
-                 viz2 = f2_pack(vi[64], vi[64]);
-        double sox = 0.0, soy = 0.0, soz = 0.0;
-
-        auto next_tile = [&](int &nb, uint32_t &b) {
-            while (nb < 27 && b * 32u >= nbr[nb].end) {
-                ++nb;
-                if (nb < 27) b = nbr[nb].start >> 5;
-            }
-        };
-        auto issue = [&](int nb, uint32_t b, int to) {
-            const uint32_t bend = min(b + kVjpBlocksPerTile, (nbr[nb].end + 31) >> 5);
-            const uint32_t bytes = (bend - b) * (uint32_t)(kBlockFloats * sizeof(float));
-            const uint32_t box_bytes = (bend - b) * (uint32_t)(2 * sizeof(float4));
-            mbar_expect_tx(&bar[to], 2 * bytes + box_bytes);
-            bulk_load(&sj[to][0], relx + (size_t)b * kBlockFloats, bytes, &bar[to]);
-            bulk_load(&sv[to][0], vfx + (size_t)b * kBlockFloats, bytes, &bar[to]);
-            bulk_load(&sbox[to][0], block_box + 2 * (size_t)b, box_bytes, &bar[to]);
-        };
-
-        int nb_c = 0;
-        uint32_t b_c = nbr[0].start >> 5;
-        next_tile(nb_c, b_c);
-        int buf = 0;
-        if (nb_c < 27 && lane == 0) issue(nb_c, b_c, 0);
-        // x_i in the current neighbour cell's frame, set when the tile walk enters the cell
-        int nb_frame = -1;
-        f2 xs2 = make_float2(0.0f, 0.0f), ys2 = xs2, zs2 = xs2;
-        float cxs = 0.0f, cys = 0.0f, czs = 0.0f;
-        while (nb_c < 27) {
-            const uint32_t nstart = nbr[nb_c].start, nend = nbr[nb_c].end;
-            const uint32_t bend = min(b_c + kVjpBlocksPerTile, (nend + 31) >> 5);
-            int nb_n = nb_c;
-            uint32_t b_n = bend;
-            next_tile(nb_n, b_n);
-            __syncwarp();  // every lane is done with the other buffer before it is refilled
-            if (nb_n < 27 && lane == 0) issue(nb_n, b_n, buf ^ 1);
-            const bool ok = mbar_wait_bounded(&bar[buf], (parity >> buf) & 1u);
-            parity ^= 1u << buf;
-            if (__any_sync(0xffffffffu, !ok)) {
-                timed_out = true;
-                if (nb_n < 27) mbar_wait_bounded(&bar[buf ^ 1], (parity >> (buf ^ 1)) & 1u);
-                break;
-            }
-            if (nb_c != nb_frame) {
-                nb_frame = nb_c;
-                const NeighbourF &q = nbr[nb_c];
-                const float xs = (xi.x - q.sx) - q.rx;
-                const float ys = (xi.y - q.sy) - q.ry;
-                const float zs = (xi.z - q.sz) - q.rz;
-                xs2 = f2_pack(xs, xs);
-                ys2 = f2_pack(ys, ys);
-                zs2 = f2_pack(zs, zs);
-                cxs = xa - q.imx;
-                cys = ya - q.imy;
-                czs = za - q.imz;
-            }
-            f2 ox = make_float2(0.0f, 0.0f), oy = ox, oz = ox;
-
-            // pair (j, j+1) from packed coordinates (x, y, z) and v (u, v, w); lo/hi: which
-            // halves take part; test: r < r_c; own: the work item's own cell (r^2 > kVjpTiny test)
-            auto pair_vjp = [&](auto own, f2 xj, f2 yj, f2 zj, f2 uj, f2 vj, f2 wj, bool lo,
-                                bool hi, bool test) {
-                const f2 dx = f2_sub(xj, xs2), dy = f2_sub(yj, ys2), dz = f2_sub(zj, zs2);
-                const f2 r2 = f2_fma(dz, dz, f2_fma(dy, dy, f2_fma(dx, dx, kc.tiny)));
-                float r2l, r2h;
-                f2_unpack(r2, r2l, r2h);
-                const bool own_c = decltype(own)::value;
-                const bool inl = lo && (!own_c || r2l > kVjpTiny) && (!test || r2l < rc2);
-                const bool inh = hi && (!own_c || r2h > kVjpTiny) && (!test || r2h < rc2);
-                if (test && !__any_sync(0xffffffffu, inl || inh)) return;
-                f2 h, hr;
-                pair_jac2(r2, kc, h, hr);
-                const f2 wx = f2_sub(uj, vix2), wy = f2_sub(vj, viy2), wz = f2_sub(wj, viz2);
-                const f2 dw = f2_fma(dz, wz, f2_fma(dy, wy, f2_mul(dx, wx)));
-                f2 hs = h, cs = f2_mul(hr, dw);
-                if (own_c || test || !(lo && hi)) {
-                    float hl, hh, cl, ch;
-                    f2_unpack(hs, hl, hh);
-                    f2_unpack(cs, cl, ch);
-                    hs = f2_pack(inl ? hl : 0.0f, inh ? hh : 0.0f);
-                    cs = f2_pack(inl ? cl : 0.0f, inh ? ch : 0.0f);
-                }
-                ox = f2_fma(cs, dx, f2_fma(hs, wx, ox));
-                oy = f2_fma(cs, dy, f2_fma(hs, wy, oy));
-                oz = f2_fma(cs, dz, f2_fma(hs, wz, oz));
-            };
-            // the aligned pair (p, p+1) of the block at bx / bv
-            auto pair_at = [&](auto own, const float *bx, const float *bv, uint32_t p, bool lo,
-                               bool hi, bool test) {
-                const f2 *x2 = (const f2 *)bx, *v2 = (const f2 *)bv;
-                pair_vjp(own, x2[p / 2], x2[16 + p / 2], x2[32 + p / 2], v2[p / 2], v2[16 + p / 2],
-                         v2[32 + p / 2], lo, hi, test);
-            };
-
-            auto blocks = [&](auto own) {
-            for (uint32_t b = b_c; b < bend; ++b) {
-                const float4 lo = sbox[buf][2 * (b - b_c)], hi = sbox[buf][2 * (b - b_c) + 1];
-                const float ex = fmaxf(fmaxf(lo.x - cxs, cxs - hi.x), 0.0f);
-                const float ey = fmaxf(fmaxf(lo.y - cys, cys - hi.y), 0.0f);
-                const float ez = fmaxf(fmaxf(lo.z - czs, czs - hi.z), 0.0f);
-                if (!__any_sync(0xffffffffu, valid && ex * ex + ey * ey + ez * ez < rcull2)) continue;
-                const uint32_t j0 = max(b * 32, nstart) - b * 32;
-                const uint32_t j1 = min(b * 32 + 32, nend) - b * 32;
-                const float *bx = sj[buf] + (b - b_c) * kBlockFloats;
-                const float *bv = sv[buf] + (b - b_c) * kBlockFloats;
-                const float fx = fmaxf(cxs - lo.x, hi.x - cxs);
-                const float fy = fmaxf(cys - lo.y, hi.y - cys);
-                const float fz = fmaxf(czs - lo.z, hi.z - czs);
-                const bool test =
-                    !__all_sync(0xffffffffu, !valid || fx * fx + fy * fy + fz * fz < rin2);
-                uint32_t p = j0 & ~1u;
-                if ((j0 & 1u) && j0 < j1) {
-                    pair_at(own, bx, bv, p, false, true, true);
-                    p += 2;
-                }
-                if (test) {
-                    for (; p + 1 < j1; p += 2) pair_at(own, bx, bv, p, true, true, true);
-                } else {
-                    if ((p & 2u) && p + 1 < j1) {
-                        pair_at(own, bx, bv, p, true, true, false);
-                        p += 2;
-                    }
-                    for (; p + 3 < j1; p += 4) {  // four j: 16-byte loads
-                        const float4 X = *(const float4 *)(bx + p), Y = *(const float4 *)(bx + 32 + p),
-                                     Z = *(const float4 *)(bx + 64 + p);
-                        const float4 U = *(const float4 *)(bv + p), V = *(const float4 *)(bv + 32 + p),
-                                     W = *(const float4 *)(bv + 64 + p);
-                        pair_vjp(own, f2_pack(X.x, X.y), f2_pack(Y.x, Y.y), f2_pack(Z.x, Z.y),
-                                 f2_pack(U.x, U.y), f2_pack(V.x, V.y), f2_pack(W.x, W.y), true, true,
-                                 false);
-                        pair_vjp(own, f2_pack(X.z, X.w), f2_pack(Y.z, Y.w), f2_pack(Z.z, Z.w),
-                                 f2_pack(U.z, U.w), f2_pack(V.z, V.w), f2_pack(W.z, W.w), true, true,
-                                 false);
-                    }
-                    for (; p + 1 < j1; p += 2) pair_at(own, bx, bv, p, true, true, false);
-                }
-                if (p < j1) pair_at(own, bx, bv, p, true, false, true);
-            }
-            };
-            if (nb_c == 13)
-                blocks(std::true_type{});
-            else
-                blocks(std::false_type{});
-            float lo_, hi_;
-            f2_unpack(ox, lo_, hi_);
-            sox += (double)(lo_ + hi_);
-            f2_unpack(oy, lo_, hi_);
-            soy += (double)(lo_ + hi_);
-            f2_unpack(oz, lo_, hi_);
-            soz += (double)(lo_ + hi_);
-            buf ^= 1;
-            nb_c = nb_n;
-            b_c = b_n;
+        for (int t = lane; t < 3 * kG; t += 32) {
+            const int d = t / kG, k = t % kG;
+            const uint32_t i = first + k;
+            if (i >= cend) continue;
+            double s = 0.0;
+#pragma unroll
+            for (int o_ = 0; o_ < 32 / kPairsI; ++o_) s += sum[3 * (k / kPairsI) + d][o_ * kPairsI + k % kPairsI];
+            out[d * n + i] += scale * s;
         }
-        if (timed_out) break;
-        if (valid) {
-            out[i] += g.gm * sox;
-            out[n + i] += g.gm * soy;
-            out[2 * n + i] += g.gm * soz;
-        }
+        __syncwarp();  // sum is cleared for the next group
     }
-    if (timed_out && lane == 0) atomicOr(flags, P3M_FLAG_TIMEOUT);
 }
 
 // ------------------------------------------------------------------ potential energy
@@ -940,7 +905,8 @@ cudaError_t vjp_pairs(p3m_ctx *c, const double *v_slots, double *out_slots)
 {
     int per_sm = 0;
     const bool fp32 = c->precision == P3M_PREC_MIXED;
-    cudaError_t e = fp32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pairs_vjp_x2, 32, 0)
+    auto list = c->pair_factor.additive ? k_pairs_vjp_list<true> : k_pairs_vjp_list<false>;
+    cudaError_t e = fp32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, list, 32, 0)
                          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pairs_vjp64, 32, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
@@ -951,12 +917,11 @@ cudaError_t vjp_pairs(p3m_ctx *c, const double *v_slots, double *out_slots)
     const float rcull2 = (float)(rcull * rcull), rin2 = rin > 0.0 ? (float)(rin * rin) : 0.0f;
     c->launches += 1;
     if (fp32) {
-        GPolyA gp;
-        for (int k = 0; k < 12; ++k) gp.c[k] = c->gpoly[k];
-        k_pairs_vjp_x2<<<c->num_sms * per_sm, 32, 0, c->stream>>>(
-            c->relx, c->adj_vfx, (const float4 *)c->rel, c->pos, c->block_box, c->cell_start, c->work,
-            c->work_order, c->work_off + c->g.n_cells, c->g, gp, rcull2, rin2, c->counters + 3,
-            c->counters + 1, out_slots);
+        const double len = ldexp(c->g.cs, -kFixBits) / (double)c->pair_factor.lambda;
+        list<<<c->num_sms * per_sm, 32, 0, c->stream>>>(
+            c->relq, c->adj_vfx, c->block_box, c->cell_start, c->work, c->work_order,
+            c->work_off + c->g.n_cells, c->g, c->pair_factor, c->g.gm / (len * len * len), rcull2,
+            c->counters + 3, out_slots);
     } else {
         k_pairs_vjp64<<<c->num_sms * per_sm, 32, 0, c->stream>>>(
             (const double4_16a *)c->rel, c->pos, c->block_box, v_slots, c->cell_start, c->work,

@@ -77,13 +77,8 @@ double quad(const p3m_cosmology &cs, double a1, double a2, int power)
     return 0.5 * (a2 - a1) * s;
 }
 
-// ---------------------------------------------------------------- split factor fit
-// g(x) = erfc(x/2) + x/sqrt(pi) exp(-x^2/4) = 1 + x^3 Q(x^2).  Q is smooth (entire) in u = x^2;
-// it is interpolated at Chebyshev-Gauss nodes of u in [0, u_c], u_c = (r_c/r_s)^2, truncated to
-// the wanted degree (a near-minimax polynomial), and rewritten in monomial form in
-// tau = 2u/u_c - 1 for Horner evaluation (the monomial coefficients stay below 0.03 in size up to
-// degree 22, so the rewriting costs no accuracy).  The kernels evaluate g = 1 + r^3 Q'(tau)
-// directly from r^2, so the coefficients are scaled by r_s^-3 and tau = r^2 (2 / (u_c r_s^2)) - 1.
+// ---------------------------------------------------------------- split factor
+// g(x) = erfc(x/2) + x/sqrt(pi) exp(-x^2/4) = 1 + x^3 Q(x^2), Q smooth (entire) in u = x^2.
 
 // Q(u): below u = 1 from its Taylor series (the closed form cancels there),
 // Q(u) = (1/sqrt(pi)) sum_{n>=1} (-1)^n u^(n-1) 2n / (4^n n! (2n+1)); above, (g - 1)/(u x).
@@ -101,46 +96,6 @@ double split_q(double u)
     const double x = sqrt(u);
     const double gval = erfc(0.5 * x) + x * inv_sqrt_pi * exp(-0.25 * u);
     return (gval - 1.0) / (u * x);
-}
-
-// Monomial coefficients mono[0..deg] of Q in tau (unscaled), from `nodes` Chebyshev nodes.
-void fit_split_mono(double cutoff_in_rs, int deg, int nodes, double *mono)
-{
-    const double uc = cutoff_in_rs * cutoff_in_rs;
-    std::vector<double> cheb(deg + 1, 0.0), tk_prev(deg + 1, 0.0), tk(deg + 1, 0.0), next(deg + 1);
-    for (int j = 0; j < nodes; ++j) {
-        const double th = M_PI * (j + 0.5) / nodes, t = cos(th);
-        const double q = split_q(0.5 * (t + 1.0) * uc);
-        for (int k = 0; k <= deg; ++k) cheb[k] += q * cos(k * th);
-    }
-    for (int k = 0; k <= deg; ++k) cheb[k] *= (k == 0 ? 1.0 : 2.0) / nodes;
-    // Chebyshev series -> monomials: T_0 = 1, T_1 = t, T_{k+1} = 2 t T_k - T_{k-1}
-    for (int i = 0; i <= deg; ++i) mono[i] = 0.0;
-    tk_prev[0] = 1.0;
-    mono[0] += cheb[0];
-    if (deg >= 1) {
-        tk[1] = 1.0;
-        for (int i = 0; i <= deg; ++i) mono[i] += cheb[1] * tk[i];
-    }
-    for (int k = 2; k <= deg; ++k) {
-        for (int i = 0; i <= deg; ++i) next[i] = -tk_prev[i] + (i > 0 ? 2.0 * tk[i - 1] : 0.0);
-        for (int i = 0; i <= deg; ++i) {
-            mono[i] += cheb[k] * next[i];
-            tk_prev[i] = tk[i];
-            tk[i] = next[i];
-        }
-    }
-}
-
-// FP32 coefficients (degree P3M_SPLIT_DEG) into out[0..10], tau's scale into out[11].
-void fit_split_poly(double cutoff_in_rs, double r_s, float out[12])
-{
-    double mono[P3M_SPLIT_DEG + 1];
-    fit_split_mono(cutoff_in_rs, P3M_SPLIT_DEG, 40, mono);
-    const double uc = cutoff_in_rs * cutoff_in_rs, inv_rs3 = 1.0 / (r_s * r_s * r_s);
-    for (int i = 0; i <= P3M_SPLIT_DEG; ++i) out[i] = (float)(mono[i] * inv_rs3);
-    for (int i = P3M_SPLIT_DEG + 1; i < 11; ++i) out[i] = 0.0f;
-    out[11] = (float)(2.0 / (uc * r_s * r_s));
 }
 
 // g on kSplitTab64 equal intervals of r in [0, r_c]: row k holds the coefficients of a degree-7
@@ -285,6 +240,9 @@ PairFactor fit_pair_factor(double cutoff_in_rs, const P3MGeom &g)
     // (accelerations scale with length^-2; lambda's FP32 rounding is the unit that the kernel uses)
     const double len = ldexp(g.cs, -kFixBits) / (double)p.lambda;
     p.scale = g.gm / (len * len);
+    p.grad[0] = (float)(0.25 / kappa);
+    p.grad[1] = (float)(-0.28209479177387814347 / (rho * rho * rho));
+    p.grad[2] = -3.0f;
     p.additive = additive ? 1 : 0;
     return p;
 }
@@ -320,7 +278,7 @@ void release(p3m_ctx *c)
                     c->tab_one,   c->ps_acc,   c->fac_table,    c->step_idx, c->cur_fac,
                     c->tab_origin,
                     c->adj_u,     c->adj_vfx,  c->adj_vs,       c->adj_out,  c->kself,
-                    c->li,        c->relx,     c->relq,     c->sort_status,  c->sort_hist,
+                    c->li,        c->relq,     c->sort_status,  c->sort_hist,
                     c->rho_fix,   c->fix_exp,  c->ps_part,     c->sort_probe, c->split_tab};
     for (void *p : bufs)
         if (p) cudaFree(p);
@@ -734,7 +692,6 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
             {(void **)&c->pid, 4 * N},        {(void **)&c->pid_alt, 4 * N},
             {(void **)&c->rel, 4 * real * N}, {(void **)&c->keys, 4 * N},
             {(void **)&c->block_box, 32 * ((N + 31) / 32)},
-            {(void **)&c->relx, opt.precision == P3M_PREC_MIXED ? 384 * ((N + 31) / 32) : 16},
             {(void **)&c->relq, 384 * ((N + 31) / 32)},
             {(void **)&c->keys_alt, 4 * N},   {(void **)&c->vals, 4 * N},
             {(void **)&c->vals_alt, 4 * N},   {(void **)&c->digit_counts, 4 * 256 * (size_t)c->n_tiles},
@@ -801,7 +758,6 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
             tg[i] = t;
         }
         c->green_const = -4.0 * M_PI * (g.gm / (h * h * h)) / ((double)M3);
-        fit_split_poly(cutoff_in_rs, g.r_s, c->gpoly);
         c->pair_factor = fit_pair_factor(cutoff_in_rs, g);
         if (c->precision == P3M_PREC_MIXED) {
             std::vector<float> f(M);

@@ -7,12 +7,6 @@
 
 #include "p3m.h"
 
-// Degree of the fitted FP32 split factor Q (Chebyshev fit on [0, r_c]).  Its largest error in g
-// is 5.8e-6 (near r_c, where g = 0.0175).  Against the FP64 oracle the FP32 short-range force
-// then differs by 7.50e-6 relative RMS on the 32^3 Zel'dovich state at a = 0.02 (7.31e-6 at
-// degree 10, 1.8e-5 at degree 7: the FP32 rounding of nearly cancelling pair sums dominates)
-// and by 1.7e-6 on a clustered state.
-#define P3M_SPLIT_DEG 8
 // The FP64 pair kernel's table of g (fit_split_table): intervals of [0, r_c], and doubles per row
 // (8 coefficients, the interval's centre, one of padding against bank conflicts).
 constexpr int kSplitTab64 = 64, kSplitRow64 = 10;
@@ -34,6 +28,8 @@ struct PairFactor {
     float lambda;        // scaled lengths per fixed-point unit
     float cell, length;  // side of a chaining cell; one scaled length
     double scale;        // accelerations = scale * sum f d
+    float grad[3];       // general form of f'(r)/r: exponent of exp(-r^2/(4 r_s^2)) over t's,
+                         // -1/(2 sqrt(pi)) in scaled lengths, and -3
     int additive;
 };
 
@@ -90,7 +86,6 @@ struct p3m_ctx {
     uint32_t *pid_alt;
     void *rel;  // float4 (mixed) or double4_16a (fp64): position relative to its cell origin
     float4 *block_box;  // per 32-slot block of the sorted order: lo, hi (FP32, absolute)
-    float *relx;        // FP32 mode: rel as block-SoA, per 32-slot block x[32] y[32] z[32]
     uint32_t *relq;     // fixed-point coordinates (kFixBits), per 32-slot block x[32] y[32] z[32]
     int tile_blocks;    // FP32 pair kernel: its list is evaluated every 32 tile_blocks entries (3 or 5)
 
@@ -130,9 +125,7 @@ struct p3m_ctx {
     unsigned long long *rho_fix;
     int *fix_exp;  // scale exponent of the vector deposit (set on the device)
     double green_const;
-    float gpoly[12];  // FP32 split factor: g = 1 + r^3 Q(tau), Q = sum gpoly[k] tau^k
-                      // (k <= P3M_SPLIT_DEG), tau = r^2 gpoly[11] - 1
-    PairFactor pair_factor;  // of the FP32 force kernel
+    PairFactor pair_factor;  // of the FP32 pair kernels
     double *split_tab;  // FP64 mode: the table of g (kSplitTab64 rows)
     cufftHandle plan_r2c, plan_c2r, plan_c2r_one;  // R2C, batched 3 x C2R, single C2R
     bool plans_made;
@@ -222,49 +215,6 @@ struct PairArgs {
     PairFactor fac;
     float rcull2, pad;
 };
-
-// A neighbour cell of a pair work item, for the FP32 pair kernels: the shift between the two
-// cells' origins (periodic image included) as an FP32 value plus the FP32 residual of the FP64
-// shift, the periodic image alone, and the neighbour's range of sorted slots.
-struct NeighbourF {
-    uint32_t start, end;
-    float sx, sy, sz, rx, ry, rz;
-    float imx, imy, imz, pad;
-};
-
-// Neighbour nb (0..26, offsets (nb%3-1, nb/3%3-1, nb/9-1)) of cell (cx, cy, cz); an empty
-// neighbour gets start = end = 0.
-__device__ __forceinline__ NeighbourF make_neighbour(const P3MGeom &g, const uint32_t *cell_start,
-                                                     int cx, int cy, int cz, int nb)
-{
-    const int nc = g.n_c;
-    const int ux = cx + nb % 3 - 1, uy = cy + (nb / 3) % 3 - 1, uz = cz + nb / 9 - 1;
-    const int wx = (ux + nc) % nc, wy = (uy + nc) % nc, wz = (uz + nc) % nc;
-    const uint32_t q = ((uint32_t)wz * nc + wy) * nc + wx;
-    NeighbourF r;
-    r.start = cell_start[q];
-    r.end = cell_start[q + 1];
-    if (!p3m_in_bounds(r.start <= r.end && r.end <= (uint32_t)g.n, g.flags)) r.end = r.start;
-    if (r.start == r.end) r.start = r.end = 0;
-    const double L = g.box, cs = g.cs;
-    const double imx = ux < 0 ? -L : (ux >= nc ? L : 0.0);
-    const double imy = uy < 0 ? -L : (uy >= nc ? L : 0.0);
-    const double imz = uz < 0 ? -L : (uz >= nc ? L : 0.0);
-    const double sx = ((double)wx * cs + imx) - (double)cx * cs;
-    const double sy = ((double)wy * cs + imy) - (double)cy * cs;
-    const double sz = ((double)wz * cs + imz) - (double)cz * cs;
-    r.sx = (float)sx;
-    r.sy = (float)sy;
-    r.sz = (float)sz;
-    r.rx = (float)(sx - (double)r.sx);
-    r.ry = (float)(sy - (double)r.sy);
-    r.rz = (float)(sz - (double)r.sz);
-    r.imx = (float)imx;
-    r.imy = (float)imy;
-    r.imz = (float)imz;
-    r.pad = 0.0f;
-    return r;
-}
 
 #define P3M_FLAG_NONFINITE 2u
 

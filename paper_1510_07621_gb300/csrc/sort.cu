@@ -480,8 +480,7 @@ __global__ void __launch_bounds__(256, 6) k_permute(const uint32_t *__restrict__
                           const double *__restrict__ mom, const uint32_t *__restrict__ pid,
                           double *__restrict__ pos_out, double *__restrict__ mom_out,
                           uint32_t *__restrict__ pid_out, R4 *__restrict__ rel,
-                          float4 *__restrict__ block_box, float *__restrict__ relx,
-                          uint32_t *__restrict__ relq, double fix_scale,
+                          float4 *__restrict__ block_box, uint32_t *__restrict__ relq, double fix_scale,
                           const double *__restrict__ origin)
 {
     // one warp per 32-slot block of the sorted order; the warp also writes the block's
@@ -513,12 +512,6 @@ __global__ void __launch_bounds__(256, 6) k_permute(const uint32_t *__restrict__
                            cz = cell / (g.n_c * g.n_c);
             rv = rel_coords<R4>(x, y, z, cx, cy, cz, origin);
             rel[k] = rv;
-        }
-        if (relx) {  // block-SoA copy of the relative coordinates (zero past the end)
-            float *dst = relx + blk * 96;
-            dst[lane] = (float)rv.x;
-            dst[32 + lane] = (float)rv.y;
-            dst[64 + lane] = (float)rv.z;
         }
         {  // fixed point: 1.5 * 2^52 rounds x * scale to an integer in the low word (modulo 2^32)
             uint32_t *fix = relq + blk * 96;
@@ -738,14 +731,14 @@ cudaError_t launch_permute_and_cells(p3m_ctx *c)
     if (c->precision == P3M_PREC_MIXED)
         k_permute<float4><<<gb, 256, 0, c->stream>>>(c->vals, c->keys, c->g, c->pos, c->mom,
                                                      c->pid, c->pos_alt, c->mom_alt, c->pid_alt,
-                                                     (float4 *)c->rel, c->block_box, c->relx, c->relq,
+                                                     (float4 *)c->rel, c->block_box, c->relq,
                                                      fix_scale,
                                                      c->tab_origin);
     else
         k_permute<double4_16a><<<gb, 256, 0, c->stream>>>(c->vals, c->keys, c->g, c->pos, c->mom,
                                                       c->pid, c->pos_alt, c->mom_alt,
                                                       c->pid_alt, (double4_16a *)c->rel, c->block_box,
-                                                      nullptr, c->relq, fix_scale, c->tab_origin);
+                                                      c->relq, fix_scale, c->tab_origin);
     double *t = c->pos;
     c->pos = c->pos_alt;
     c->pos_alt = t;

@@ -9,7 +9,10 @@ lies within 1e-6 of the cutoff.
 
 FP64: groups of 8 particles with one more or one less, more candidate blocks than one round of masks
 holds, and a table of the split factor that covers a short or a long range.  Bars: 1e-12 relative RMS
-(the FP64 bar) and the same number of pairs."""
+(the FP64 bar) and the same number of pairs.
+
+FP32 force VJP: the same lists with v, both forms of the factor's derivative, coincident particles
+(which have w but no force).  Bar: 2e-5 relative RMS of the oracle, the FP32 bar of the force VJP."""
 
 import math
 
@@ -87,3 +90,29 @@ def test_pair_masks_fp64(kind, n, mesh, cutoff, softening):
         got = sim.diagnostics()["pairs"]
     assert math.sqrt(float(np.sum((sr - ref) ** 2))) <= 1e-12 * math.sqrt(float(np.sum(ref ** 2)))
     assert got == pairs
+
+
+@pytest.mark.parametrize("kind,n,mesh,cutoff,softening", [
+    ("cell", 30, 20, 4.5, 0.02), ("cell", 34, 32, 4.5, 0.5), ("cell", 700, 20, 4.5, 0.02),
+    ("twins", 700, 26, 4.5, 0.02), ("twins", 700, 24, 4.5, 0.5), ("uniform", 1000, 24, 1.5, 0.02),
+    ("uniform", 1000, 48, 6.0, 1.0),
+])
+def test_force_vjp_lists(kind, n, mesh, cutoff, softening):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1510_07621_gb300 import P3M, build
+    build.build()
+    box = 50.0
+    x = _set("uniform" if kind == "twins" else kind, n, box, 3000 + n + mesh)
+    if kind == "twins":
+        x[:, 1::7] = x[:, ::7]
+    v = S.gaussian(17, 3 * n).reshape(3, n)
+    p = O.Params(box, n, mesh, 1.25, cutoff, softening)
+    ref = O.sr_vjp(O.wrap(x, box), v, p)
+    with P3M(box, n, mesh, 1.25, cutoff, softening=softening) as sim:
+        sim.set_particles(x, np.zeros_like(x), a=1.0)
+        got = sim.force_vjp(v)
+    mesh_part = O.pm_vjp(O.wrap(x, box), v, p)
+    err = got - mesh_part - ref
+    assert math.sqrt(float(np.sum(err ** 2))) <= 2e-5 * math.sqrt(float(np.sum((ref + mesh_part) ** 2)))
