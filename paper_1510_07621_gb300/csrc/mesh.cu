@@ -569,15 +569,39 @@ __global__ void __launch_bounds__(256)
 // delta_k = rho_k / N; every mode (ix, iy, iz) stands for itself and, for 0 < iz < M/2, for its
 // conjugate partner (weight 2).  Shell b = round(|n|) - 1 accumulates w |delta_k|^2 / W^2,
 // w |k| and w; with radius > 0 the top-hat sum w |delta_k|^2 / W^2 W_TH(|k| R)^2 goes to
-// row entry 3 n_bins.  The additions happen in an order fixed by the launch shape alone: the
-// lanes of a warp that hold modes of one shell are summed in lane order by the lowest of them,
-// which adds the sums to its warp's private shared-memory row; the block adds its warps' rows in
-// warp order into its row of part[], and k_powspec_final adds the blocks' rows in block order.
-// So every run gives the same bits.
+// row entry 3 n_bins.
+// The up to 8 rows (+-a, +-b), (+-b, +-a) of the spectrum have the same |n|, shell and window at
+// the same iz.  A warp takes one such set (a >= b) and 32 iz at a time: lane iz sums |rho_k|^2 over
+// the rows, applies window and weight once, and the lanes of one shell (|n| grows with iz, so they
+// are neighbours) are summed by a segmented scan whose last lane adds the sums to its warp's private
+// shared-memory row.  |n| and W_TH^2 depend on |n|^2 only and come from a table (k_powspec_table).
+// FP64 arithmetic bounded the former kernel (a square root, a sine and a cosine per mode, and up to
+// 32 rounds of shuffles and additions per 32 modes): 256^3 mesh with the top-hat sum 1.60 -> 0.145
+// ms.  It is still what bounds it: about 50 FP64 operations per 256 modes (0.13 ms at the pipe's rate,
+// a fifth of it for the lone iz = M/2); 8 warps per block are no faster.
+// The additions happen in an order fixed by the launch shape alone: the block adds its warps' rows
+// in warp order into its row of part[], and k_powspec_final the blocks' rows in a fixed order.  So
+// every run gives the same bits.
+
+// tab[s] = (sqrt(s), W_TH(sqrt(s) kf R)^2 or 0 when R = 0), 0 <= s < count
+__global__ void k_powspec_table(int count, double kf, double radius, double2 *__restrict__ tab)
+{
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < count; s += gridDim.x * blockDim.x) {
+        const double nk = sqrt((double)s);
+        double wt = 0.0;
+        if (radius > 0.0) {
+            const double x = nk * kf * radius;
+            wt = x < 1e-3 ? 1.0 - x * x / 10.0 : 3.0 * (sin(x) - x * cos(x)) / (x * x * x);
+        }
+        tab[s] = make_double2(nk, wt * wt);
+    }
+}
+
 template <typename C2>
 __global__ void __launch_bounds__(128)
-    k_powspec(const C2 *__restrict__ rk, int M, const double *__restrict__ inv_w2, double kf,
-              double inv_n2, double radius, int n_bins, double *__restrict__ part)
+    k_powspec(const C2 *__restrict__ rk, int M, const double *__restrict__ inv_w2,
+              const double2 *__restrict__ tab, double kf, double inv_n2, int n_bins,
+              double *__restrict__ part)
 {
     extern __shared__ double sacc[];  // (blockDim / 32) rows of 3 n_bins + 1
     const int nacc = 3 * n_bins + 1;
@@ -585,56 +609,74 @@ __global__ void __launch_bounds__(128)
     double *mine = sacc + (size_t)warp * nacc;
     for (int t = lane; t < nacc; t += 32) mine[t] = 0.0;
     __syncwarp();
-    const int nz = M / 2 + 1;
-    const size_t total = (size_t)M * M * nz;
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t base = ((size_t)blockIdx.x * nw + warp) * 32; base < total; base += stride) {
-        const size_t idx = base + lane;
-        int b = -1;
-        double v0 = 0.0, v1 = 0.0, v2 = 0.0, vt = 0.0;
-        if (idx < total && idx != 0) {
-            const int iz = (int)(idx % nz);
-            const size_t t = idx / nz;
-            const int iy = (int)(t % M), ix = (int)(t / M);
-            const int sx = ix <= M / 2 ? ix : ix - M, sy = iy <= M / 2 ? iy : iy - M;
-            const double w = (iz == 0 || iz == M / 2) ? 1.0 : 2.0;
-            const double nk = sqrt((double)sx * sx + (double)sy * sy + (double)iz * iz);
-            const C2 r = rk[idx];
-            const double p = ((double)r.x * r.x + (double)r.y * r.y) * inv_n2 * inv_w2[ix] *
-                             inv_w2[iy] * inv_w2[iz];
-            b = (int)floor(nk + 0.5) - 1;
-            if (b >= n_bins) b = -1;
-            v0 = w * p;
-            v1 = w * nk * kf;
-            v2 = w;
-            if (radius > 0.0) {
-                const double x = nk * kf * radius;
-                const double wt = x < 1e-3 ? 1.0 - x * x / 10.0 : 3.0 * (sin(x) - x * cos(x)) / (x * x * x);
-                vt = w * p * wt * wt;
-            }
-        }
-        const unsigned grp = __match_any_sync(0xffffffffu, b);
-        if (b >= 0) {
-            double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-            for (unsigned m = grp; m; m &= m - 1u) {
-                const int src = __ffs(m) - 1;
-                s0 += __shfl_sync(grp, v0, src);
-                s1 += __shfl_sync(grp, v1, src);
-                s2 += __shfl_sync(grp, v2, src);
-            }
-            if (lane == __ffs(grp) - 1) {
-                mine[3 * b] += s0;
-                mine[3 * b + 1] += s1;
-                mine[3 * b + 2] += s2;
-            }
-        }
-        if (radius > 0.0) {
+    const int H = M / 2, nz = H + 1;
+    const long long sets = (long long)(H + 1) * (H + 2) / 2;  // pairs 0 <= b <= a <= M/2
+    double vt = 0.0;
+    for (long long set = (long long)blockIdx.x * nw + warp; set < sets; set += (long long)gridDim.x * nw) {
+        // set = a (a + 1) / 2 + b
+        int a = (int)((sqrt(8.0f * (float)set + 1.0f) - 1.0f) * 0.5f);
+        while ((long long)a * (a + 1) / 2 > set) --a;
+        while ((long long)(a + 1) * (a + 2) / 2 <= set) ++a;
+        const int b = (int)(set - (long long)a * (a + 1) / 2);
+        // the rows: bits 0 and 1 of r negate the components, bit 2 exchanges them
+        const C2 *row[8];
+        bool use[8];
+        int rows = 0;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) vt += __shfl_xor_sync(0xffffffffu, vt, o);
-            if (lane == 0) mine[3 * n_bins] += vt;
+        for (int r = 0; r < 8; ++r) {
+            const int u = r & 4 ? b : a, v = r & 4 ? a : b;
+            use[r] = !((r & 1) && (u == 0 || u == H)) && !((r & 2) && (v == 0 || v == H)) && !((r & 4) && a == b);
+            row[r] = rk + ((size_t)(r & 1 ? M - u : u) * M + (r & 2 ? M - v : v)) * nz;
+            rows += use[r];
         }
-        __syncwarp();
+        const double wab = inv_n2 * inv_w2[a] * inv_w2[b];
+        for (int z0 = 0; z0 < nz; z0 += 32) {
+            const int iz = z0 + lane;
+            const bool in = iz < nz;
+            double p = 0.0;
+            if (in) {
+                C2 q[8];
+#pragma unroll
+                for (int r = 0; r < 8; ++r)
+                    if (use[r]) q[r] = row[r][iz];
+#pragma unroll
+                for (int r = 0; r < 8; ++r)
+                    if (use[r]) p = fma((double)q[r].x, (double)q[r].x, fma((double)q[r].y, (double)q[r].y, p));
+            }
+            const int s = a * a + b * b + iz * iz;  // |n|^2 (< 2^22)
+            // round(sqrt(s)): the m with m^2 - m < s <= m^2 + m
+            int m = (int)(sqrtf((float)s) + 0.5f);
+            m -= m * m - m >= s && m > 0;
+            m += m * m + m < s;
+            const int bin = in && s > 0 && m <= n_bins ? m - 1 : -1;
+            const double w = iz == 0 || iz == H ? 1.0 : 2.0;
+            const double2 e = tab[in ? s : 0];
+            double v0 = s > 0 && in ? w * p * (wab * inv_w2[in ? iz : 0]) : 0.0;
+            vt = fma(v0, e.y, vt);
+            double v1 = w * rows * e.x * kf;
+            int cnt = (iz == 0 || iz == H ? 1 : 2) * rows;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int bo = __shfl_up_sync(0xffffffffu, bin, o), co = __shfl_up_sync(0xffffffffu, cnt, o);
+                const double x0 = __shfl_up_sync(0xffffffffu, v0, o), x1 = __shfl_up_sync(0xffffffffu, v1, o);
+                if (lane >= o && bo == bin) {
+                    v0 += x0;
+                    v1 += x1;
+                    cnt += co;
+                }
+            }
+            const int next = __shfl_down_sync(0xffffffffu, bin, 1);
+            if (bin >= 0 && (lane == 31 || next != bin)) {
+                mine[3 * bin] += v0;
+                mine[3 * bin + 1] += v1;
+                mine[3 * bin + 2] += (double)cnt;
+            }
+            __syncwarp();
+        }
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) vt += __shfl_xor_sync(0xffffffffu, vt, o);
+    if (lane == 0) mine[3 * n_bins] = vt;
     __syncthreads();
     for (int t = threadIdx.x; t < nacc; t += blockDim.x) {
         double s = 0.0;
@@ -643,14 +685,18 @@ __global__ void __launch_bounds__(128)
     }
 }
 
+// One warp per sum: lane l adds the rows l, l + 32, ..., then the lanes are added pairwise.
 __global__ void k_powspec_final(const double *__restrict__ part, int blocks, int nacc,
                                 double *__restrict__ acc)
 {
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nacc; t += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int b = 0; b < blocks; ++b) s += part[(size_t)b * nacc + t];
-        acc[t] = s;
-    }
+    const int lane = threadIdx.x & 31;
+    const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (t >= nacc) return;
+    double s = 0.0;
+    for (int b = lane; b < blocks; b += 32) s += part[(size_t)b * nacc + t];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) acc[t] = s;
 }
 
 inline int grid_for(size_t n, int threads, int num_sms)
@@ -728,24 +774,27 @@ cudaError_t launch_powspec(p3m_ctx *c, const double *inv_w2, double radius, int 
     const size_t smem = sizeof(double) * (size_t)nacc * (threads / 32);
     const double kf = 2.0 * M_PI / c->g.box;
     const double inv_n2 = 1.0 / ((double)c->g.n * (double)c->g.n);
-    c->launches += 2;
+    c->launches += 3;
     cudaError_t e = cudaSuccess;
+    double2 *tab = (double2 *)c->adj_u;  // scratch of at least 3 M^3 floats; |n|^2 <= 3 M^2 / 4
+    const int count = 3 * (M / 2) * (M / 2) + 1;
+    k_powspec_table<<<grid_for((size_t)count, 128, c->num_sms), 128, 0, c->stream>>>(count, kf, radius, tab);
     if (c->precision == P3M_PREC_MIXED) {
         if (smem > 48 * 1024)
             e = cudaFuncSetAttribute(k_powspec<cufftComplex>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem);
         if (e != cudaSuccess) return e;
         k_powspec<cufftComplex><<<c->ps_blocks, threads, smem, c->stream>>>(
-            (const cufftComplex *)c->rho_k, M, inv_w2, kf, inv_n2, radius, n_bins, c->ps_part);
+            (const cufftComplex *)c->rho_k, M, inv_w2, tab, kf, inv_n2, n_bins, c->ps_part);
     } else {
         if (smem > 48 * 1024)
             e = cudaFuncSetAttribute(k_powspec<cufftDoubleComplex>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         k_powspec<cufftDoubleComplex><<<c->ps_blocks, threads, smem, c->stream>>>(
-            (const cufftDoubleComplex *)c->rho_k, M, inv_w2, kf, inv_n2, radius, n_bins, c->ps_part);
+            (const cufftDoubleComplex *)c->rho_k, M, inv_w2, tab, kf, inv_n2, n_bins, c->ps_part);
     }
-    k_powspec_final<<<(nacc + 255) / 256, 256, 0, c->stream>>>(c->ps_part, c->ps_blocks, nacc, acc);
+    k_powspec_final<<<(nacc + 3) / 4, 128, 0, c->stream>>>(c->ps_part, c->ps_blocks, nacc, acc);
     return cudaGetLastError();
 }
 
