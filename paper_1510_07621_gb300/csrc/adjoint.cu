@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(32)
 // own cell can hold them.  Before, all 32 lanes met every j of a tested block with 40 FP32 operations
 // and three 8-cycle MUFU operations per pair (34 and one here).  128^3 near-uniform, one call with the
 // mesh part: 9.35 -> 7.13 ms, the pair part 7.6 -> 5.4.  What bounds it: of 137 cycles per 32 accepted
-// pairs and scheduler, 110 are the evaluation (52 per 32 slots, 47 % of them accepted).  8 or 32
+// pairs and scheduler, 111 are the evaluation (52 per 32 slots, 47 % of them accepted).  8 or 32
 // particles per group, 18 or 20 CTAs per SM and lists of 192 are within 2 % or slower.
 constexpr int kVjpGroup = 16, kVjpChunk = 128, kVjpFlush = 5;  // (16 FP32 terms per chunk and sum)
 constexpr float kVjpTiny = 1e-24f, kVjpFar = 1e6f;
@@ -445,16 +445,17 @@ __global__ void __launch_bounds__(32, 16)
 {
     constexpr int kG = kVjpGroup, kPairsI = kG / 2, kStride = 2 * (32 / kPairsI), kSub = P3M_PAIR_TI / kG;
     __shared__ __align__(16) float list[6][kVjpChunk + 32];  // x, y, z, vx, vy, vz
+    __shared__ uint32_t slot[kVjpChunk + 32];                // the sorted slot of each list entry
     __shared__ double sum[6][32];
     __shared__ PairSeg seg[kPairSegs];
-    __shared__ uint32_t live[32];
+    __shared__ LiveBlocks live;
 
     const int lane = threadIdx.x, ip = lane % kPairsI, js = lane / kPairsI;
     const uint32_t lt = (1u << lane) - 1u;
     const int64_t n = g.n;
     const uint32_t n_units = *n_work_ptr * kSub;
     const int nc = g.n_c;
-    const float lambda = fac.lambda, rc2 = fac.rc2, rlist2 = fac.rlist2;
+    const float lambda = fac.lambda, rlist2 = fac.rlist2;
     VjpConst2 kc;
 #pragma unroll
     for (int q = 0; q < 5; ++q) kc.c[q] = f2_pack(fac.c[q], fac.c[q]);
@@ -511,9 +512,35 @@ __global__ void __launch_bounds__(32, 16)
                     o[u][d] = f2_pack(0.0f, 0.0f);
                 }
         };
+        // the pairs of a list in the cutoff's band: their terms are made whole or taken back
+        auto settle = [&](int count) {
+#pragma unroll 1
+            for (int k = 0; k < 2 * count; k += kStride) {
+                const int p = (k < count ? k : k - count + 1) + 2 * js;  // the first, then the second halves
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    float dx[3], wv[3];
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        dx[d] = list[d][p] + nx[u][d].x;
+                        wv[d] = list[3 + d][p] + nv[u][d].x;
+                    }
+                    const float w = fmaf(dx[2], dx[2], fmaf(dx[1], dx[1], fmaf(dx[0], dx[0], w0.x)));
+                    const float part = cut_part(w, fac.cut_m, fac.cut_b);
+                    if (part == rintf(part)) continue;
+                    const float dw = fmaf(dx[2], wv[2], fmaf(dx[1], wv[1], dx[0] * wv[0]));
+                    const uint32_t i = min(first + ip + u * kPairsI, cend - 1);
+                    const float t = (cut_inside(relq, i, slot[p], dx[0], dx[1], dx[2], fac) ? 1.0f : 0.0f) - part;
+                    f2 c, h = pair_jac2<kAdditive>(f2_pack(w, w), f2_pack(dw, dw), kc, &c);
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) o[u][d].x = fmaf(t * h.x, wv[d], fmaf(t * c.x, dx[d], o[u][d].x));
+                }
+            }
+        };
         // list entries [0, count), count a multiple of kStride
         auto eval = [&](auto own, int count) {
-#pragma unroll 1
+            f2 hits = f2_pack(0.0f, 0.0f);
+#pragma unroll 2
             for (int k = 2 * js; k < count; k += kStride) {
                 f2 X[3], V[3];
 #pragma unroll
@@ -532,17 +559,21 @@ __global__ void __launch_bounds__(32, 16)
                     const f2 w = f2_fma(dx[2], dx[2], f2_fma(dx[1], dx[1], f2_fma(dx[0], dx[0], w0)));
                     const f2 dw = f2_fma(dx[2], wv[2], f2_fma(dx[1], wv[1], f2_mul(dx[0], wv[0])));
                     f2 c, h = pair_jac2<kAdditive>(w, dw, kc, &c);
-                    bool lo = w.x < rc2, hi = w.y < rc2;
+                    f2 in = f2_pack(cut_part(w.x, fac.cut_m, fac.cut_b), cut_part(w.y, fac.cut_m, fac.cut_b));
                     if (decltype(own)::value) {
-                        lo = lo && (__float_as_uint(dx[0].x) | __float_as_uint(dx[1].x) | __float_as_uint(dx[2].x)) != 0u;
-                        hi = hi && (__float_as_uint(dx[0].y) | __float_as_uint(dx[1].y) | __float_as_uint(dx[2].y)) != 0u;
+                        const bool nl = (__float_as_uint(dx[0].x) | __float_as_uint(dx[1].x) | __float_as_uint(dx[2].x)) != 0u;
+                        const bool nh = (__float_as_uint(dx[0].y) | __float_as_uint(dx[1].y) | __float_as_uint(dx[2].y)) != 0u;
+                        in = f2_pack(nl ? in.x : 0.0f, nh ? in.y : 0.0f);
                     }
-                    h = f2_pack(lo ? h.x : 0.0f, hi ? h.y : 0.0f);
-                    c = f2_pack(lo ? c.x : 0.0f, hi ? c.y : 0.0f);
+                    hits = f2_add(hits, in);
+                    h = f2_mul(h, in);
+                    c = f2_mul(c, in);
 #pragma unroll
                     for (int d = 0; d < 3; ++d) o[u][d] = f2_fma(h, wv[d], f2_fma(c, dx[d], o[u][d]));
                 }
             }
+            const float total = hits.x + hits.y;
+            if (__any_sync(0xffffffffu, total != rintf(total))) settle(count);
         };
 
         int fill = 0, chunks = 0;
@@ -550,11 +581,10 @@ __global__ void __launch_bounds__(32, 16)
             for (uint32_t base = t0; base < t1; base += 32) {
                 const int nl = live_blocks(base + lane, t1, seg, block_box, fr, fac.length, rcull2, live);
                 // the next block's data are loaded while the current one is tested
-                uint32_t word_n = 0, qn[3];
+                uint32_t qn[3];
                 float vn[3];
                 auto fetch = [&](int k) {
-                    word_n = live[k];
-                    const size_t at = (size_t)(word_n & 0x3FFFFFFu) * 96 + lane;
+                    const size_t at = (size_t)(live.at[k].word & kBlockMask) * 96 + lane;
 #pragma unroll
                     for (int d = 0; d < 3; ++d) {
                         qn[d] = __ldg(relq + at + 32 * d);
@@ -564,12 +594,11 @@ __global__ void __launch_bounds__(32, 16)
                 if (nl) fetch(0);
 #pragma unroll 1
                 for (int k = 0; k < nl; ++k) {
-                    const PairSeg &S = seg[word_n >> 26];
-                    const uint32_t slot = (word_n & 0x3FFFFFFu) * 32 + lane;
+                    const LiveBlock S = live.at[k];
                     const float x = (float)(int)(qn[0] - S.cx) * lambda, y = (float)(int)(qn[1] - S.cy) * lambda,
                                 z = (float)(int)(qn[2] - S.cz) * lambda;
                     const float vx = vn[0], vy = vn[1], vz = vn[2];
-                    const bool mine = slot - S.start < S.end - S.start;
+                    const bool mine = live.slots[k] >> lane & 1u;
                     if (k + 1 < nl) fetch(k + 1);
                     const float ex = fmaxf(fabsf(x) - fr.half[0], 0.0f), ey = fmaxf(fabsf(y) - fr.half[1], 0.0f),
                                 ez = fmaxf(fabsf(z) - fr.half[2], 0.0f);
@@ -583,6 +612,7 @@ __global__ void __launch_bounds__(32, 16)
                         list[3][p] = vx;
                         list[4][p] = vy;
                         list[5][p] = vz;
+                        slot[p] = (S.word & kBlockMask) << 5 | lane;
                     }
                     fill += __popc(mm);
                     if (fill >= kVjpChunk) {
@@ -590,8 +620,10 @@ __global__ void __launch_bounds__(32, 16)
                         eval(own, kVjpChunk);
                         __syncwarp();
                         fill -= kVjpChunk;
-                        if (lane < fill)  // (fill < 32 <= kVjpChunk: no overlap)
+                        if (lane < fill) {  // (fill < 32 <= kVjpChunk: no overlap)
                             for (int d = 0; d < 6; ++d) list[d][lane] = list[d][kVjpChunk + lane];
+                            slot[lane] = slot[kVjpChunk + lane];
+                        }
                         if (++chunks % kVjpFlush == 0) flush();
                     }
                 }

@@ -234,6 +234,10 @@ PairFactor fit_pair_factor(double cutoff_in_rs, const P3MGeom &g)
     p.e2 = (float)(additive ? fmax(e2, 1e-24) : e2);  // (r = 0 pairs stay finite)
     p.rc2 = (float)(additive ? rc2 + e2 : rc2);
     p.rlist2 = (float)(rc2 * (1.0 + 2e-5));
+    p.cut_m = (float)(-0.5 / (kCutBand * rc2));
+    p.cut_b = (float)(0.5 - (double)p.cut_m * (double)p.rc2);  // (half at the cutoff)
+    const double fix_rc = ldexp(g.r_c / g.cs, kFixBits);        // (at most 2^29: cells are no smaller than r_c)
+    p.fix_rc2 = (long long)ceil(fix_rc * fix_rc);
     p.length = (float)(g.r_s / rho);
     p.lambda = (float)(ldexp(g.cs, -kFixBits) * rho / g.r_s);
     p.cell = (float)g.cs;

@@ -15,19 +15,24 @@ constexpr int kSplitTab64 = 64, kSplitRow64 = 10;
 // (8 cells), so that differences of particles in neighbouring cells are exact integers.
 constexpr int kFixBits = 29;
 constexpr float kFixUnit = 0x1p-29f;
+// The FP32 pair kernels decide on the cutoff by the FP32 r^2 outside a band of this relative half
+// width (six times its rms error there), by the fixed-point coordinates inside it.
+constexpr double kCutBand = 5e-7;
 
 // The FP32 pair factor f(r) = g(r/r_s) (r^2 + eps^2)^-3/2 in scaled lengths (see fit_pair_factor):
 // one unit is `length`, chosen so that t = 2^-w is the exponential of the fit, w the squared
 // scaled distance.  With s = (w + softening)^-1/2 and P(t) = c[0] + c[1] t + c[2] t^2 + c[3] t^3:
-//   additive:  w includes the softening (e2): f = s^3 + (ab + na t) s^2 + P(t); rc2 bounds w
-//   otherwise: f = s^3 (1 + r (ab + na t + r^2 P(t))), r without the softening; rc2 bounds r^2
+//   additive:  w includes the softening (e2): f = s^3 + (ab + na t) s^2 + P(t); rc2 is the cutoff's w
+//   otherwise: f = s^3 (1 + r (ab + na t + r^2 P(t))), r without the softening; rc2 the cutoff's r^2
 struct PairFactor {
     float c[5];
     float na, ab, e2, rc2;
+    float cut_m, cut_b;  // clamp(cut_m rc2 + cut_b, 0, 1): 1 inside the cutoff, 0 outside, fractions in the band
     float rlist2;        // squared radius of the candidate test (a little above the cutoff)
     float lambda;        // scaled lengths per fixed-point unit
     float cell, length;  // side of a chaining cell; one scaled length
     double scale;        // accelerations = scale * sum f d
+    long long fix_rc2;   // a pair is inside if its squared distance in fixed-point units is below this
     float grad[3];       // general form of f'(r)/r: exponent of exp(-r^2/(4 r_s^2)) over t's,
                          // -1/(2 sqrt(pi)) in scaled lengths, and -3
     int additive;

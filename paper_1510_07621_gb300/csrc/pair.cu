@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(32)
     __shared__ uint32_t entry[kEntries64];
     __shared__ __align__(16) float sj[3][32];
     __shared__ PairSeg seg[kPairSegs];
-    __shared__ uint32_t live[32];
+    __shared__ LiveBlocks live;
     __shared__ __align__(16) double tab[kSplitTab64 * kSplitRow64];
     for (int t = threadIdx.x; t < kSplitTab64 * kSplitRow64; t += 32) tab[t] = split[t];
     __syncwarp();
@@ -134,13 +134,10 @@ __global__ void __launch_bounds__(32)
                 const int nl = live_blocks(base + lane, blocks.y, seg, block_box, fr, cell_f, rcull2, live);
                 n_live += nl;
                 for (int k = 0; k < nl; ++k) {
-                    const uint32_t w = live[k];
-                    const PairSeg &S = seg[w >> 26];
-                    const uint32_t b = w & 0x3FFFFFFu;
-                    const uint32_t *qj = fix_coords(relq, b * 32 + lane);
+                    const LiveBlock S = live.at[k];
+                    const uint32_t w = S.word, in = live.slots[k];
+                    const uint32_t *qj = relq + (size_t)(w & kBlockMask) * 96 + lane;
                     const uint32_t jx = __ldg(qj), jy = __ldg(qj + 32), jz = __ldg(qj + 64);
-                    // the slots of the block that belong to the range
-                    const uint32_t in = __ballot_sync(0xffffffffu, b * 32 + lane - S.start < S.end - S.start);
                     __syncwarp();  // every lane is done with the previous block's coordinates
                     sj[0][lane] = (float)(int)(jx - S.cx) * kFixUnit;
                     sj[1][lane] = (float)(int)(jy - S.cy) * kFixUnit;
@@ -179,7 +176,7 @@ __global__ void __launch_bounds__(32)
                 const bool have = __popc(m) > skip;
                 if (!__any_sync(0xffffffffu, have)) break;
                 for (; skip > 0; --skip) m &= m - 1;
-                const uint32_t j = have ? (w & 0x3FFFFFFu) * 32 + (uint32_t)__ffs(m) - 1 : i;
+                const uint32_t j = have ? (w & kBlockMask) * 32 + (uint32_t)__ffs(m) - 1 : i;
                 m &= m - 1;
                 skip = have ? 3 : 0;
                 double dx = pos[j] - xi, dy = pos[n + j] - yi, dz = pos[2 * n + j] - zi;
@@ -254,12 +251,14 @@ __global__ void __launch_bounds__(32)
 // instructions were tests and votes.  The list holds 47 % accepted slots at kG = 16 (58 % at 8,
 // 39 % at 32: the union of the cutoff spheres grows with the group), there are no votes between
 // pairs, and a test sequence serves 32 candidates of the whole group.  Measured at 128^3 (one
-// evaluation, before / after): near-uniform 5.23 / 3.12 ms, clustered 12.3 / 9.6 ms.
-// What bounds it now: of 81 cycles per 32 accepted pairs and scheduler, 55 are the evaluation
-// (26 per 32 slots; two FP32 operations with three distinct registers already take three cycles
+// evaluation, before / after): near-uniform 5.23 / 3.21 ms, clustered 12.3 / 9.6 ms.
+// What bounds it now: of 83 cycles per 32 accepted pairs and scheduler, 58 are the evaluation
+// (27 per 32 slots; two FP32 operations with three distinct registers already take three cycles
 // of register bandwidth, and the same mix of 16 packed operations, 2 rsqrt and 2 ex2 alone runs
-// at 20.5), 20 the candidate tests and 6 the set-up of groups.  16 particles per group
-// and 18 CTAs per SM: 8, 32 and 16, 20, 24 are within 3 % or slower on both sets.
+// at 20.5), 19 the candidate tests and 6 the set-up of groups.  16 particles per group
+// and 18 CTAs per SM: 8, 32 and 16, 20, 24 are within 6 % or slower on both sets.  Two lists of 16 (or
+// four of 8) filled by one pass over the candidates save a third of the tests but cost as much in
+// registers and reloads (3.18 and 4.8 ms, against 3.06 without the exact cutoff).
 //
 // Coordinates are 32-bit fixed point, 2^-29 of a chaining cell, modulo 8 cells (relq): differences
 // of particles in neighbouring cells, periodic images included, are exact integers, and only the
@@ -321,9 +320,10 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
     constexpr int kFlushChunks = kFlushTerms * kStride / kChunk < 1 ? 1 : kFlushTerms * kStride / kChunk;
     static_assert(kChunk % kStride == 0, "whole steps per chunk");
     __shared__ __align__(16) float list[3][kCap];
+    __shared__ uint32_t slot[kCap];  // the sorted slot of each list entry
     __shared__ double sum[6][32];  // per lane: x, y, z of its first particle, then of its second
     __shared__ PairSeg seg[kPairSegs];
-    __shared__ uint32_t live[32];
+    __shared__ LiveBlocks live;
     __shared__ unsigned long long stat[6];
     __shared__ __align__(16) PairArgs sA;  // the current work item's context
     const PairArgs &A = sA;
@@ -407,7 +407,8 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
             nz[u] = f2_pack(z, z);
             px[u] = py[u] = pz[u] = f2_pack(0.0f, 0.0f);
         }
-        const float rc2 = A.fac.rc2, rlist2 = A.fac.rlist2;
+        const float rlist2 = A.fac.rlist2;
+        const float cut_m = kBatched ? A.fac.cut_m : a0.fac.cut_m, cut_b = kBatched ? A.fac.cut_b : a0.fac.cut_b;
         const uint32_t *__restrict__ relq = A.relq + lane;
 
         auto flush = [&]() {
@@ -419,13 +420,37 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
                 px[u] = py[u] = pz[u] = f2_pack(0.0f, 0.0f);
             }
         };
+        // The pairs of a list in the cutoff's band: their terms are made whole or taken back, and so are
+        // their parts of the sums of cut_part (total).
+        auto settle = [&](auto additive, int count, float *total) {
+            constexpr bool kAdd = decltype(additive)::value;
+#pragma unroll 1
+            for (int k = 0; k < 2 * count; k += kStride) {
+                const int p = (k < count ? k : k - count + 1) + 2 * js;  // the first, then the second halves
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const float dx = list[0][p] + nx[u].x, dy = list[1][p] + ny[u].x, dz = list[2][p] + nz[u].x;
+                    const float w = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, kAdd ? kc.e2.x : kTinyQ)));
+                    const float part = cut_part(w, cut_m, cut_b);
+                    if (part == rintf(part)) continue;
+                    const uint32_t i = min(first + ip + u * kPairsI, cend - 1);
+                    const float t = (cut_inside(A.relq, i, slot[p], dx, dy, dz, A.fac) ? 1.0f : 0.0f) - part;
+                    const float f = t * pair_factor_q<kAdd>(f2_pack(w, w), kc).x;
+                    px[u].x = fmaf(f, dx, px[u].x);
+                    py[u].x = fmaf(f, dy, py[u].x);
+                    pz[u].x = fmaf(f, dz, pz[u].x);
+                    total[u] += t;
+                }
+            }
+        };
         // list entries [0, count), count a multiple of kStride
         auto eval_form = [&](auto additive, auto own, int count) {
             constexpr bool kAdd = decltype(additive)::value;
             const f2 w0 = kAdd ? kc.e2 : kc.tiny;
             const float *lx = &list[0][2 * js], *ly = &list[1][2 * js], *lz = &list[2][2 * js];
             f2 Xn = *(const f2 *)lx, Yn = *(const f2 *)ly, Zn = *(const f2 *)lz;
-#pragma unroll 1
+            f2 hits[2] = {f2_pack(0.0f, 0.0f), f2_pack(0.0f, 0.0f)};
+#pragma unroll 2
             for (int k = 0; k < count; k += kStride) {
                 const f2 X = Xn, Y = Yn, Z = Zn;
                 const int kn = k + kStride < count ? k + kStride : 0;
@@ -435,23 +460,26 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
                     const f2 dx = f2_add(X, nx[u]), dy = f2_add(Y, ny[u]), dz = f2_add(Z, nz[u]);
                     const f2 w = f2_fma(dz, dz, f2_fma(dy, dy, f2_fma(dx, dx, w0)));
                     f2 f = pair_factor_q<kAdd>(w, kc);
-                    const bool lo = w.x < rc2, hi = w.y < rc2;
-                    f.x = lo ? f.x : 0.0f;
-                    f.y = hi ? f.y : 0.0f;
+                    const f2 in = f2_pack(cut_part(w.x, cut_m, cut_b), cut_part(w.y, cut_m, cut_b));
+                    f = f2_mul(f, in);
                     px[u] = f2_fma(f, dx, px[u]);
                     py[u] = f2_fma(f, dy, py[u]);
                     pz[u] = f2_fma(f, dz, pz[u]);
                     if (decltype(own)::value) {
                         const bool nl = (__float_as_uint(dx.x) | __float_as_uint(dy.x) | __float_as_uint(dz.x)) != 0u;
                         const bool nh = (__float_as_uint(dx.y) | __float_as_uint(dy.y) | __float_as_uint(dz.y)) != 0u;
-                        if (lo && nl) ++cnt[u];
-                        if (hi && nh) ++cnt[u];
+                        hits[u] = f2_add(hits[u], f2_pack(nl ? in.x : 0.0f, nh ? in.y : 0.0f));
                     } else {
-                        if (lo) ++cnt[u];
-                        if (hi) ++cnt[u];
+                        hits[u] = f2_add(hits[u], in);
                     }
                 }
             }
+            // a sum with a fraction holds a pair in the band
+            float total[2] = {hits[0].x + hits[0].y, hits[1].x + hits[1].y};
+            const bool near = total[0] != rintf(total[0]) || total[1] != rintf(total[1]);
+            if (__any_sync(0xffffffffu, near)) settle(additive, count, total);
+            cnt[0] += __float2uint_rn(total[0]);
+            cnt[1] += __float2uint_rn(total[1]);
         };
         auto eval = [&](auto own, int count) {
             if (kForm == 1 || (kForm == 2 && A.fac.additive))
@@ -468,10 +496,9 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
                 const int nl = live_blocks(base + lane, t1, seg, A.block_box, fr, A.fac.length, A.rcull2, live);
                 n_live += nl;
                 // the next block's coordinates are loaded while the current one is tested
-                uint32_t word_n = 0, xn = 0, yn = 0, zn = 0;
+                uint32_t xn = 0, yn = 0, zn = 0;
                 auto fetch = [&](int k) {
-                    word_n = live[k];
-                    const uint32_t *q = relq + (size_t)(word_n & 0x3FFFFFFu) * 96;
+                    const uint32_t *q = relq + (size_t)(live.at[k].word & kBlockMask) * 96;
                     xn = __ldg(q);
                     yn = __ldg(q + 32);
                     zn = __ldg(q + 64);
@@ -479,11 +506,10 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
                 if (nl) fetch(0);
 #pragma unroll 1
                 for (int k = 0; k < nl; ++k) {
-                    const PairSeg &S = seg[word_n >> 26];
-                    const uint32_t slot = (word_n & 0x3FFFFFFu) * 32 + lane;
+                    const LiveBlock S = live.at[k];
                     const float x = (float)(int)(xn - S.cx) * lambda, y = (float)(int)(yn - S.cy) * lambda,
                                 z = (float)(int)(zn - S.cz) * lambda;
-                    const bool mine = slot - S.start < S.end - S.start;
+                    const bool mine = live.slots[k] >> lane & 1u;
                     if (k + 1 < nl) fetch(k + 1);
                     const float ex = fmaxf(fabsf(x) - hx, 0.0f), ey = fmaxf(fabsf(y) - hy, 0.0f),
                                 ez = fmaxf(fabsf(z) - hz, 0.0f);
@@ -494,6 +520,7 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
                         list[0][p] = x;
                         list[1][p] = y;
                         list[2][p] = z;
+                        slot[p] = (S.word & kBlockMask) << 5 | lane;
                     }
                     fill += __popc(mm);
                     if (fill >= kChunk) {
@@ -505,6 +532,7 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
                             list[0][lane] = list[0][kChunk + lane];
                             list[1][lane] = list[1][kChunk + lane];
                             list[2][lane] = list[2][kChunk + lane];
+                            slot[lane] = slot[kChunk + lane];
                         }
                         n_list += kChunk;
                         if (++n_chunks % kFlushChunks == 0) flush();

@@ -104,35 +104,88 @@ __device__ __forceinline__ uint2 group_ranges(PairSeg *seg, const uint32_t *cell
     return make_uint2(__shfl_sync(0xffffffffu, blocks, 1), __shfl_sync(0xffffffffu, blocks, kPairSegs - 1));
 }
 
+// A surviving block: (range << 26) | block, the group's centre in its image, and its slots that belong
+// to the range.
+struct __align__(16) LiveBlock {
+    uint32_t word, cx, cy, cz;
+};
+struct LiveBlocks {
+    LiveBlock at[32];
+    uint32_t slots[32];
+};
+constexpr uint32_t kBlockMask = 0x3FFFFFFu;
+
 // Tests block t of the ranges in sequence (t >= t1: none) against the group's box; the survivors of
-// the warp's 32 blocks go to live[0 ..] in order, coded (range << 26) | block.  Returns their number.
+// the warp's 32 blocks go to live[0 ..] in order.  Returns their number.
 // length: one scaled length (as in f.half); rcull2: the squared cutoff, padded by more than the FP32
 // rounding of absolute coordinates.
 __device__ __forceinline__ int live_blocks(uint32_t t, uint32_t t1, const PairSeg *seg,
                                            const float4 *block_box, const GroupFrame &f, float length,
-                                           float rcull2, uint32_t *live)
+                                           float rcull2, LiveBlocks &live)
 {
     const int lane = threadIdx.x & 31;
     bool keep = false;
-    uint32_t word = 0;
+    LiveBlock q = {0u, 0u, 0u, 0u};
+    uint32_t slots = 0;
     if (t < t1) {
         int s = 0;  // the last range that starts at or before block t
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
             if (s + o < kPairSegs && seg[s + o].first_block <= t) s += o;
-        const uint32_t b = (seg[s].start >> 5) + (t - seg[s].first_block);
+        const PairSeg &S = seg[s];
+        const uint32_t b = (S.start >> 5) + (t - S.first_block);
         const float4 lo = __ldg(block_box + 2 * (size_t)b), hi = __ldg(block_box + 2 * (size_t)b + 1);
-        const float ex = fmaxf(fmaxf(lo.x - seg[s].ax, seg[s].ax - hi.x) - f.half[0] * length, 0.0f);
-        const float ey = fmaxf(fmaxf(lo.y - seg[s].ay, seg[s].ay - hi.y) - f.half[1] * length, 0.0f);
-        const float ez = fmaxf(fmaxf(lo.z - seg[s].az, seg[s].az - hi.z) - f.half[2] * length, 0.0f);
+        const float ex = fmaxf(fmaxf(lo.x - S.ax, S.ax - hi.x) - f.half[0] * length, 0.0f);
+        const float ey = fmaxf(fmaxf(lo.y - S.ay, S.ay - hi.y) - f.half[1] * length, 0.0f);
+        const float ez = fmaxf(fmaxf(lo.z - S.az, S.az - hi.z) - f.half[2] * length, 0.0f);
         keep = ex * ex + ey * ey + ez * ez < rcull2;
-        word = ((uint32_t)s << 26) | b;
+        const uint32_t j0 = max(b * 32, S.start) - b * 32, j1 = min(S.end - b * 32, 32u);
+        slots = (0xffffffffu << j0) & (0xffffffffu >> (32 - j1));  // (0 <= j0 < j1 <= 32)
+        q = {((uint32_t)s << 26) | b, S.cx, S.cy, S.cz};
     }
     const uint32_t m = __ballot_sync(0xffffffffu, keep);
     __syncwarp();  // every lane is done with the previous survivors
-    if (keep) live[__popc(m & ((1u << lane) - 1u))] = word;
+    if (keep) {
+        const int k = __popc(m & ((1u << lane) - 1u));
+        live.at[k] = q;
+        live.slots[k] = slots;
+    }
     __syncwarp();
     return __popc(m);
+}
+
+// ------------------------------------------------------------------ the cutoff
+// FP32 r^2 has an rms error of 8e-8 at the cutoff, which would put about one pair in 10^7 on the wrong
+// side of it: the force jumps there, and for nearly uniform sets those few pairs were the largest part
+// of the error (2e-6 against 4e-7 of the rest; any FP32 evaluation has its own).  So the kernels
+// evaluate with a factor that is 1 inside, 0 outside and a fraction within kCutBand, sum it per lane
+// (it also counts the pairs), and where a sum has a fraction (one list of 160 in 600) look at the list
+// again and decide by the exact fixed-point distance.  (Two clamped FMAs, a product and a sum per two
+// pairs take 4 % of the force kernel's time; compares, selects and counts beside a minimum of
+// |w - rc2| took 9 %.)
+
+// 1 inside the cutoff, 0 outside
+__device__ __forceinline__ float cut_part(float w, float cut_m, float cut_b)
+{
+    return __saturatef(fmaf(w, cut_m, cut_b));
+}
+
+// Whether i and j, whose scaled FP32 difference is (dx, dy, dz), are closer than the cutoff.
+__device__ __forceinline__ bool cut_inside(const uint32_t *relq, uint32_t i, uint32_t j, float dx, float dy,
+                                           float dz, const PairFactor &f)
+{
+    const uint32_t *qi = fix_coords(relq, i), *qj = fix_coords(relq, j);
+    const float d3[3] = {dx, dy, dz};
+    long long r2 = 0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        // the difference of the images: known up to whole cells from the coordinates, which cell from FP32
+        constexpr uint32_t kCell = 1u << kFixBits;
+        const uint32_t e = __ldg(qj + 32 * d) - __ldg(qi + 32 * d), near = (uint32_t)(int)(d3[d] / f.lambda);
+        const long long x = (int)(e + ((near - e + kCell / 2) & ~(kCell - 1u)));
+        r2 += x * x;
+    }
+    return r2 < f.fix_rc2;
 }
 
 }  // namespace

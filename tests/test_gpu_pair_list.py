@@ -116,3 +116,41 @@ def test_force_vjp_lists(kind, n, mesh, cutoff, softening):
     mesh_part = O.pm_vjp(O.wrap(x, box), v, p)
     err = got - mesh_part - ref
     assert math.sqrt(float(np.sum(err ** 2))) <= 2e-5 * math.sqrt(float(np.sum((ref + mesh_part) ** 2)))
+
+
+@pytest.mark.parametrize("box,mesh,cutoff,softening", [
+    (100.0, 48, 4.5, 0.02), (100.0, 64, 4.5, 0.02), (70.0, 54, 4.5, 0.5), (30.0, 24, 2.5, 0.0),
+])
+@pytest.mark.parametrize("off", [3e-8, 2e-7, 1e-5])
+def test_cutoff_decided_exactly(box, mesh, cutoff, softening, off):
+    """Isolated pairs closer to the cutoff than FP32 resolves (its r is 4e-8 off at one sigma), in any
+    direction and across the box's faces: each is inside or outside as its FP64 distance says, in the
+    force and in its derivative.  Bar: the FP32 rounding, 1e-4 of the largest value; a pair on the wrong
+    side is off by all of its short-range force, and by more than 1e-3 of the largest derivative."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1510_07621_gb300 import P3M, build
+    build.build()
+    rng = np.random.default_rng(mesh)
+    rc = cutoff * 1.25 * box / mesh
+    k = int(box / (2.5 * rc))  # pairs on a lattice wide enough that only partners meet
+    assert k >= 1
+    at = np.stack(np.meshgrid(*[np.arange(k)] * 3, indexing="ij")).reshape(3, -1) * (box / k)
+    m = at.shape[1]
+    u = rng.normal(size=(3, m))
+    u /= np.sqrt((u ** 2).sum(0))
+    side = np.where(np.arange(m) % 2 == 0, -1.0, 1.0)  # inside, outside
+    mid = at + 0.1 * rc * rng.uniform(-1, 1, (3, m))
+    half = 0.5 * rc * (1.0 + side * off) * u
+    x = np.mod(np.concatenate([mid - half, mid + half], axis=1), box)
+    v = rng.normal(size=x.shape)
+    got = {}
+    for precision in ("mixed", "fp64"):
+        with P3M(box, 2 * m, mesh, 1.25, cutoff, softening=softening, precision=precision) as sim:
+            sim.set_particles(x, np.zeros_like(x), a=1.0)
+            _, sr = sim.forces_split()
+            got[precision] = sr, sim.force_vjp(v), sim.diagnostics()["pairs"]
+    assert got["mixed"][2] == got["fp64"][2] == 2 * int((side < 0).sum())
+    for a, b in zip(got["mixed"][:2], got["fp64"][:2]):
+        assert np.abs(a - b).max() <= 1e-4 * np.abs(b).max()
