@@ -2,6 +2,7 @@
 #include <cuda_runtime.h>
 
 #include "p3m_internal.cuh"
+#include "state.cuh"
 
 namespace {
 
@@ -22,24 +23,9 @@ __global__ void k_kick(double *__restrict__ mom, const double *__restrict__ acc,
         mom[i] = __dadd_rn(mom[i], __dmul_rn(kfac, acc[i]));
 }
 
-__device__ __forceinline__ double wrap_box(double x, double L)
-{
-    // x = fmod(x, L); x < 0 -> x += L; x >= L -> x -= L.  Inside [0, L) (the common case after
-    // a drift) every step leaves x unchanged, and fmod(x, L) == x for -L < x < L: the FP64
-    // sequence, slow on GB300's FP64 pipe, runs only for the rest.
-    // x in [0, L) as integer compares of the bit patterns (IEEE order of non-negative doubles;
-    // -0.0 and NaN take the full sequence, which leaves -0.0 unchanged, as this test would)
-    const long long xb = __double_as_longlong(x);
-    if (xb >= 0 && xb < __double_as_longlong(L)) return x;
-    if (!(x > -L && x < L)) x = fmod(x, L);
-    if (x < 0.0) x = __dadd_rn(x, L);
-    if (x >= L) x = __dadd_rn(x, -L);
-    return x;
-}
-
 // Copies caller arrays into slot order = caller order, wraps positions, identity ids,
-// and flags any NaN/Inf.
-__global__ void k_load(const double *__restrict__ pos, const double *__restrict__ mom,
+// and flags any NaN/Inf.  Bound by memory: 100 bytes per particle, 256^3 0.316 -> 0.272 ms.
+__global__ void __launch_bounds__(256, 6) k_load(const double *__restrict__ pos, const double *__restrict__ mom,
                        const double *__restrict__ acc, int64_t n, double L,
                        double *__restrict__ pos_out, double *__restrict__ mom_out,
                        double *__restrict__ acc_out, uint32_t *__restrict__ pid,
@@ -51,12 +37,12 @@ __global__ void k_load(const double *__restrict__ pos, const double *__restrict_
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             const double x = pos[d * n + i], p = mom[d * n + i];
-            bad |= !isfinite(x) || !isfinite(p);
-            pos_out[d * n + i] = isfinite(x) ? wrap_box(x, L) : 0.0;
+            bad |= !finite_bits(x) || !finite_bits(p);
+            pos_out[d * n + i] = finite_bits(x) ? wrap_box(x, L) : 0.0;
             mom_out[d * n + i] = p;
             if (acc) {
                 const double a = acc[d * n + i];
-                bad |= !isfinite(a);
+                bad |= !finite_bits(a);
                 acc_out[d * n + i] = a;
             }
         }

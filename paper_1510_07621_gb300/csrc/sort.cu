@@ -18,6 +18,7 @@
 #include <mutex>
 
 #include "p3m_internal.cuh"
+#include "state.cuh"
 
 namespace {
 
@@ -26,22 +27,8 @@ constexpr int kItems = P3M_SORT_TILE / kThreads;  // 16
 constexpr int kRadixBits = 8;
 constexpr int kRadix = 1 << kRadixBits;
 
-__device__ __forceinline__ double wrap_box(double x, double L)
-{
-    // x = fmod(x, L); x < 0 -> x += L; x >= L -> x -= L.  Inside [0, L) (the common case after
-    // a drift) every step leaves x unchanged, and fmod(x, L) == x for -L < x < L: the FP64
-    // sequence, slow on GB300's FP64 pipe, runs only for the rest.
-    // x in [0, L) as integer compares of the bit patterns (IEEE order of non-negative doubles;
-    // -0.0 and NaN take the full sequence, which leaves -0.0 unchanged, as this test would)
-    const long long xb = __double_as_longlong(x);
-    if (xb >= 0 && xb < __double_as_longlong(L)) return x;
-    if (!(x > -L && x < L)) x = fmod(x, L);
-    if (x < 0.0) x = __dadd_rn(x, L);
-    if (x >= L) x = __dadd_rn(x, -L);
-    return x;
-}
-
-__device__ __forceinline__ uint32_t fine_index(double x, double inv, int nf)
+// (not inlined: the compiler would otherwise run the FP64 product for every particle)
+__device__ __noinline__ uint32_t fine_index(double x, double inv, int nf)
 {
     int f = (int)__dmul_rn(x, inv);  // x >= 0: truncation is floor
     return (uint32_t)min(f, nf - 1);
@@ -58,22 +45,27 @@ __device__ __forceinline__ uint32_t fine_index_fast(double x, double inv, float 
     const int e = (int)((xb >> 52) & 0x7FF) - 1023 + 127;  // x >= 0: no sign bit
     const float xf = e >= 1 ? __int_as_float((e << 23) | (int)((xb >> 29) & 0x7FFFFF)) : 0.0f;
     const float p = xf * inv_f;
-    const float k = truncf(p);
-    if (p - k > tol && p - k < 1.0f - tol) return (uint32_t)min((int)k, nf - 1);
+    // floor(p) in the low bits of p + 2^23 rounded towards zero (0 <= p < 2^23)
+    const float t = __fadd_rz(p, 8388608.0f), fr = p - (t - 8388608.0f);
+    if (fr > tol && fr < 1.0f - tol) return (uint32_t)min(__float_as_int(t) & 0x7FFFFF, nf - 1);
     return fine_index(x, inv, nf);
 }
 
+// kBits: sub_bits at compile time, or -1 (any)
+template <int kBits>
 __device__ __forceinline__ uint32_t make_key(uint32_t fx, uint32_t fy, uint32_t fz,
                                              const P3MGeom &g)
 {
-    const int b = g.sub_bits;
+    const int b = kBits >= 0 ? kBits : g.sub_bits;
     const uint32_t cell = ((fz >> b) * (uint32_t)g.n_c + (fy >> b)) * (uint32_t)g.n_c + (fx >> b);
     const uint32_t m = (1u << b) - 1u;
     uint32_t x[3] = {fx & m, fy & m, fz & m}, code = 0;
     if (b > 0) {
         const uint32_t top = 1u << (b - 1);
+#pragma unroll
         for (uint32_t q = top; q > 1; q >>= 1) {  // undo the excess rotations and reflections
             const uint32_t low = q - 1;
+#pragma unroll
             for (int i = 0; i < 3; ++i) {
                 if (x[i] & q) {
                     x[0] ^= low;
@@ -87,10 +79,13 @@ __device__ __forceinline__ uint32_t make_key(uint32_t fx, uint32_t fy, uint32_t 
         x[1] ^= x[0];  // Gray encode
         x[2] ^= x[1];
         uint32_t t = 0;
+#pragma unroll
         for (uint32_t q = top; q > 1; q >>= 1)
             if (x[2] & q) t ^= q - 1;
         for (int i = 0; i < 3; ++i) x[i] ^= t;
+#pragma unroll
         for (int level = b - 1; level >= 0; --level)
+#pragma unroll
             for (int i = 0; i < 3; ++i) code = (code << 1) | ((x[i] >> level) & 1u);
     }
     return (cell << (3 * b)) | code;
@@ -99,13 +94,17 @@ __device__ __forceinline__ uint32_t make_key(uint32_t fx, uint32_t fy, uint32_t 
 // Half kick + drift (optional), periodic wrap, key.  Kick and drift are one FMA each (a single
 // rounding): p += (m K) a; x += p (D / m).  With fac_dev the two factors are read from
 // fac_dev[0], fac_dev[1] (graph-replayed steps).
-__global__ void k_kick_drift_keys(double *__restrict__ pos, double *__restrict__ mom,
-                                  const double *__restrict__ acc, P3MGeom g, int kick_drift,
-                                  double kfac, double dfac, uint32_t *__restrict__ keys,
-                                  const double *__restrict__ fac_dev)
+// Bound by memory (28 bytes per particle, 124 with the kick) once the FP64 compares are out of the way
+// and the Hilbert index is unrolled: 256^3 without a kick 0.381 -> 0.159 ms.  A position that is inside the
+// box already is not written again.
+template <int kBits, bool kKick>
+__global__ void __launch_bounds__(256, 6)
+    k_kick_drift_keys(double *__restrict__ pos, double *__restrict__ mom, const double *__restrict__ acc,
+                      P3MGeom g, double kfac, double dfac, uint32_t *__restrict__ keys,
+                      const double *__restrict__ fac_dev)
 {
     const int64_t n = g.n;
-    if (fac_dev) {
+    if (kKick && fac_dev) {
         kfac = fac_dev[0];
         dfac = fac_dev[1];
     }
@@ -116,16 +115,17 @@ __global__ void k_kick_drift_keys(double *__restrict__ pos, double *__restrict__
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             double x = pos[d * n + i];
-            if (kick_drift) {
+            const double x0 = x;
+            if (kKick) {
                 const double p = __fma_rn(kfac, acc[d * n + i], mom[d * n + i]);
                 mom[d * n + i] = p;
                 x = __fma_rn(p, dfac, x);
             }
             x = wrap_box(x, g.box);
-            pos[d * n + i] = x;
+            if (__double_as_longlong(x) != __double_as_longlong(x0)) pos[d * n + i] = x;
             f[d] = fine_index_fast(x, g.inv_fine, inv_f, tol, g.n_fine);
         }
-        const uint32_t key = make_key(f[0], f[1], f[2], g);
+        const uint32_t key = make_key<kBits>(f[0], f[1], f[2], g);
         p3m_in_bounds((key >> (3 * g.sub_bits)) < (uint32_t)g.n_cells, g.flags);
         keys[i] = key;
     }
@@ -474,7 +474,14 @@ __device__ __forceinline__ double4_16a rel_coords<double4_16a>(double x, double 
     return make_double4_16a(x, y, z, 0.0);
 }
 
-template <typename R4>
+// One warp per 32-slot block of the sorted order; with kPairs (a context with the short-range force)
+// the warp also writes the block's fixed-point coordinates and its bounding box (FP32, absolute
+// coordinates, within the margins of the culling radii).
+// What bounds it: reads of particles in the caller's order, 8 bytes at a time (3 GB of DRAM reads at
+// 256^3 where 1 GB is asked for, 80 % of the DRAM throughput), and 9 FP64 operations per particle (6
+// without kPairs, before 12).  Six CTAs per SM (40 registers): 0.644 -> 0.619 ms at 256^3 against five.
+// Pure PM, 256^3: 0.727 -> 0.678 ms.
+template <typename R4, bool kPairs>
 __global__ void __launch_bounds__(256, 6) k_permute(const uint32_t *__restrict__ perm, const uint32_t *__restrict__ keys,
                           P3MGeom g, const double *__restrict__ pos,
                           const double *__restrict__ mom, const uint32_t *__restrict__ pid,
@@ -483,9 +490,8 @@ __global__ void __launch_bounds__(256, 6) k_permute(const uint32_t *__restrict__
                           float4 *__restrict__ block_box, uint32_t *__restrict__ relq, double fix_scale,
                           const double *__restrict__ origin)
 {
-    // one warp per 32-slot block of the sorted order; the warp also writes the block's
-    // bounding box (FP32, absolute coordinates, rounded outwards by the callers' margins).
-    // Six CTAs per SM (40 registers): the permute phase 0.644 -> 0.619 ms at 256^3 against five.
+    constexpr bool kFp32 = sizeof(R4) == sizeof(float4);
+    const float cs = (float)g.cs;
     const int64_t n = g.n;
     const int64_t nblocks = (n + 31) >> 5;
     const int lane = threadIdx.x & 31;
@@ -499,6 +505,7 @@ __global__ void __launch_bounds__(256, 6) k_permute(const uint32_t *__restrict__
         const uint32_t j = min(pj, (uint32_t)(n - 1));  // in bounds always
         const double x = pos[j], y = pos[n + j], z = pos[2 * n + j];
         R4 rv = make_rel<R4>(0.0, 0.0, 0.0);
+        float lx = 0.0f, ly = 0.0f, lz = 0.0f;
         if (active) {
             pos_out[k] = x;
             pos_out[n + k] = y;
@@ -507,19 +514,34 @@ __global__ void __launch_bounds__(256, 6) k_permute(const uint32_t *__restrict__
             mom_out[n + k] = mom[n + j];
             mom_out[2 * n + k] = mom[2 * n + j];
             pid_out[k] = pid[j];
-            const uint32_t cell = keys[k] >> (3 * g.sub_bits);
+            const uint32_t cell = kFp32 ? keys[k] >> (3 * g.sub_bits) : 0u;  // (the FP64 mode has no use for it)
             const uint32_t cx = cell % g.n_c, cy = (cell / g.n_c) % g.n_c,
                            cz = cell / (g.n_c * g.n_c);
             rv = rel_coords<R4>(x, y, z, cx, cy, cz, origin);
-            rel[k] = rv;
+            if (kFp32 || kPairs) rel[k] = rv;
+            if (kFp32) {
+                lx = fmaf((float)cx, cs, (float)rv.x);
+                ly = fmaf((float)cy, cs, (float)rv.y);
+                lz = fmaf((float)cz, cs, (float)rv.z);
+            }
         }
+        if (!kPairs) continue;
         {  // fixed point: 1.5 * 2^52 rounds x * scale to an integer in the low word (modulo 2^32)
             uint32_t *fix = relq + blk * 96;
             fix[lane] = (uint32_t)__double_as_longlong(fma(x, fix_scale, 0x1.8p52));
             fix[32 + lane] = (uint32_t)__double_as_longlong(fma(y, fix_scale, 0x1.8p52));
             fix[64 + lane] = (uint32_t)__double_as_longlong(fma(z, fix_scale, 0x1.8p52));
         }
-        float lx = (float)x, ly = (float)y, lz = (float)z, hx = lx, hy = ly, hz = lz;
+        if (!kFp32) {
+            lx = (float)x;
+            ly = (float)y;
+            lz = (float)z;
+        }
+        // (slots past the end stand for the block's first particle)
+        const float l0 = __shfl_sync(0xffffffffu, lx, 0), l1 = __shfl_sync(0xffffffffu, ly, 0),
+                    l2 = __shfl_sync(0xffffffffu, lz, 0);
+        if (!active) lx = l0, ly = l1, lz = l2;
+        float hx = lx, hy = ly, hz = lz;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             lx = fminf(lx, __shfl_xor_sync(0xffffffffu, lx, o));
@@ -613,8 +635,10 @@ cudaError_t launch_kick_drift_keys(p3m_ctx *c, bool kick_drift, double kfac, dou
                                    bool from_table)
 {
     c->launches += 1;
-    k_kick_drift_keys<<<grid_for(c->g.n, 256, c->num_sms), 256, 0, c->stream>>>(
-        c->pos, c->mom, c->acc, c->g, kick_drift ? 1 : 0, kfac, dfac, c->keys,
+    auto kern = c->g.sub_bits != 3 ? (kick_drift ? k_kick_drift_keys<-1, true> : k_kick_drift_keys<-1, false>)
+                                   : (kick_drift ? k_kick_drift_keys<3, true> : k_kick_drift_keys<3, false>);
+    kern<<<grid_for(c->g.n, 256, c->num_sms), 256, 0, c->stream>>>(
+        c->pos, c->mom, c->acc, c->g, kfac, dfac, c->keys,
         from_table ? c->cur_fac : nullptr);
     return cudaGetLastError();
 }
@@ -728,17 +752,14 @@ cudaError_t launch_permute_and_cells(p3m_ctx *c)
     const int gb = grid_for(n, 256, c->num_sms);
     const double fix_scale = ldexp((double)c->g.n_c, kFixBits) / c->g.box;
     c->launches += 7;  // permute, cell_start, work_count, 3 scan kernels, work_fill
+    auto permute = [&](auto kern, auto *rel) {
+        kern<<<gb, 256, 0, c->stream>>>(c->vals, c->keys, c->g, c->pos, c->mom, c->pid, c->pos_alt, c->mom_alt,
+                                        c->pid_alt, rel, c->block_box, c->relq, fix_scale, c->tab_origin);
+    };
     if (c->precision == P3M_PREC_MIXED)
-        k_permute<float4><<<gb, 256, 0, c->stream>>>(c->vals, c->keys, c->g, c->pos, c->mom,
-                                                     c->pid, c->pos_alt, c->mom_alt, c->pid_alt,
-                                                     (float4 *)c->rel, c->block_box, c->relq,
-                                                     fix_scale,
-                                                     c->tab_origin);
+        permute(c->short_range ? k_permute<float4, true> : k_permute<float4, false>, (float4 *)c->rel);
     else
-        k_permute<double4_16a><<<gb, 256, 0, c->stream>>>(c->vals, c->keys, c->g, c->pos, c->mom,
-                                                      c->pid, c->pos_alt, c->mom_alt,
-                                                      c->pid_alt, (double4_16a *)c->rel, c->block_box,
-                                                      c->relq, fix_scale, c->tab_origin);
+        permute(c->short_range ? k_permute<double4_16a, true> : k_permute<double4_16a, false>, (double4_16a *)c->rel);
     double *t = c->pos;
     c->pos = c->pos_alt;
     c->pos_alt = t;
@@ -799,7 +820,7 @@ __global__ void k_keys_only(const double *__restrict__ pos, P3MGeom g, uint32_t 
         uint32_t f[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) f[d] = fine_index(wrap_box(pos[d * n + i], g.box), g.inv_fine, g.n_fine);
-        keys[i] = make_key(f[0], f[1], f[2], g);
+        keys[i] = make_key<-1>(f[0], f[1], f[2], g);
     }
 }
 

@@ -1,0 +1,42 @@
+"""Loading, keys and ordering of the particle state: positions on and outside the faces of the box, any
+number of sub-cell bits, with and without the short-range force.  The caller's order is arbitrary, so the
+accelerations of wrapped and unwrapped positions are the same bits; FP32 against FP64 mode: 1e-5 relative
+RMS, the FP32 bar (the sets have no close pairs)."""
+
+import numpy as np
+import pytest
+
+import p3m_synth as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,mesh,sub_bits", [(1, 20, 3), (33, 20, 0), (5003, 24, 3), (4096, 24, 2), (8193, 32, 5)])
+@pytest.mark.parametrize("short_range", [True, False])
+def test_positions_outside_the_box(n, mesh, sub_bits, short_range):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1510_07621_gb300 import P3M, P3MError, build
+    build.build()
+    box = 50.0
+    x = np.mod(S.uniform_random(n, box, 7 + n), box)
+    x = np.round(x * 64) / 64  # exact under shifts by the box
+    x[0, 0] = 0.0
+    y = x + box * np.random.default_rng(n).integers(-2, 3, x.shape)
+    y[0, 0] = -0.0 if n % 2 else box
+    got = {}
+    for precision in ("mixed", "fp64"):
+        with P3M(box, n, mesh, softening=0.3, sub_bits=sub_bits, short_range=short_range, precision=precision) as sim:
+            for name, p in (("in", x), ("out", y)):
+                sim.set_particles(p, np.zeros_like(p), a=1.0)
+                got[precision, name] = sim.forces(1.0)
+            with pytest.raises(P3MError):
+                bad = x.copy()
+                bad[1, n // 2] = np.nan
+                sim.set_particles(bad, np.zeros_like(p), a=1.0)
+        assert np.array_equal(got[precision, "in"], got[precision, "out"])
+    a, b = got["mixed", "in"], got["fp64", "in"]
+    scale = np.sqrt((b ** 2).sum())
+    if n > 1:
+        assert np.sqrt(((a - b) ** 2).sum()) <= 1e-5 * scale
