@@ -282,7 +282,7 @@ void release(p3m_ctx *c)
                     c->tab_one,   c->ps_acc,   c->fac_table,    c->step_idx, c->cur_fac,
                     c->tab_origin,
                     c->adj_u,     c->adj_vfx,  c->adj_vs,       c->adj_out,  c->kself,
-                    c->li,        c->relq,     c->sort_status,  c->sort_hist,
+                    c->li,        c->relq,     c->sort_hist,
                     c->rho_fix,   c->fix_exp,  c->ps_part,     c->sort_probe, c->split_tab};
     for (void *p : bufs)
         if (p) cudaFree(p);
@@ -684,6 +684,9 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
         c->max_work = N / P3M_PAIR_TI + (size_t)g.n_cells + 1;
         const size_t nsort = N > c->max_work ? N : c->max_work;  // longest array the sorts see
         c->n_tiles = (int)((nsort + P3M_SORT_TILE - 1) / P3M_SORT_TILE);
+        const size_t small_n = nsort < P3M_SORT_SMALL ? nsort : P3M_SORT_SMALL;
+        size_t status_bytes = 4 * 256 * 4 * ((small_n + 1023) / 1024);  // per pass, tiles of 1024
+        if (status_bytes < 4 * 256 * (size_t)c->n_tiles) status_bytes = 4 * 256 * (size_t)c->n_tiles;
         const size_t scan_n = (size_t)256 * c->n_tiles > (size_t)g.n_cells + 1 ? (size_t)256 * c->n_tiles
                                                                                : (size_t)g.n_cells + 1;
         struct {
@@ -700,8 +703,7 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
             {(void **)&c->keys_alt, 4 * N},   {(void **)&c->vals, 4 * N},
             {(void **)&c->vals_alt, 4 * N},   {(void **)&c->digit_counts, 4 * 256 * (size_t)c->n_tiles},
             {(void **)&c->scan_aux, 4 * (scan_n / P3M_SORT_TILE + 4)},
-            {(void **)&c->sort_status, 8 * 256 * (size_t)c->n_tiles},
-            {(void **)&c->sort_hist, 4 * (4 * 256 + 4)},
+            {(void **)&c->sort_hist, P3M_SORT_HIST_BYTES + status_bytes},
             {(void **)&c->cell_start, 4 * ((size_t)g.n_cells + 1)},
             {(void **)&c->work, 8 * c->max_work}, {(void **)&c->work_off, 4 * ((size_t)g.n_cells + 1)},
             {(void **)&c->work_key, 4 * c->max_work}, {(void **)&c->work_key_alt, 4 * c->max_work},
@@ -735,6 +737,7 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
         }
         if (rc != P3M_OK) break;
         c->g.flags = c->counters + 1;
+        c->sort_status = c->sort_hist + P3M_SORT_HIST_BYTES / 4;
         cudaMemsetAsync(c->counters, 0, 16, c->stream);
         cudaMemsetAsync(c->pair_count, 0, 64, c->stream);
         // sort buffers start at zero: every key and slot they ever hold is then in range
@@ -1175,7 +1178,7 @@ extern "C" int p3m_inject_fault(p3m_ctx *c, int what, int64_t arg)
         if (!c) return fail(c, P3M_EINVAL, "p3m_inject_fault: the sort timeout needs a context");
         if (arg < 1 || arg > (1ll << 31)) return fail(c, P3M_EINVAL, "p3m_inject_fault: wait limit out of range");
         if (!c->sort_probe) {
-            const size_t bytes = sizeof(unsigned long long) * 256 * (size_t)c->n_tiles;
+            const size_t bytes = sizeof(uint32_t) * 256 * 4 * (size_t)c->n_tiles;  // (tiles of 1024 keys or more)
             CK(cudaMalloc((void **)&c->sort_probe, bytes));
             CK(cudaMemset(c->sort_probe, 0, bytes));
         }

@@ -98,12 +98,12 @@ struct p3m_ctx {
     uint32_t *keys, *keys_alt, *vals, *vals_alt;
     uint32_t *digit_counts;  // 256 * n_tiles
     uint32_t *scan_aux;      // block sums of the scans
-    unsigned long long *sort_status;  // particle sort: 256 look-back entries per 4096-key tile
-    uint32_t *sort_hist;              // particle sort: 4 x 256 digit counts, 4 tile counters
+    uint32_t *sort_hist;              // particle sort: 4 x 256 digit counts, 4 tile counters, then
+    uint32_t *sort_status;            // (same allocation) 256 look-back entries per tile
     int n_tiles;
     int key_bits;
     long long sort_wait_limit;          // clock cycles one look-back wait may take (2^31 ~ 1 s)
-    unsigned long long *sort_probe;     // injected sort timeout: a zeroed status that nothing sets
+    uint32_t *sort_probe;               // injected sort timeout: a zeroed status that nothing sets
     uint32_t *cell_start;  // n_cells + 1
     uint32_t *work;        // pair work items (cell, first slot)
     uint32_t *work_off;    // n_cells + 1
@@ -195,6 +195,11 @@ enum {
 
 #define P3M_MAX_GRAPH_STEPS 4096  // steps per p3m_run_steps / p3m_ensemble_run call
 #define P3M_SORT_TILE 4096   // keys per radix-sort tile (256 threads x 16)
+// Up to this many keys the particle sort takes tiles of 1024 (4096 leave most SMs idle: 48^3 keys are 27
+// tiles), one look-back pass per digit and a status array per pass; above, counted passes.  64^3 keys: 42 us
+// against 84; 128^3: 123 us counted, 133 by look-back.
+#define P3M_SORT_SMALL 262144
+#define P3M_SORT_HIST_BYTES (4 * (4 * 256 + 4))
 #define P3M_PAIR_TI 32       // i-particles per pair work item (one per lane of a warp)
 #define P3M_PAIR_GROUP 16    // particles of a work item that share one list (FP32 kernel)
 #define P3M_PAIR_CTAS 18     // one-warp CTAs per SM that the FP32 kernel's registers leave room for

@@ -132,9 +132,36 @@ __global__ void __launch_bounds__(256, 6)
 }
 
 // ------------------------------------------------------------------ radix sort, 8-bit digits
+
+// The valid lanes whose digit (bits wide) equals this lane's, from one ballot per bit: about 40
+// instructions, where __match_any_sync takes some ten cycles per distinct digit, 300 for random ones.
+__device__ __forceinline__ uint32_t match_digit(uint32_t d, bool valid, int bits)
+{
+    uint32_t peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+    for (int b = 0; b < kRadixBits; ++b) {
+        if (b >= bits) break;
+        const uint32_t one = d >> b & 1u;
+        peers &= ~(__ballot_sync(0xffffffffu, one) ^ (0u - one));
+    }
+    return peers;
+}
+
 // Tile t holds keys [t*4096, (t+1)*4096), visited in 16 rounds of 256 consecutive keys;
 // within a round warp w holds keys [w*32, w*32+32).  That visiting order is the input order,
 // so ranks assigned round by round, warp by warp, lane by lane make each pass stable.
+
+// hist[d] += 1 of every valid lane.  A warp whose digits agree (the upper digits of a set that is nearly
+// sorted) adds once, the others one by one in shared memory.
+__device__ __forceinline__ void count_digit(uint32_t *hist, uint32_t d, bool valid, int lane)
+{
+    const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
+    if (__all_sync(0xffffffffu, valid && d == d0)) {
+        if (lane == 0) atomicAdd(&hist[d0], 32u);
+    } else if (valid) {
+        atomicAdd(&hist[d], 1u);
+    }
+}
 
 __global__ void __launch_bounds__(kThreads)
     k_radix_upsweep(const uint32_t *__restrict__ keys, int64_t n, int shift,
@@ -145,13 +172,15 @@ __global__ void __launch_bounds__(kThreads)
     hist[tid] = 0;
     __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * P3M_SORT_TILE;
+    uint32_t key[kItems];
+#pragma unroll
     for (int r = 0; r < kItems; ++r) {
         const int64_t idx = base + r * kThreads + tid;
-        const bool valid = idx < n;
-        const uint32_t d = valid ? (keys[idx] >> shift) & (kRadix - 1) : (uint32_t)kRadix;
-        const uint32_t peers = __match_any_sync(0xffffffffu, d);
-        if (valid && lane == __ffs(peers) - 1) atomicAdd(&hist[d], (uint32_t)__popc(peers));
+        key[r] = idx < n ? keys[idx] : 0u;
     }
+#pragma unroll
+    for (int r = 0; r < kItems; ++r)
+        count_digit(hist, (key[r] >> shift) & (kRadix - 1), base + r * kThreads + tid < n, lane);
     __syncthreads();
     counts[(size_t)tid * n_tiles + blockIdx.x] = hist[tid];
 }
@@ -179,8 +208,8 @@ __global__ void __launch_bounds__(kThreads)
             key = keys_in[idx];
             val = vals_in ? vals_in[idx] : (uint32_t)idx;
         }
-        const uint32_t d = valid ? (key >> shift) & (kRadix - 1) : (uint32_t)kRadix;
-        const uint32_t peers = __match_any_sync(0xffffffffu, d);
+        const uint32_t d = (key >> shift) & (kRadix - 1);
+        const uint32_t peers = match_digit(d, valid, kRadixBits);
         const uint32_t rank = __popc(peers & lt);
         if (valid && rank == 0) s_cnt[warp][d] = __popc(peers);
         __syncthreads();
@@ -205,9 +234,9 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // ------------------------------------------------------------------ one-sweep LSD radix sort
-// The particle sort: one histogram kernel for all passes, then one kernel per 8-bit pass.  A
-// pass's CTAs take 4096-key tiles in launch order from an atomic counter; each ranks its tile
-// (warp w the keys [512 w, 512 w + 512), round by round and lane by lane, so ranks are
+// The particle sort of few keys: one histogram kernel for all passes, then one kernel per 8-bit pass.  A
+// pass's CTAs take tiles (4096 keys, fewer for few particles) in launch order from an atomic counter; each ranks its tile
+// (warp w its w-th eighth, round by round and lane by lane, so ranks are
 // stable), publishes its per-digit counts, and finds the count of each digit in all earlier
 // tiles by walking back over their published values (decoupled look-back: an entry holds a
 // tile's own count, flag kAgg, or the running total through that tile, flag kInc).  A tile
@@ -216,12 +245,21 @@ __global__ void __launch_bounds__(kThreads)
 // gives up.  The tile is then reordered in shared memory by digit and written out in runs,
 // coalesced, at global position = (keys of smaller digits) + (keys of the digit in earlier
 // tiles) + (rank in the tile).
+// Above P3M_SORT_SMALL keys a pass first counts every tile's digits and scans the counts instead: with
+// hundreds of tiles in flight a tile looks back over hundreds of entries of 256 digits, and that traffic
+// took more time than reading the keys twice.  Sort phase, before / now: 256^3 0.75 / 0.54 ms (look-back
+// with eight entries at once: 0.63), 128^3 0.165 / 0.123, 48^3 (look-back, tiles of 1024; counting: 87 us)
+// 50 / 35 us, 5003 keys 43 / 22 us.  What bounds a pass now is the ranking: 26 ballots per key and their
+// integer operations keep the ALU pipe 75 % busy.
 
 constexpr int kWarps = kThreads / 32;
-constexpr int kWarpItems = P3M_SORT_TILE / kWarps;  // 512
-constexpr unsigned long long kAgg = 1ull << 62, kInc = 2ull << 62, kCountMask = (1ull << 62) - 1;
+constexpr int kLookBack = 8;  // earlier tiles whose entries are read at once (a chain of single reads before)
+constexpr uint32_t kAgg = 1u << 30, kInc = 2u << 30, kCountMask = kAgg - 1;  // (fewer than 2^30 keys)
 
-// hist[p * 256 + d] += number of keys whose digit p is d, for p < passes (<= 4)
+// hist[p * 256 + d] += number of keys whose digit p is d, for p < passes (<= 4).   (Counted by
+// shared-memory atomics: matching equal digits first kept the vote pipe 73 % busy, 256^3 0.118 -> 0.050 ms;
+// 5003 keys, in blocks of 1024 instead of 4096: 8 -> 3.6 us.)
+constexpr int kHistItems = 4;
 __global__ void __launch_bounds__(kThreads)
     k_digit_hist(const uint32_t *__restrict__ keys, int64_t n, int passes, uint32_t *__restrict__ hist)
 {
@@ -229,15 +267,19 @@ __global__ void __launch_bounds__(kThreads)
     for (int i = threadIdx.x; i < 4 * kRadix; i += kThreads) h[i] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * kThreads;
-    for (int64_t i0 = (int64_t)blockIdx.x * kThreads; i0 < n; i0 += stride) {
-        const int64_t i = i0 + threadIdx.x;
-        const bool valid = i < n;
-        const uint32_t k = valid ? keys[i] : 0u;
-        for (int p = 0; p < passes; ++p) {
-            const uint32_t d = valid ? (k >> (p * kRadixBits)) & (kRadix - 1) : (uint32_t)kRadix;
-            const uint32_t peers = __match_any_sync(0xffffffffu, d);
-            if (valid && lane == __ffs(peers) - 1) atomicAdd(&h[p * kRadix + d], (uint32_t)__popc(peers));
+    const int64_t stride = (int64_t)gridDim.x * kThreads * kHistItems;
+    for (int64_t i0 = (int64_t)blockIdx.x * kThreads * kHistItems; i0 < n; i0 += stride) {
+        uint32_t k[kHistItems];
+#pragma unroll
+        for (int r = 0; r < kHistItems; ++r) {
+            const int64_t i = i0 + r * kThreads + threadIdx.x;
+            k[r] = i < n ? keys[i] : 0u;
+        }
+#pragma unroll
+        for (int r = 0; r < kHistItems; ++r) {
+            const bool valid = i0 + r * kThreads + threadIdx.x < n;
+            for (int p = 0; p < passes; ++p)
+                count_digit(h + p * kRadix, (k[r] >> (p * kRadixBits)) & (kRadix - 1), valid, lane);
         }
     }
     __syncthreads();
@@ -247,41 +289,45 @@ __global__ void __launch_bounds__(kThreads)
 
 __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *total);
 
+// kTileItems: keys per thread.  kChain: the counts of earlier tiles by look-back (hist: the digits' totals);
+// otherwise hist holds, digit by digit, the first position of every tile's keys.
+template <int kTileItems, bool kChain>
 __global__ void __launch_bounds__(kThreads, 3)
     k_onesweep(const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin, int64_t n,
-               int shift, const uint32_t *__restrict__ hist, unsigned long long *status,
+               int shift, int bits, const uint32_t *__restrict__ hist, uint32_t *status,
                uint32_t *tile_counter, uint32_t *__restrict__ kout, uint32_t *__restrict__ vout,
-               uint32_t *flags, const unsigned long long *lookback, long long wait_limit)
+               uint32_t *flags, const uint32_t *lookback, long long wait_limit)
 {
-    __shared__ uint32_t s_key[P3M_SORT_TILE];
-    __shared__ uint32_t s_val[P3M_SORT_TILE];
+    constexpr int kTile = kTileItems * kThreads, kWarpItems = kTileItems * 32;
+    __shared__ uint32_t s_key[kTile];
+    __shared__ uint32_t s_val[kTile];
     __shared__ uint32_t s_wcnt[kWarps][kRadix];  // per-warp digit counts, then offsets
     __shared__ uint32_t s_off[kRadix];           // first tile slot of each digit
     __shared__ uint32_t s_out[kRadix];           // global position of the digit's first key
     __shared__ uint32_t s_tile;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) s_tile = atomicAdd(tile_counter, 1u);
+    if (tid == 0) s_tile = kChain ? atomicAdd(tile_counter, 1u) : blockIdx.x;
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) s_wcnt[w][tid] = 0;
     __syncthreads();
     const uint32_t tile = s_tile;
-    const int64_t wbase = (int64_t)tile * P3M_SORT_TILE + (int64_t)warp * kWarpItems;
+    const int64_t wbase = (int64_t)tile * kTile + (int64_t)warp * kWarpItems;
     const uint32_t lt = (1u << lane) - 1u;
 
     // the warp's 512 keys and values (all loads in flight at once), then their ranks
-    uint32_t key[kItems], val[kItems], rank[kItems];
+    uint32_t key[kTileItems], val[kTileItems], rank[kTileItems];
 #pragma unroll
-    for (int r = 0; r < kItems; ++r) {
+    for (int r = 0; r < kTileItems; ++r) {
         const int64_t idx = wbase + r * 32 + lane;
         const bool valid = idx < n;
         key[r] = valid ? kin[idx] : 0u;
         val[r] = valid ? (vin ? vin[idx] : (uint32_t)idx) : 0u;
     }
 #pragma unroll
-    for (int r = 0; r < kItems; ++r) {
+    for (int r = 0; r < kTileItems; ++r) {
         const bool valid = wbase + r * 32 + lane < n;
-        const uint32_t d = valid ? (key[r] >> shift) & (kRadix - 1) : (uint32_t)kRadix;
-        const uint32_t peers = __match_any_sync(0xffffffffu, d);
+        const uint32_t d = (key[r] >> shift) & (kRadix - 1);
+        const uint32_t peers = match_digit(d, valid, bits);
         const int lead = __ffs(peers) - 1;
         uint32_t before = 0;
         if (valid && lane == lead) {
@@ -303,42 +349,57 @@ __global__ void __launch_bounds__(kThreads, 3)
         s_wcnt[w][d] = cnt;
         cnt += c;
     }
-    unsigned long long *mine = status + (size_t)tile * kRadix + d;
-    if (tile == 0)
-        atomicExch(mine, kInc | cnt);
-    else
-        atomicExch(mine, kAgg | cnt);
+    uint32_t *mine = status + (size_t)tile * kRadix + d;
+    if (kChain) atomicExch(mine, (tile == 0 ? kInc : kAgg) | cnt);
     s_off[d] = block_exclusive_scan(cnt, nullptr);
-    const uint32_t first = block_exclusive_scan(hist[d], nullptr);
+    const uint32_t first = kChain ? block_exclusive_scan(hist[d], nullptr) : hist[(size_t)d * gridDim.x + tile];
     // keys of digit d in the tiles before this one
-    unsigned long long before = 0;
-    if (tile > 0) {
+    uint32_t before = 0;
+    if (kChain && tile > 0) {
         long long t = (long long)tile - 1;
         const long long t0 = clock64();
-        for (;;) {
+        for (bool done = false; !done;) {
             // lookback is status itself, except under an injected timeout (a zeroed copy)
-            const unsigned long long v = *(volatile const unsigned long long *)(lookback + (size_t)t * kRadix + d);
-            const unsigned long long f = v & ~kCountMask;
-            if (f == 0ull) {
+            uint32_t v[kLookBack], any = 0, all = kAgg, sum = 0;
+#pragma unroll
+            for (int q = 0; q < kLookBack; ++q) {  // (before tile 0, which publishes kInc: never used)
+                v[q] = t >= q ? *(const volatile uint32_t *)(lookback + (size_t)(t - q) * kRadix + d) : kInc;
+                any |= v[q];
+                all &= v[q];
+                sum += v[q] & kCountMask;
+            }
+            int used = 0;
+            if (!(any & kInc) && all) {  // all of them published, none with a running total
+                before += sum;
+                used = kLookBack;
+            } else {
+                bool ready = true;
+#pragma unroll
+                for (int q = 0; q < kLookBack; ++q) {
+                    ready = ready && !done && (v[q] & ~kCountMask) != 0;
+                    if (!ready) continue;
+                    before += v[q] & kCountMask;
+                    done = (v[q] & kInc) != 0;
+                    ++used;
+                }
+            }
+            t -= used;
+            if (used == 0) {
                 if (clock64() - t0 > wait_limit) {
                     atomicOr(flags, P3M_FLAG_TIMEOUT);
                     break;
                 }
                 __nanosleep(32);
-                continue;
             }
-            before += v & kCountMask;
-            if (f == kInc) break;
-            --t;
         }
         atomicExch(mine, kInc | (before + cnt));
     }
-    s_out[d] = first + (uint32_t)before;
+    s_out[d] = first + before;
     __syncthreads();
 
     // the tile in digit order in shared memory, then written out in runs
 #pragma unroll
-    for (int r = 0; r < kItems; ++r) {
+    for (int r = 0; r < kTileItems; ++r) {
         const int64_t idx = wbase + r * 32 + lane;
         if (idx < n) {
             const uint32_t dd = (key[r] >> shift) & (kRadix - 1);
@@ -348,8 +409,8 @@ __global__ void __launch_bounds__(kThreads, 3)
         }
     }
     __syncthreads();
-    const int64_t left = n - (int64_t)tile * P3M_SORT_TILE;
-    const int count = left < P3M_SORT_TILE ? (int)left : P3M_SORT_TILE;
+    const int64_t left = n - (int64_t)tile * kTile;
+    const int count = left < kTile ? (int)left : kTile;
     for (int j = tid; j < count; j += kThreads) {
         const uint32_t k = s_key[j];
         const uint32_t dd = (k >> shift) & (kRadix - 1);
@@ -474,6 +535,18 @@ __device__ __forceinline__ double4_16a rel_coords<double4_16a>(double x, double 
     return make_double4_16a(x, y, z, 0.0);
 }
 
+// cell_start[c] = first sorted slot whose cell is >= c, the part that slot k (of cell `cell`) writes:
+// the cells after the previous slot's up to its own, and the last slot also the cells after its own.
+__device__ __forceinline__ void first_slots(const uint32_t *keys, int64_t k, uint32_t cell, const P3MGeom &g,
+                                            uint32_t *cell_start)
+{
+    const int64_t prev = k > 0 ? (int64_t)(keys[k - 1] >> (3 * g.sub_bits)) : -1;
+    if (!p3m_in_bounds(cell < (uint32_t)g.n_cells, g.flags)) return;
+    for (int64_t c = prev + 1; c <= (int64_t)cell; ++c) cell_start[c] = (uint32_t)k;
+    if (k == g.n - 1)
+        for (int64_t c = (int64_t)cell + 1; c <= (int64_t)g.n_cells; ++c) cell_start[c] = (uint32_t)g.n;
+}
+
 // One warp per 32-slot block of the sorted order; with kPairs (a context with the short-range force)
 // the warp also writes the block's fixed-point coordinates and its bounding box (FP32, absolute
 // coordinates, within the margins of the culling radii).
@@ -488,7 +561,7 @@ __global__ void __launch_bounds__(256, 6) k_permute(const uint32_t *__restrict__
                           double *__restrict__ pos_out, double *__restrict__ mom_out,
                           uint32_t *__restrict__ pid_out, R4 *__restrict__ rel,
                           float4 *__restrict__ block_box, uint32_t *__restrict__ relq, double fix_scale,
-                          const double *__restrict__ origin)
+                          const double *__restrict__ origin, uint32_t *__restrict__ cell_start)
 {
     constexpr bool kFp32 = sizeof(R4) == sizeof(float4);
     const float cs = (float)g.cs;
@@ -514,7 +587,8 @@ __global__ void __launch_bounds__(256, 6) k_permute(const uint32_t *__restrict__
             mom_out[n + k] = mom[n + j];
             mom_out[2 * n + k] = mom[2 * n + j];
             pid_out[k] = pid[j];
-            const uint32_t cell = kFp32 ? keys[k] >> (3 * g.sub_bits) : 0u;  // (the FP64 mode has no use for it)
+            const uint32_t cell = keys[k] >> (3 * g.sub_bits);
+            first_slots(keys, k, cell, g, cell_start);
             const uint32_t cx = cell % g.n_c, cy = (cell / g.n_c) % g.n_c,
                            cz = cell / (g.n_c * g.n_c);
             rv = rel_coords<R4>(x, y, z, cx, cy, cz, origin);
@@ -558,19 +632,13 @@ __global__ void __launch_bounds__(256, 6) k_permute(const uint32_t *__restrict__
     }
 }
 
-// cell_start[c] = first sorted slot whose cell is >= c (slots k = 0..n, cell(n) = n_cells).
 __global__ void k_cell_start(const uint32_t *__restrict__ keys, P3MGeom g,
                              uint32_t *__restrict__ cell_start)
 {
     const int64_t n = g.n;
-    const int sh = 3 * g.sub_bits;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k <= n;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t prev = k > 0 ? (int64_t)(keys[k - 1] >> sh) : -1;
-        const int64_t cur = k < n ? (int64_t)(keys[k] >> sh) : (int64_t)g.n_cells;
-        if (!p3m_in_bounds(cur <= (int64_t)g.n_cells, g.flags)) continue;
-        for (int64_t c = prev + 1; c <= cur; ++c) cell_start[c] = (uint32_t)k;
-    }
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
+         k += (int64_t)gridDim.x * blockDim.x)
+        first_slots(keys, k, keys[k] >> (3 * g.sub_bits), g, cell_start);
 }
 
 __global__ void k_work_count(const uint32_t *__restrict__ cell_start, int n_cells,
@@ -698,24 +766,44 @@ cudaError_t radix_sort_onesweep(p3m_ctx *c, uint32_t **k, uint32_t **v, bool ide
                                 int64_t n, int key_bits)
 {
     const int passes = (key_bits + kRadixBits - 1) / kRadixBits;
-    const unsigned n_tiles = (unsigned)((n + P3M_SORT_TILE - 1) / P3M_SORT_TILE);
+    const bool small = n <= P3M_SORT_SMALL;
+    const int64_t tile = small ? 4 * kThreads : P3M_SORT_TILE;
+    const unsigned n_tiles = (unsigned)((n + tile - 1) / tile);
+    // (an injected timeout needs a look-back to wait in)
+    const bool chain = small || c->sort_probe;
+    const size_t status_words = (size_t)kRadix * n_tiles;
     cudaStream_t s = c->stream;
-    // sort_hist: 4 x 256 digit counts, then one tile counter per pass
-    cudaError_t e = cudaMemsetAsync(c->sort_hist, 0, sizeof(uint32_t) * (4 * kRadix + 4), s);
-    if (e != cudaSuccess) return e;
-    const unsigned hist_grid = (unsigned)min((int64_t)n_tiles, (int64_t)c->num_sms * 4);
-    k_digit_hist<<<hist_grid, kThreads, 0, s>>>(k[0], n, passes, c->sort_hist);
-    c->launches += 1;
+    cudaError_t e = cudaSuccess;
+    if (chain) {
+        // sort_hist: 4 x 256 digit counts, then one tile counter per pass; sort_status follows it.  Few
+        // particles have a status array per pass, cleared together.
+        e = cudaMemsetAsync(c->sort_hist, 0, P3M_SORT_HIST_BYTES + 4 * status_words * (small ? passes : 1), s);
+        if (e != cudaSuccess) return e;
+        const unsigned hist_grid = (unsigned)min((n + kHistItems * kThreads - 1) / (kHistItems * kThreads),
+                                                 (int64_t)c->num_sms * 8);
+        k_digit_hist<<<hist_grid, kThreads, 0, s>>>(k[0], n, passes, c->sort_hist);
+        c->launches += 1;
+    }
     uint32_t *kin = k[0], *kout = k[1];
     uint32_t *vin = identity_vals ? nullptr : v[0], *vout = identity_vals ? v[0] : v[1];
     for (int p = 0; p < passes; ++p) {
-        e = cudaMemsetAsync(c->sort_status, 0, sizeof(unsigned long long) * kRadix * n_tiles, s);
-        if (e != cudaSuccess) return e;
-        k_onesweep<<<n_tiles, kThreads, 0, s>>>(kin, vin, n, p * kRadixBits, c->sort_hist + p * kRadix,
-                                                c->sort_status, c->sort_hist + 4 * kRadix + p, kout,
-                                                vout, c->counters + 1,
-                                                c->sort_probe ? c->sort_probe : c->sort_status,
-                                                c->sort_wait_limit);
+        const int shift = p * kRadixBits, bits = min(kRadixBits, key_bits - shift);
+        if (chain) {
+            uint32_t *status = c->sort_status + (small ? p * status_words : 0);
+            if (!small && p > 0) e = cudaMemsetAsync(status, 0, 4 * status_words, s);
+            if (e != cudaSuccess) return e;
+            auto sweep = small ? k_onesweep<4, true> : k_onesweep<kItems, true>;
+            sweep<<<n_tiles, kThreads, 0, s>>>(kin, vin, n, shift, bits, c->sort_hist + p * kRadix, status,
+                                               c->sort_hist + 4 * kRadix + p, kout, vout, c->counters + 1,
+                                               c->sort_probe ? c->sort_probe : status, c->sort_wait_limit);
+        } else {
+            k_radix_upsweep<<<n_tiles, kThreads, 0, s>>>(kin, n, shift, c->digit_counts, n_tiles);
+            e = launch_scan_u32(c->digit_counts, c->digit_counts, status_words, c->scan_aux, s);
+            if (e != cudaSuccess) return e;
+            k_onesweep<kItems, false><<<n_tiles, kThreads, 0, s>>>(kin, vin, n, shift, bits, c->digit_counts, nullptr,
+                                                                   nullptr, kout, vout, nullptr, nullptr, 0);
+            c->launches += 4;
+        }
         c->launches += 1;
         uint32_t *t = kin;  // the next pass reads what this one wrote
         kin = kout;
@@ -751,10 +839,10 @@ cudaError_t launch_permute_and_cells(p3m_ctx *c)
     const int64_t n = c->g.n;
     const int gb = grid_for(n, 256, c->num_sms);
     const double fix_scale = ldexp((double)c->g.n_c, kFixBits) / c->g.box;
-    c->launches += 7;  // permute, cell_start, work_count, 3 scan kernels, work_fill
+    c->launches += 6;  // permute, work_count, 3 scan kernels, work_fill
     auto permute = [&](auto kern, auto *rel) {
         kern<<<gb, 256, 0, c->stream>>>(c->vals, c->keys, c->g, c->pos, c->mom, c->pid, c->pos_alt, c->mom_alt,
-                                        c->pid_alt, rel, c->block_box, c->relq, fix_scale, c->tab_origin);
+                                        c->pid_alt, rel, c->block_box, c->relq, fix_scale, c->tab_origin, c->cell_start);
     };
     if (c->precision == P3M_PREC_MIXED)
         permute(c->short_range ? k_permute<float4, true> : k_permute<float4, false>, (float4 *)c->rel);
@@ -770,8 +858,6 @@ cudaError_t launch_permute_and_cells(p3m_ctx *c)
     c->pid = c->pid_alt;
     c->pid_alt = u;
 
-    k_cell_start<<<grid_for(n + 1, 256, c->num_sms), 256, 0, c->stream>>>(c->keys, c->g,
-                                                                         c->cell_start);
     cudaMemsetAsync(c->counters + 2, 0, sizeof(uint32_t), c->stream);
     const int gc = grid_for(c->g.n_cells, 256, c->num_sms);
     cudaMemsetAsync(c->work_off + c->g.n_cells, 0, sizeof(uint32_t), c->stream);
@@ -911,7 +997,7 @@ extern "C" int p3m_cell_sort_noalloc(const double *pos3n, int64_t n, double box,
     if (e == cudaSuccess && v[0] != ids_out)
         e = cudaMemcpyAsync(ids_out, v[0], 4 * (size_t)n, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess) {
-        k_cell_start<<<grid_for(n + 1, 256, sms), 256, 0, s>>>(keys_out, g, cell_start_out);
+        k_cell_start<<<grid_for(n, 256, sms), 256, 0, s>>>(keys_out, g, cell_start_out);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess)

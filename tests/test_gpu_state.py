@@ -40,3 +40,30 @@ def test_positions_outside_the_box(n, mesh, sub_bits, short_range):
     scale = np.sqrt((b ** 2).sum())
     if n > 1:
         assert np.sqrt(((a - b) ** 2).sum()) <= 1e-5 * scale
+
+
+@pytest.mark.parametrize("n,mesh", [(1, 20), (1023, 48), (1024, 48), (1025, 48), (4097, 64), (262143, 192), (262144, 192),
+                                    (262145, 192), (270337, 192)])
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_sort_at_tile_edges(n, mesh, precision):
+    """The sort at the edges of its tiles and of its two methods: every particle is found by its neighbours
+    (the number of pairs within the cutoff, against a k-d tree; at most two pairs lie within the FP32 mode's
+    coordinate rounding of the cutoff) and again after a second sort of the sorted state."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    spatial = pytest.importorskip("scipy.spatial")
+    from paper_1510_07621_gb300 import P3M, build
+    build.build()
+    box = 100.0
+    x = np.mod(S.uniform_random(n, box, 11 + n), box)
+    tree = spatial.cKDTree(x.T, boxsize=box)
+    rc = 4.5 * 1.25 * box / mesh
+    want = int(tree.count_neighbors(tree, rc)) - n
+    with P3M(box, n, mesh, softening=0.3, precision=precision) as sim:
+        sim.set_particles(x, np.zeros_like(x), a=1.0)
+        first = sim.forces(1.0)
+        for _ in range(2):
+            assert abs(sim.diagnostics()["pairs"] - want) <= (4 if precision == "mixed" else 0)
+            again = sim.forces(1.0)
+        assert np.array_equal(first, again)
