@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(32)
     k_pairs_vjp64(const double4_16a *__restrict__ rel, const double *__restrict__ pos,
                   const float4 *__restrict__ block_box, const double *__restrict__ vs,
                   const uint32_t *__restrict__ cell_start, const uint32_t *__restrict__ work,
-                  const uint32_t *__restrict__ order, const uint32_t *__restrict__ n_work_ptr,
+                  const uint32_t *__restrict__ n_work_ptr,
                   P3MGeom g, float rcull2, float rin2, uint32_t *__restrict__ cursor,
                   double *__restrict__ out)
 {
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(32)
         if (lane == 0) slot = atomicAdd(cursor, 1u);
         slot = __shfl_sync(0xffffffffu, slot, 0);
         if (slot >= n_work) break;
-        const uint32_t item = order[slot];
+        const uint32_t item = slot;
         const uint32_t cell = work[2 * (size_t)item], first = work[2 * (size_t)item + 1];
         const uint32_t cend = cell_start[cell + 1];
         const int cx = (int)(cell % nc), cy = (int)((cell / nc) % nc), cz = (int)(cell / (nc * nc));
@@ -439,7 +439,7 @@ template <bool kAdditive>
 __global__ void __launch_bounds__(32, 16)
     k_pairs_vjp_list(const uint32_t *__restrict__ relq, const float *__restrict__ vfx,
                      const float4 *__restrict__ block_box, const uint32_t *__restrict__ cell_start,
-                     const uint32_t *__restrict__ work, const uint32_t *__restrict__ order,
+                     const uint32_t *__restrict__ work,
                      const uint32_t *__restrict__ n_work_ptr, P3MGeom g, PairFactor fac, double scale,
                      float rcull2, uint32_t *__restrict__ cursor, double *__restrict__ out)
 {
@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(32, 16)
         if (lane == 0) unit = atomicAdd(cursor, 1u);
         unit = __shfl_sync(0xffffffffu, unit, 0);
         if (unit >= n_units) break;
-        const uint32_t item = order[unit / kSub];
+        const uint32_t item = unit / kSub;
         const uint32_t cell = work[2 * (size_t)item];
         const uint32_t first = work[2 * (size_t)item + 1] + (unit % kSub) * kG;
         const uint32_t cend = cell_start[cell + 1];
@@ -729,7 +729,7 @@ template <typename T>
 __global__ void __launch_bounds__(32)
     k_pairs_potential(const typename V4Of<T>::type *__restrict__ rel, const double *__restrict__ pos,
                       const float4 *__restrict__ block_box, const uint32_t *__restrict__ cell_start,
-                      const uint32_t *__restrict__ work, const uint32_t *__restrict__ order,
+                      const uint32_t *__restrict__ work,
                       const uint32_t *__restrict__ n_work_ptr, P3MGeom g, float rcull2,
                       uint32_t *__restrict__ cursor, double *__restrict__ phi_out)
 {
@@ -745,7 +745,7 @@ __global__ void __launch_bounds__(32)
         if (lane == 0) slot = atomicAdd(cursor, 1u);
         slot = __shfl_sync(0xffffffffu, slot, 0);
         if (slot >= n_work) break;
-        const uint32_t item = order[slot];
+        const uint32_t item = slot;
         const uint32_t cell = work[2 * (size_t)item], first = work[2 * (size_t)item + 1];
         const uint32_t cend = cell_start[cell + 1];
         const int cx = (int)(cell % nc), cy = (int)((cell / nc) % nc), cz = (int)(cell / (nc * nc));
@@ -883,7 +883,7 @@ cudaError_t potential_impl(p3m_ctx *c, double cst, double *phi_slots, double *su
         c->launches += 1;
         k_pairs_potential<T><<<c->num_sms * (per_sm < 1 ? 1 : per_sm), 32, 0, c->stream>>>(
             (const typename V4Of<T>::type *)c->rel, c->pos, c->block_box, c->cell_start, c->work,
-            c->work_order, c->work_off + c->g.n_cells, c->g, (float)(rcull * rcull), c->counters + 3,
+            c->n_work, c->g, (float)(rcull * rcull), c->counters + 3,
             phi_slots);
     }
     c->launches += 2;
@@ -951,13 +951,13 @@ cudaError_t vjp_pairs(p3m_ctx *c, const double *v_slots, double *out_slots)
     if (fp32) {
         const double len = ldexp(c->g.cs, -kFixBits) / (double)c->pair_factor.lambda;
         list<<<c->num_sms * per_sm, 32, 0, c->stream>>>(
-            c->relq, c->adj_vfx, c->block_box, c->cell_start, c->work, c->work_order,
-            c->work_off + c->g.n_cells, c->g, c->pair_factor, c->g.gm / (len * len * len), rcull2,
+            c->relq, c->adj_vfx, c->block_box, c->cell_start, c->work,
+            c->n_work, c->g, c->pair_factor, c->g.gm / (len * len * len), rcull2,
             c->counters + 3, out_slots);
     } else {
         k_pairs_vjp64<<<c->num_sms * per_sm, 32, 0, c->stream>>>(
             (const double4_16a *)c->rel, c->pos, c->block_box, v_slots, c->cell_start, c->work,
-            c->work_order, c->work_off + c->g.n_cells, c->g, rcull2, rin2, c->counters + 3,
+            c->n_work, c->g, rcull2, rin2, c->counters + 3,
             out_slots);
     }
     return cudaGetLastError();

@@ -275,10 +275,9 @@ void release(p3m_ctx *c)
     void *bufs[] = {c->pos,       c->mom,      c->acc,          c->acc_lr,   c->pid,
                     c->pos_alt,   c->mom_alt,  c->pid_alt,      c->rel,      c->keys,
                     c->keys_alt,  c->vals,     c->vals_alt,     c->digit_counts, c->scan_aux,
-                    c->cell_start, c->work,    c->work_off,     c->counters, c->pair_count,
+                    c->cell_start, c->work,    c->counters, c->pair_count,
                     c->red,       c->rho,      c->rho_k,        c->frc_k,    c->frc,
-                    c->tab_k,     c->tab_kg,   c->tab_g,        c->work_key, c->work_key_alt,
-                    c->work_order, c->work_order_alt, c->block_box, c->tab_invw2,
+                    c->tab_k,     c->tab_kg,   c->tab_g,        c->work_key, c->block_box, c->tab_invw2,
                     c->tab_one,   c->ps_acc,   c->fac_table,    c->step_idx, c->cur_fac,
                     c->tab_origin,
                     c->adj_u,     c->adj_vfx,  c->adj_vs,       c->adj_out,  c->kself,
@@ -521,15 +520,14 @@ int step_pre(p3m_ctx *c, double a, double da, bool from_table, int slot, PairArg
     c->launches += 2;
     CK(launch_store_pair_args(desc, pair_args(c, c->acc_lr, c->acc, k2, from_table ? c->cur_fac + 2 : nullptr),
                               c->stream));
-    CK(launch_ens_gather(slot, c->work_key, c->work_order, c->max_work, gk, gv, c->stream));
+    CK(launch_ens_gather(slot, c->work_key, c->max_work, gk, gv, c->stream));
     return P3M_OK;
 }
 
 PtrState save_ptrs(const p3m_ctx *c)
 {
     return PtrState{c->pos,      c->mom,      c->pos_alt,  c->mom_alt,      c->pid,
-                    c->pid_alt,  c->keys,     c->keys_alt, c->vals,         c->vals_alt,
-                    c->work_key, c->work_key_alt, c->work_order, c->work_order_alt};
+                    c->pid_alt,  c->keys,     c->keys_alt, c->vals,         c->vals_alt};
 }
 
 void load_ptrs(p3m_ctx *c, const PtrState &s)
@@ -544,10 +542,6 @@ void load_ptrs(p3m_ctx *c, const PtrState &s)
     c->keys_alt = s.keys_alt;
     c->vals = s.vals;
     c->vals_alt = s.vals_alt;
-    c->work_key = s.work_key;
-    c->work_key_alt = s.work_key_alt;
-    c->work_order = s.work_order;
-    c->work_order_alt = s.work_order_alt;
 }
 
 }  // namespace p3m_host
@@ -682,13 +676,11 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
         const size_t N = (size_t)n, M = (size_t)mesh, nk = M * M * (M / 2 + 1), M3 = M * M * M;
         const size_t real = c->precision == P3M_PREC_MIXED ? 4 : 8;
         c->max_work = N / P3M_PAIR_TI + (size_t)g.n_cells + 1;
-        const size_t nsort = N > c->max_work ? N : c->max_work;  // longest array the sorts see
-        c->n_tiles = (int)((nsort + P3M_SORT_TILE - 1) / P3M_SORT_TILE);
-        const size_t small_n = nsort < P3M_SORT_SMALL ? nsort : P3M_SORT_SMALL;
+        c->n_tiles = (int)((N + P3M_SORT_TILE - 1) / P3M_SORT_TILE);
+        const size_t small_n = N < P3M_SORT_SMALL ? N : P3M_SORT_SMALL;
         size_t status_bytes = 4 * 256 * 4 * ((small_n + 1023) / 1024);  // per pass, tiles of 1024
         if (status_bytes < 4 * 256 * (size_t)c->n_tiles) status_bytes = 4 * 256 * (size_t)c->n_tiles;
-        const size_t scan_n = (size_t)256 * c->n_tiles > (size_t)g.n_cells + 1 ? (size_t)256 * c->n_tiles
-                                                                               : (size_t)g.n_cells + 1;
+        const size_t scan_n = (size_t)256 * c->n_tiles;
         struct {
             void **p;
             size_t bytes;
@@ -705,10 +697,8 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
             {(void **)&c->scan_aux, 4 * (scan_n / P3M_SORT_TILE + 4)},
             {(void **)&c->sort_hist, P3M_SORT_HIST_BYTES + status_bytes},
             {(void **)&c->cell_start, 4 * ((size_t)g.n_cells + 1)},
-            {(void **)&c->work, 8 * c->max_work}, {(void **)&c->work_off, 4 * ((size_t)g.n_cells + 1)},
-            {(void **)&c->work_key, 4 * c->max_work}, {(void **)&c->work_key_alt, 4 * c->max_work},
-            {(void **)&c->work_order, 4 * c->max_work}, {(void **)&c->work_order_alt, 4 * c->max_work},
-            {(void **)&c->counters, 16},      {(void **)&c->pair_count, 64},
+            {(void **)&c->work, 8 * c->max_work}, {(void **)&c->work_key, 4 * c->max_work},
+            {(void **)&c->counters, 4 * P3M_COUNTERS},      {(void **)&c->pair_count, 64},
             {(void **)&c->red, 8 * (1024 * 4 + 8)},
             {(void **)&c->rho, real * M3},    {(void **)&c->rho_k, 2 * real * nk},
             {(void **)&c->frc_k, 6 * real * nk}, {(void **)&c->frc, 3 * real * M3},
@@ -738,7 +728,8 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
         if (rc != P3M_OK) break;
         c->g.flags = c->counters + 1;
         c->sort_status = c->sort_hist + P3M_SORT_HIST_BYTES / 4;
-        cudaMemsetAsync(c->counters, 0, 16, c->stream);
+        c->n_work = c->counters + 4 + 256;
+        cudaMemsetAsync(c->counters, 0, 4 * P3M_COUNTERS, c->stream);
         cudaMemsetAsync(c->pair_count, 0, 64, c->stream);
         // sort buffers start at zero: every key and slot they ever hold is then in range
         cudaMemsetAsync(c->keys_alt, 0, 4 * N, c->stream);

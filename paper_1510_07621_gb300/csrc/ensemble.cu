@@ -409,7 +409,7 @@ extern "C" int p3m_ensemble_create(p3m_ensemble **out, p3m_ctx *const *ctxs, int
         if (ok) {
             e->base[e->nb] = e->cap;
             e->cap += c->max_work;
-            nw.push_back(c->work_off + c->g.n_cells);
+            nw.push_back(c->n_work);
             ++e->nb;
         }
     }

@@ -94,7 +94,6 @@ int step_pre(p3m_ctx *c, double a, double da, bool from_table, int slot, PairArg
 struct PtrState {
     double *pos, *mom, *pos_alt, *mom_alt;
     uint32_t *pid, *pid_alt, *keys, *keys_alt, *vals, *vals_alt;
-    uint32_t *work_key, *work_key_alt, *work_order, *work_order_alt;
     bool operator==(const PtrState &o) const { return memcmp(this, &o, sizeof(*this)) == 0; }
 };
 

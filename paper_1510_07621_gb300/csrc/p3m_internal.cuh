@@ -105,12 +105,12 @@ struct p3m_ctx {
     long long sort_wait_limit;          // clock cycles one look-back wait may take (2^31 ~ 1 s)
     uint32_t *sort_probe;               // injected sort timeout: a zeroed status that nothing sets
     uint32_t *cell_start;  // n_cells + 1
-    uint32_t *work;        // pair work items (cell, first slot)
-    uint32_t *work_off;    // n_cells + 1
-    uint32_t *work_key, *work_key_alt;      // cost keys of the work items (max_work)
-    uint32_t *work_order, *work_order_alt;  // work items, most expensive first (max_work)
+    uint32_t *work;        // pair work items (cell, first slot), most expensive first (max_work)
+    uint32_t *work_key;    // their cost keys (max_work)
     size_t max_work;
-    uint32_t *counters;  // [0] work cursor [1] error flags [2] max cell count [3] spare
+    // [0] work cursor [1] error flags [2] max cell count [3] spare, then the work list's 256 class counts,
+    // its length (n_work) and 256 places
+    uint32_t *counters, *n_work;
     unsigned long long *pair_count;  // [0] last evaluation [1] cumulative
     unsigned long long launches;     // kernels launched by the library (host-side count)
     double *red;  // reduction partials
@@ -203,6 +203,7 @@ enum {
 #define P3M_PAIR_TI 32       // i-particles per pair work item (one per lane of a warp)
 #define P3M_PAIR_GROUP 16    // particles of a work item that share one list (FP32 kernel)
 #define P3M_PAIR_CTAS 18     // one-warp CTAs per SM that the FP32 kernel's registers leave room for
+#define P3M_COUNTERS (4 + 256 + 1 + 256)  // 32-bit words of counters
 #define P3M_FLAG_TIMEOUT 1u  // counters[1] bit: a bounded wait gave up
 
 // Everything the FP32 pair kernel needs from one context: its arrays, geometry, fitted split
@@ -266,10 +267,9 @@ cudaError_t launch_pairs_batched(const PairArgs *descs, const uint32_t *order,
                                  cudaStream_t s);
 // dst (device) = a, as one kernel (so that captured graphs write the current pointers).
 cudaError_t launch_store_pair_args(PairArgs *dst, const PairArgs &a, cudaStream_t s);
-// Batched launch bookkeeping: copies one context's sorted work list (n entries) into the merged
+// Batched launch bookkeeping: copies the keys of one context's work list (n entries) into the merged
 // arrays, values coded (slot << 24) | item; *total = sum over nb contexts of *nwork[k].
-cudaError_t launch_ens_gather(int slot, const uint32_t *key, const uint32_t *order, size_t n,
-                              uint32_t *gkey, uint32_t *gval, cudaStream_t s);
+cudaError_t launch_ens_gather(int slot, const uint32_t *key, size_t n, uint32_t *gkey, uint32_t *gval, cudaStream_t s);
 cudaError_t launch_ens_total(const uint32_t *const *nwork, int nb, uint32_t *total, cudaStream_t s);
 // Stable LSD radix sort of n (key, value) pairs on the low key_bits bits; k[0]/v[0] hold the
 // result on return (the arrays are swapped when an odd number of passes ran).

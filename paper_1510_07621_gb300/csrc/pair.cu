@@ -77,7 +77,7 @@ constexpr int kEntries64 = 96;  // blocks per round (about what a group of 8 has
 __global__ void __launch_bounds__(32)
     k_pairs64(const uint32_t *__restrict__ relq, const double *__restrict__ pos,
               const float4 *__restrict__ block_box, const uint32_t *__restrict__ cell_start,
-              const uint32_t *__restrict__ work, const uint32_t *__restrict__ order,
+              const uint32_t *__restrict__ work,
               const uint32_t *__restrict__ n_work_ptr, P3MGeom g, const double *__restrict__ split, float rcull2, float rlist2,
               const double *__restrict__ acc_in, double *__restrict__ acc_out,
               double *__restrict__ mom, double kfac, const double *__restrict__ kfac_dev,
@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(32)
         if (lane == 0) unit = atomicAdd(cursor, 1u);
         unit = __shfl_sync(0xffffffffu, unit, 0);
         if (unit >= n_units) break;
-        const uint32_t item = order[unit / kSub];
+        const uint32_t item = unit / kSub;
         const uint32_t cell = work[2 * (size_t)item];
         const uint32_t first = work[2 * (size_t)item + 1] + (unit % kSub) * kG;
         const uint32_t cend = cell_start[cell + 1];
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
         if (lane == 0) unit = atomicAdd(cursor, 1u);
         unit = __shfl_sync(0xffffffffu, unit, 0);
         if (unit >= n_units) break;
-        uint32_t item = order[unit / kSub];
+        uint32_t item = kBatched ? order[unit / kSub] : unit / kSub;
         if (kBatched) {
             const int sim = (int)(item >> 24);
             item &= 0xFFFFFFu;
@@ -599,7 +599,7 @@ cudaError_t pairs64_impl(p3m_ctx *c, const double *acc_in, double *acc_out, doub
     const double rcull = c->g.r_c * (1.0 + 1e-4) + c->g.box * 1e-6, rlist = c->g.r_c / c->g.cs + 2e-6;
     c->launches += 1;
     k_pairs64<<<grid, 32, 0, c->stream>>>(c->relq, c->pos, c->block_box, c->cell_start, c->work,
-                                          c->work_order, c->work_off + c->g.n_cells, c->g, c->split_tab,
+                                          c->n_work, c->g, c->split_tab,
                                           (float)(rcull * rcull), (float)(rlist * rlist), acc_in, acc_out,
                                           c->mom, kfac, kfac_dev, c->counters, c->pair_count);
     return cudaGetLastError();
@@ -625,23 +625,21 @@ cudaError_t pairs_list_impl(p3m_ctx *c, const double *acc_in, double *acc_out, d
     cudaMemsetAsync(c->pair_count, 0, sizeof(unsigned long long), c->stream);  // last evaluation
     c->launches += 1;
     const PairArgs a = pair_args(c, acc_in, acc_out, kfac, kfac_dev);
-    const uint32_t *n_work = c->work_off + c->g.n_cells;
     const bool add = c->pair_factor.additive != 0;
     auto launch = c->tile_blocks == kShortChunk ? (add ? launch_list<false, 1, kShortChunk> : launch_list<false, 0, kShortChunk>)
                                                 : (add ? launch_list<false, 1, kLongChunk> : launch_list<false, 0, kLongChunk>);
-    return launch(a, nullptr, c->work_order, n_work, c->counters, c->num_sms, c->stream);
+    return launch(a, nullptr, nullptr, c->n_work, c->counters, c->num_sms, c->stream);
 }
 
 __global__ void k_store_pair_args(PairArgs *dst, PairArgs a) { *dst = a; }
 
 __global__ void k_ens_gather(uint32_t slot, const uint32_t *__restrict__ key,
-                             const uint32_t *__restrict__ order, size_t n, uint32_t *__restrict__ gk,
-                             uint32_t *__restrict__ gv)
+                             size_t n, uint32_t *__restrict__ gk, uint32_t *__restrict__ gv)
 {
     for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n;
          k += (size_t)gridDim.x * blockDim.x) {
         gk[k] = key[k];
-        gv[k] = (slot << 24) | (order[k] & 0xFFFFFFu);
+        gv[k] = (slot << 24) | ((uint32_t)k & 0xFFFFFFu);
     }
 }
 
@@ -696,12 +694,11 @@ cudaError_t launch_store_pair_args(PairArgs *dst, const PairArgs &a, cudaStream_
     return cudaGetLastError();
 }
 
-cudaError_t launch_ens_gather(int slot, const uint32_t *key, const uint32_t *order, size_t n,
-                              uint32_t *gkey, uint32_t *gval, cudaStream_t s)
+cudaError_t launch_ens_gather(int slot, const uint32_t *key, size_t n, uint32_t *gkey, uint32_t *gval, cudaStream_t s)
 {
     const size_t blocks = (n + 255) / 256;
     k_ens_gather<<<(unsigned)(blocks < 1 ? 1 : (blocks > 1024 ? 1024 : blocks)), 256, 0, s>>>(
-        (uint32_t)slot, key, order, n, gkey, gval);
+        (uint32_t)slot, key, n, gkey, gval);
     return cudaGetLastError();
 }
 
