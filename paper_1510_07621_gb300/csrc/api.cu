@@ -713,7 +713,7 @@ extern "C" int p3m_init(p3m_ctx **out, double box, int64_t n, int mesh, double r
             {(void **)&c->kself, 8 * 27},     {(void **)&c->li, 8 * 4},
             {(void **)&c->adj_u, 3 * real * M3}, {(void **)&c->adj_vfx, opt.precision == P3M_PREC_MIXED ? 384 * ((N + 31) / 32) : 16},
             {(void **)&c->adj_vs, 24 * N},    {(void **)&c->adj_out, 24 * N},
-            {(void **)&c->split_tab, opt.precision == P3M_PREC_FP64 ? 8 * kSplitTab64 * kSplitRow64 : 16},
+            {(void **)&c->split_tab, opt.precision == P3M_PREC_FP64 ? (size_t)8 * kSplitTab64 * kSplitRow64 : 16},
         };
         int idx = 0;
         for (auto &a : allocs) {
@@ -929,9 +929,9 @@ extern "C" int p3m_forces_split(p3m_ctx *c, double *acc_lr, double *acc_sr, int 
     for (int t = 0; t < 2; ++t) {
         if (!outs[t]) continue;
         if (on_device) {
-            CK(launch_scatter_out(c, srcs[t], outs[t]));
+            CK(launch_output(c, srcs[t], outs[t]));
         } else {
-            CK(launch_scatter_out(c, srcs[t], c->pos_alt));
+            CK(launch_output(c, srcs[t], c->pos_alt));
             CK(cudaMemcpyAsync(outs[t], c->pos_alt, bytes, cudaMemcpyDeviceToHost, c->stream));
             CK(cudaStreamSynchronize(c->stream));
         }
@@ -1001,22 +1001,23 @@ extern "C" int p3m_get_particles(p3m_ctx *c, double *pos, double *mom, double *a
     const size_t bytes = 3 * sizeof(double) * (size_t)c->g.n;
     double *outs[3] = {pos, mom, acc};
     const double *srcs[3] = {c->pos, c->mom, c->acc};
-    bool inv_ready = false;  // pid_alt is free between sorts: the inverse permutation
+    // device arrays, page-locked host arrays (written in place), other host arrays (staged)
+    const double *from[3][3];
+    double *to[3][3], *const stage[3] = {c->pos_alt, c->mom_alt, c->acc_lr};
+    int count[3] = {0, 0, 0};
     for (int t = 0; t < 3; ++t) {
         if (!outs[t]) continue;
         double *direct = on_device ? nullptr : (double *)pinned_view(outs[t]);
-        if (on_device) {
-            CK(launch_scatter_out(c, srcs[t], outs[t]));
-        } else if (direct) {  // pinned host array: written in place, sequentially
-            if (!inv_ready) CK(launch_inverse_pid(c, c->pid_alt));
-            inv_ready = true;
-            CK(launch_gather_out(c, srcs[t], c->pid_alt, direct));
-        } else {
-            double *stage = t == 0 ? c->pos_alt : (t == 1 ? c->mom_alt : c->acc_lr);
-            CK(launch_scatter_out(c, srcs[t], stage));
-            CK(cudaMemcpyAsync(outs[t], stage, bytes, cudaMemcpyDeviceToHost, c->stream));
-        }
+        const int way = on_device ? 0 : (direct ? 1 : 2);
+        from[way][count[way]] = srcs[t];
+        to[way][count[way]++] = on_device ? outs[t] : (direct ? direct : stage[t]);
     }
+    for (int way = 0; way < 3; ++way)
+        if (count[way]) CK(launch_outputs(c, from[way], to[way], count[way], way == 1));
+    if (count[2])
+        for (int t = 0; t < 3; ++t)
+            if (outs[t] && !pinned_view(outs[t]))
+                CK(cudaMemcpyAsync(outs[t], stage[t], bytes, cudaMemcpyDeviceToHost, c->stream));
     if (!on_device) return check_flags(c);
     return P3M_OK;
 }

@@ -49,10 +49,10 @@ extern "C" int p3m_force_vjp(p3m_ctx *c, const double *v3n, double *out3n, int o
     CK(launch_to_slots(c, vin, c->adj_vs));
     CK(launch_force_vjp(c, c->adj_vs, c->adj_out));
     if (on_device) {
-        CK(launch_scatter_out(c, c->adj_out, out3n));
+        CK(launch_output(c, c->adj_out, out3n));
         return P3M_OK;
     }
-    CK(launch_scatter_out(c, c->adj_out, c->pos_alt));
+    CK(launch_output(c, c->adj_out, c->pos_alt));
     CK(cudaMemcpyAsync(out3n, c->pos_alt, bytes, cudaMemcpyDeviceToHost, c->stream));
     return check_flags(c);
 }
@@ -74,9 +74,9 @@ extern "C" int p3m_density_loss(p3m_ctx *c, const double *target, double *loss, 
     CK(launch_density_loss(c, t, loss_dev, grad3n ? c->adj_out : nullptr));
     if (grad3n) {
         if (on_device) {
-            CK(launch_scatter_out(c, c->adj_out, grad3n));
+            CK(launch_output(c, c->adj_out, grad3n));
         } else {
-            CK(launch_scatter_out(c, c->adj_out, c->pos_alt));
+            CK(launch_output(c, c->adj_out, c->pos_alt));
             CK(cudaMemcpyAsync(grad3n, c->pos_alt, bytes, cudaMemcpyDeviceToHost, c->stream));
         }
     }

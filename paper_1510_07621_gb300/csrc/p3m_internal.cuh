@@ -288,10 +288,10 @@ cudaError_t launch_step_begin(p3m_ctx *c);
 cudaError_t launch_axpy(p3m_ctx *c, double *y, const double *x, double alpha);
 cudaError_t launch_load_particles(p3m_ctx *c, const double *pos, const double *mom,
                                   const double *acc);
-cudaError_t launch_scatter_out(p3m_ctx *c, const double *src, double *dst);
-// inv[pid[k]] = k, then dst[j] = src[inv[j]] (3 x n): caller order with sequential writes
-cudaError_t launch_inverse_pid(p3m_ctx *c, uint32_t *inv);
-cudaError_t launch_gather_out(p3m_ctx *c, const double *src, const uint32_t *inv, double *dst);
+// dst[t] (caller order) = src[t] (slot order), 3 x n values each; uses pid_alt as scratch.  direct: host memory
+cudaError_t launch_outputs(p3m_ctx *c, const double *const *src, double *const *dst, int count,
+                           bool direct = false);
+inline cudaError_t launch_output(p3m_ctx *c, const double *src, double *dst) { return launch_outputs(c, &src, &dst, 1); }
 cudaError_t launch_diag(p3m_ctx *c, double *host_out /* [4]: px py pz 2*kinetic*m*a^2 */);
 
 // ------------------------------------------------------------------ launchers (adjoint.cu)

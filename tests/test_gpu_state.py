@@ -67,3 +67,34 @@ def test_sort_at_tile_edges(n, mesh, precision):
             assert abs(sim.diagnostics()["pairs"] - want) <= (4 if precision == "mixed" else 0)
             again = sim.forces(1.0)
         assert np.array_equal(first, again)
+
+
+@pytest.mark.parametrize("n", [5003, 900001, 3000001])
+@pytest.mark.parametrize("where", ["device", "pinned", "pageable"])
+def test_results_in_the_callers_order(n, where):
+    """Positions and momenta come back as they were given after a sort, whichever way they take (written in
+    place or through the inverse permutation, by size), and the accelerations do not depend on what else is
+    asked for."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1510_07621_gb300 import P3M, build
+    build.build()
+    gen = torch.Generator().manual_seed(n)
+    pos = torch.rand((3, n), generator=gen, dtype=torch.float64) * 100.0
+    mom = torch.randn((3, n), generator=gen, dtype=torch.float64)
+
+    def array():
+        a = torch.zeros((3, n), dtype=torch.float64)
+        return a.cuda() if where == "device" else a.pin_memory() if where == "pinned" else a
+
+    with P3M(100.0, n, 64, short_range=False) as sim:
+        sim.set_particles(pos, mom, a=1.0)
+        alone = array()
+        sim.forces(1.0, out=alone)
+        p, m, a, only = array(), array(), array(), array()
+        sim.get_particles(p, m, a)
+        sim.get_particles(None, only)
+        torch.cuda.synchronize()
+    assert torch.equal(p.cpu(), pos) and torch.equal(m.cpu(), mom) and torch.equal(only.cpu(), mom)
+    assert torch.equal(a.cpu(), alone.cpu())
