@@ -45,6 +45,35 @@ __device__ __forceinline__ void stencil64(double x, double inv_h, int &i0, doubl
     f = u - fl;
 }
 
+// The eight CIC nodes around a wrapped position and the fractions in its mesh cell.  Node indices lie in
+// [0, M], so one compare wraps them instead of a division.
+struct CicNodes {
+    size_t row[2][2];
+    int z[2];
+    double f[3];
+    __device__ __forceinline__ CicNodes(double x, double y, double zz, double inv_h, int M)
+    {
+        int i[3];
+        stencil64(x, inv_h, i[0], f[0]);
+        stencil64(y, inv_h, i[1], f[1]);
+        stencil64(zz, inv_h, i[2], f[2]);
+        int j[3][2];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            if ((unsigned)i[d] >= (unsigned)M) i[d] = 0;  // (x / h rounded up to M; a position that is NaN)
+            j[d][0] = i[d];
+            j[d][1] = i[d] + 1 == M ? 0 : i[d] + 1;
+        }
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) row[a][b] = ((size_t)j[0][a] * M + j[1][b]) * M;
+        z[0] = j[2][0];
+        z[1] = j[2][1];
+    }
+    __device__ __forceinline__ size_t node(int a, int b, int e) const { return row[a][b] + z[e]; }
+};
+
 // v_sorted[k] = v[pid[k]] (caller order -> slot order), also an FP32 copy with w = 0.
 __global__ void k_to_slots(const double *__restrict__ v, const uint32_t *__restrict__ pid,
                            int64_t n, double *__restrict__ vs, float *__restrict__ vfx)
@@ -103,36 +132,41 @@ __global__ void k_fix_exponent(const unsigned long long *__restrict__ maxbits, i
 }
 
 // u_b(node) += W(x_k - node) v_k,b as round(W v 2^S) on three fixed-point meshes.
+// Bound by the FP64 pipe (17 cycles per warp and instruction on an SM).  |W v 2^S| < 2^(61 - nb), so from
+// 2^10 particles on (nb > 10, kSmall false) the integer is in the low bits of fma(W, v 2^S, 1.5 2^52): one
+// instruction for a product and a conversion, the same rounding to even.  128^3: 0.316 -> 0.229 ms.
+template <bool kSmall>
 __global__ void k_deposit_vec(const double *__restrict__ pos, const double *__restrict__ v,
                               P3MGeom g, const int *__restrict__ s_dev,
                               unsigned long long *__restrict__ fix)
 {
+    constexpr double kBig = 0x1.8p52;
     const int M = g.mesh;
     const int64_t n = g.n;
     const size_t M3 = (size_t)M * M * M;
     const double scale = ldexp(1.0, *s_dev);
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
          k += (int64_t)gridDim.x * blockDim.x) {
-        int ix, iy, iz;
-        double fx, fy, fz;
-        stencil64(pos[k], g.inv_h, ix, fx);
-        stencil64(pos[n + k], g.inv_h, iy, fy);
-        stencil64(pos[2 * n + k], g.inv_h, iz, fz);
-        const double wx[2] = {1.0 - fx, fx}, wy[2] = {1.0 - fy, fy}, wz[2] = {1.0 - fz, fz};
+        const CicNodes c(pos[k], pos[n + k], pos[2 * n + k], g.inv_h, M);
+        const double wx[2] = {1.0 - c.f[0], c.f[0]}, wy[2] = {1.0 - c.f[1], c.f[1]}, wz[2] = {1.0 - c.f[2], c.f[2]};
         const double vb[3] = {v[k] * scale, v[n + k] * scale, v[2 * n + k] * scale};
 #pragma unroll
         for (int a = 0; a < 2; ++a)
 #pragma unroll
-            for (int b = 0; b < 2; ++b)
+            for (int b = 0; b < 2; ++b) {
+                const double wab = wx[a] * wy[b];
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const double w = wx[a] * wy[b] * wz[c];
-                    const size_t node = ((size_t)wrap_index(ix + a, M) * M + wrap_index(iy + b, M)) * M +
-                                        wrap_index(iz + c, M);
+                for (int e = 0; e < 2; ++e) {
+                    const double w = wab * wz[e];
+                    const size_t node = c.node(a, b, e);
 #pragma unroll
-                    for (int d = 0; d < 3; ++d)
-                        atomicAdd(fix + d * M3 + node, (unsigned long long)__double2ll_rn(w * vb[d]));
+                    for (int d = 0; d < 3; ++d) {
+                        const long long q = kSmall ? __double2ll_rn(w * vb[d])
+                                                   : __double_as_longlong(fma(w, vb[d], kBig)) - __double_as_longlong(kBig);
+                        atomicAdd(fix + d * M3 + node, (unsigned long long)q);
+                    }
                 }
+            }
     }
 }
 
@@ -174,8 +208,22 @@ __global__ void k_kspace_adjoint(const C2 *__restrict__ ux, const C2 *__restrict
     }
 }
 
+// A finite FP32 value as FP64 by integer operations: the conversion instruction runs on the FP64 pipe.
+__device__ __noinline__ double widen_special(float x) { return (double)x; }
+__device__ __forceinline__ double widen(float x)
+{
+    const uint32_t u = __float_as_uint(x);
+    // normal numbers; zero, denormal, infinite and NaN take the instruction
+    if (((u << 1) - 0x01000000u) >= 0xFE000000u) return widen_special(x);
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 // out_k += scale sum_corners grad W(x_k - node) [ sum_b v_k,b E_b(node) + psi(node) ]
 // (E or v NULL: no first term; psi NULL: no second term).
+// Bound by the FP64 pipe.  The gradient of the trilinear interpolant of the eight values by nested
+// differences and interpolations (21 FP64 operations where the sum over weights takes 72), and the FP32
+// meshes are widened by integer operations (32 values per particle): 128^3 0.563 -> 0.234 ms.
 template <typename T>
 __global__ void k_gather_grad(const double *__restrict__ pos, P3MGeom g, const T *__restrict__ E,
                               const double *__restrict__ v, const T *__restrict__ psi,
@@ -184,42 +232,43 @@ __global__ void k_gather_grad(const double *__restrict__ pos, P3MGeom g, const T
     const int M = g.mesh;
     const int64_t n = g.n;
     const size_t M3 = (size_t)M * M * M;
-    const double ih = g.inv_h;
+    const double factor = scale * g.inv_h;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
          k += (int64_t)gridDim.x * blockDim.x) {
-        int ix, iy, iz;
-        double fx, fy, fz;
-        stencil64(pos[k], ih, ix, fx);
-        stencil64(pos[n + k], ih, iy, fy);
-        stencil64(pos[2 * n + k], ih, iz, fz);
-        const double wx[2] = {1.0 - fx, fx}, wy[2] = {1.0 - fy, fy}, wz[2] = {1.0 - fz, fz};
-        const double dx[2] = {-ih, ih};
+        const CicNodes c(pos[k], pos[n + k], pos[2 * n + k], g.inv_h, M);
         double vb[3] = {0.0, 0.0, 0.0};
         if (E && v) {
             vb[0] = v[k];
             vb[1] = v[n + k];
             vb[2] = v[2 * n + k];
         }
-        double o0 = 0.0, o1 = 0.0, o2 = 0.0;
+        double dz[2][2], m[2][2];  // per edge along z: difference, and value at the particle
 #pragma unroll
         for (int a = 0; a < 2; ++a)
 #pragma unroll
-            for (int b = 0; b < 2; ++b)
+            for (int b = 0; b < 2; ++b) {
+                double s[2];
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const size_t node = ((size_t)wrap_index(ix + a, M) * M + wrap_index(iy + b, M)) * M +
-                                        wrap_index(iz + c, M);
-                    double s = psi ? (double)psi[node] : 0.0;
+                for (int e = 0; e < 2; ++e) {
+                    const size_t node = c.node(a, b, e);
+                    s[e] = psi ? widen(psi[node]) : 0.0;
                     if (E && v)
-                        s += vb[0] * (double)E[node] + vb[1] * (double)E[M3 + node] +
-                             vb[2] * (double)E[2 * M3 + node];
-                    o0 += dx[a] * wy[b] * wz[c] * s;
-                    o1 += wx[a] * dx[b] * wz[c] * s;
-                    o2 += wx[a] * wy[b] * dx[c] * s;
+                        s[e] = fma(vb[2], widen(E[2 * M3 + node]),
+                                   fma(vb[1], widen(E[M3 + node]), fma(vb[0], widen(E[node]), s[e])));
                 }
-        out[k] += scale * o0;
-        out[n + k] += scale * o1;
-        out[2 * n + k] += scale * o2;
+                dz[a][b] = s[1] - s[0];
+                m[a][b] = fma(c.f[2], dz[a][b], s[0]);
+            }
+        double q[2], dy[2], dzy[2];  // per edge along y, at the particle's z
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            dy[a] = m[a][1] - m[a][0];
+            q[a] = fma(c.f[1], dy[a], m[a][0]);
+            dzy[a] = fma(c.f[1], dz[a][1] - dz[a][0], dz[a][0]);
+        }
+        out[k] = fma(factor, q[1] - q[0], out[k]);
+        out[n + k] = fma(factor, fma(c.f[0], dy[1] - dy[0], dy[0]), out[n + k]);
+        out[2 * n + k] = fma(factor, fma(c.f[0], dzy[1] - dzy[0], dzy[0]), out[2 * n + k]);
     }
 }
 
@@ -908,7 +957,8 @@ cudaError_t vjp_mesh(p3m_ctx *c, const double *v_slots, double *out_slots)
     c->launches += 6;
     k_absmax_bits<<<gn, 256, 0, c->stream>>>(v_slots, 3 * c->g.n, maxbits);
     k_fix_exponent<<<1, 1, 0, c->stream>>>(maxbits, nb, c->fix_exp);
-    k_deposit_vec<<<gn, 256, 0, c->stream>>>(c->pos, v_slots, c->g, c->fix_exp, c->rho_fix);
+    auto deposit = nb <= 10 ? k_deposit_vec<true> : k_deposit_vec<false>;
+    deposit<<<gn, 256, 0, c->stream>>>(c->pos, v_slots, c->g, c->fix_exp, c->rho_fix);
     k_fix_to_vec<T><<<grid_for((int64_t)(3 * M3), 256, c->num_sms), 256, 0, c->stream>>>(c->rho_fix, 3 * M3,
                                                                                        c->fix_exp, u);
     C2 *uk = (C2 *)c->frc_k;
