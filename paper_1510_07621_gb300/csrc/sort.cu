@@ -648,7 +648,7 @@ __global__ void k_cell_start(const uint32_t *__restrict__ keys, P3MGeom g,
 // item a place in its class (their order within a class is arbitrary: results do not depend on it).  Two
 // kernels instead of a count, a scan, a fill and a radix pass with its memsets (ten launches and memsets):
 // 5003 particles 23 -> 8 us of kernels, clustered 128^3 (a thread wrote all items of a dense cell; now its
-// warp does) 55 -> 15 us.
+// warp does) 55 -> 12 us.
 
 struct WorkItems {
     uint32_t first, full, rest;  // first slot, items of 32, particles of the last item
@@ -662,13 +662,23 @@ __device__ __forceinline__ WorkItems work_items(const uint32_t *__restrict__ cel
     const uint32_t end = cell_start[c + 1];
     if (end <= w.first) return w;
     const int cx = c % n_c, cy = (c / n_c) % n_c, cz = c / (n_c * n_c);
-    float nb = 0.0f;
-    for (int oz = -1; oz <= 1; ++oz)
-        for (int oy = -1; oy <= 1; ++oy)
-            for (int ox = -1; ox <= 1; ++ox) {
-                const int q = (((cz + oz + n_c) % n_c) * n_c + (cy + oy + n_c) % n_c) * n_c + (cx + ox + n_c) % n_c;
-                nb += (float)(cell_start[q + 1] - cell_start[q]);
-            }
+    // rows of three cells along x are consecutive slots (a row that wraps: the rest of it)
+    uint32_t near = 0;
+#pragma unroll
+    for (int oz = -1; oz <= 1; ++oz) {
+        int z = cz + oz;
+        z += z < 0 ? n_c : (z >= n_c ? -n_c : 0);
+#pragma unroll
+        for (int oy = -1; oy <= 1; ++oy) {
+            int y = cy + oy;
+            y += y < 0 ? n_c : (y >= n_c ? -n_c : 0);
+            const uint32_t *row = cell_start + ((size_t)z * n_c + y) * n_c;
+            near += row[min(cx + 2, n_c)] - row[max(cx - 1, 0)];
+            if (cx == 0) near += row[n_c] - row[n_c - 1];
+            if (cx == n_c - 1) near += row[1] - row[0];
+        }
+    }
+    const float nb = (float)near;
     auto key = [&](uint32_t particles) {  // cost >= 1
         return 255u - min((__float_as_uint((float)particles * nb) >> 20) - (127u << 3), 255u);
     };
@@ -733,7 +743,7 @@ __global__ void __launch_bounds__(kThreads)
         work[at] = make_uint2((uint32_t)cell, slot);
         work_key[at] = key;
     };
-    constexpr uint32_t kOwn = 4;  // a lane's own cell up to this many items, more by the whole warp
+    constexpr uint32_t kOwn = 16;  // a lane's own cell up to this many items, more by the whole warp
     if (w.full <= kOwn)
         for (uint32_t i = 0; i < w.full; ++i) put(at_full + i, c, w.first + i * P3M_PAIR_TI, w.key_full);
     if (w.rest) put(at_rest, c, w.first + w.full * P3M_PAIR_TI, w.key_rest);
