@@ -430,7 +430,7 @@ __global__ void __launch_bounds__(32)
     }
 }
 
-// FP32 mode: the force kernel's lists (k_pairs_list in pair.cu: groups of 16 particles, candidates
+// FP32 mode: the force kernel's lists (k_pairs_list in pair.cu: groups of 16 particles (8 or 4 of few), candidates
 // tested one per lane against the group's box, the accepted ones compacted into a list, two particles
 // and two list entries per lane in packed f32x2 arithmetic), here with v beside the coordinates, for
 //   out_k += Gm sum_j [h w + (h'/r) (d.w) d],  w = v_j - v_k,
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(32)
 // mesh part: 9.35 -> 7.13 ms, the pair part 7.6 -> 5.4.  What bounds it: of 137 cycles per 32 accepted
 // pairs and scheduler, 111 are the evaluation (52 per 32 slots, 47 % of them accepted).  8 or 32
 // particles per group, 18 or 20 CTAs per SM and lists of 192 are within 2 % or slower.
-constexpr int kVjpGroup = 16, kVjpChunk = 128, kVjpFlush = 5;  // (16 FP32 terms per chunk and sum)
+constexpr int kVjpChunk = 128, kVjpTerms = 80;  // FP32 terms per partial sum before it joins the FP64 sum
 constexpr float kVjpTiny = 1e-24f, kVjpFar = 1e6f;
 
 struct VjpConst2 {
@@ -484,7 +484,7 @@ __device__ __forceinline__ f2 pair_jac2(f2 w, f2 dw, const VjpConst2 &k, f2 *c)
     return h;
 }
 
-template <bool kAdditive>
+template <bool kAdditive, int kG>
 __global__ void __launch_bounds__(32, 16)
     k_pairs_vjp_list(const uint32_t *__restrict__ relq, const float *__restrict__ vfx,
                      const float4 *__restrict__ block_box, const uint32_t *__restrict__ cell_start,
@@ -492,7 +492,8 @@ __global__ void __launch_bounds__(32, 16)
                      const uint32_t *__restrict__ n_work_ptr, P3MGeom g, PairFactor fac, double scale,
                      float rcull2, uint32_t *__restrict__ cursor, double *__restrict__ out)
 {
-    constexpr int kG = kVjpGroup, kPairsI = kG / 2, kStride = 2 * (32 / kPairsI), kSub = P3M_PAIR_TI / kG;
+    constexpr int kPairsI = kG / 2, kStride = 2 * (32 / kPairsI), kSub = P3M_PAIR_TI / kG;
+    constexpr int kVjpFlush = kVjpTerms * kStride / kVjpChunk;
     __shared__ __align__(16) float list[6][kVjpChunk + 32];  // x, y, z, vx, vy, vz
     __shared__ uint32_t slot[kVjpChunk + 32];                // the sorted slot of each list entry
     __shared__ double sum[6][32];
@@ -987,7 +988,11 @@ cudaError_t vjp_pairs(p3m_ctx *c, const double *v_slots, double *out_slots)
 {
     int per_sm = 0;
     const bool fp32 = c->precision == P3M_PREC_MIXED;
-    auto list = c->pair_factor.additive ? k_pairs_vjp_list<true> : k_pairs_vjp_list<false>;
+    const int group = pair_group(c);
+    const bool add = c->pair_factor.additive != 0;
+    auto list = group == 4   ? (add ? k_pairs_vjp_list<true, 4> : k_pairs_vjp_list<false, 4>)
+                : group == 8 ? (add ? k_pairs_vjp_list<true, 8> : k_pairs_vjp_list<false, 8>)
+                             : (add ? k_pairs_vjp_list<true, 16> : k_pairs_vjp_list<false, 16>);
     cudaError_t e = fp32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, list, 32, 0)
                          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pairs_vjp64, 32, 0);
     if (e != cudaSuccess) return e;

@@ -201,10 +201,19 @@ enum {
 #define P3M_SORT_SMALL 262144
 #define P3M_SORT_HIST_BYTES (4 * (4 * 256 + 4))
 #define P3M_PAIR_TI 32       // i-particles per pair work item (one per lane of a warp)
-#define P3M_PAIR_GROUP 16    // particles of a work item that share one list (FP32 kernel)
 #define P3M_PAIR_CTAS 18     // one-warp CTAs per SM that the FP32 kernel's registers leave room for
 #define P3M_COUNTERS (4 + 256 + 1 + 256)  // 32-bit words of counters
 #define P3M_FLAG_TIMEOUT 1u  // counters[1] bit: a bounded wait gave up
+
+// Particles that share one list of the FP32 pair kernels: the most of 16, 8 and 4 that gives every resident
+// warp a group (smaller lists cost more tests per pair, but a group is the least a warp can take: few
+// particles leave most warps without one).  Force kernel, 16 / 8 / 4: 17^3 particles 77 / 51 / 40 us, 24^3
+// 107 / 69 / 70, 32^3 109 / 95 / 119 (clustered 310 / 197 / 213), 40^3 143 / 150, 64^3 445 / 514.
+inline int pair_group(const p3m_ctx *c)
+{
+    const int64_t warps = (int64_t)c->num_sms * P3M_PAIR_CTAS;
+    return c->g.n >= 16 * warps ? 16 : c->g.n >= 8 * warps ? 8 : 4;
+}
 
 // Everything the FP32 pair kernel needs from one context: its arrays, geometry, fitted split
 // factor and culling radii, where the accelerations go and the fused final half-kick (factor
@@ -224,7 +233,8 @@ struct PairArgs {
     double kfac;
     P3MGeom g;
     PairFactor fac;
-    float rcull2, pad;
+    float rcull2;
+    int group;  // particles per list (pair_group)
 };
 
 #define P3M_FLAG_NONFINITE 2u

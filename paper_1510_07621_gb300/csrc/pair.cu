@@ -23,7 +23,6 @@ namespace {
 
 constexpr int kLongChunk = 5;   // FP32 kernel: the list is evaluated every 160 entries
 constexpr int kShortChunk = 3;  // the autotuner's other choice
-constexpr int kGroup = P3M_PAIR_GROUP;
 
 // x^-1/2: the hardware's approximation (relative error e0 / 2 below 2^-20) and one step of the
 // third-order iteration y (1 + e/2 + 3 e^2/8), e = 1 - x y^2, whose error 5/16 e^3 is below 2^-58.
@@ -235,8 +234,9 @@ __global__ void __launch_bounds__(32)
 }
 
 // ------------------------------------------------------------------ FP32 mode, compacted j lists
-// The FP32 kernel.  A work item's up to 32 particles are taken in groups of kG (consecutive along
-// the Hilbert order inside the cell, so compact), one group at a time per one-warp CTA:
+// The FP32 kernel.  A work item's up to 32 particles are taken in groups of kG = 16 (8 or 4 when there
+// are few, see pair_group; consecutive along the Hilbert order inside the cell, so compact), one group
+// at a time per one-warp CTA:
 //   1. The neighbour cells form 9 rows of 3 along x, each a contiguous range of sorted slots (two
 //      ranges where a row wraps).  The rows' 32-slot blocks are tested 32 at a time, one per lane,
 //      against the group's bounding box (block_box, padded by more than its FP32 rounding).
@@ -251,9 +251,9 @@ __global__ void __launch_bounds__(32)
 // instructions were tests and votes.  The list holds 47 % accepted slots at kG = 16 (58 % at 8,
 // 39 % at 32: the union of the cutoff spheres grows with the group), there are no votes between
 // pairs, and a test sequence serves 32 candidates of the whole group.  Measured at 128^3 (one
-// evaluation, before / after): near-uniform 5.23 / 3.21 ms, clustered 12.3 / 9.6 ms.
-// What bounds it now: of 83 cycles per 32 accepted pairs and scheduler, 58 are the evaluation
-// (27 per 32 slots; two FP32 operations with three distinct registers already take three cycles
+// evaluation, before / after): near-uniform 5.23 / 3.27 ms, clustered 12.3 / 9.8 ms.
+// What bounds it now: of 84 cycles per 32 accepted pairs and scheduler, 59 are the evaluation
+// (28 per 32 slots; two FP32 operations with three distinct registers already take three cycles
 // of register bandwidth, and the same mix of 16 packed operations, 2 rsqrt and 2 ex2 alone runs
 // at 20.5), 19 the candidate tests and 6 the set-up of groups.  16 particles per group
 // and 18 CTAs per SM: 8, 32 and 16, 20, 24 are within 6 % or slower on both sets.  Two lists of 16 (or
@@ -314,11 +314,7 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
     constexpr int kArgWords = sizeof(PairArgs) / 8;
     static_assert(sizeof(PairArgs) % 8 == 0, "PairArgs is copied in 8-byte words");
     constexpr int kChunk = 32 * kChunkBlocks, kCap = kChunk + 32;
-    constexpr int kPairsI = kG / 2;        // lanes that share one list entry
-    constexpr int kStride = 2 * (32 / kPairsI);  // list entries per warp step
     constexpr int kSub = P3M_PAIR_TI / kG;
-    constexpr int kFlushChunks = kFlushTerms * kStride / kChunk < 1 ? 1 : kFlushTerms * kStride / kChunk;
-    static_assert(kChunk % kStride == 0, "whole steps per chunk");
     __shared__ __align__(16) float list[3][kCap];
     __shared__ uint32_t slot[kCap];  // the sorted slot of each list entry
     __shared__ double sum[6][32];  // per lane: x, y, z of its first particle, then of its second
@@ -331,7 +327,6 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
     const int lane = threadIdx.x;
     const uint32_t lt = (1u << lane) - 1u;
     const uint32_t n_units = *n_work_ptr * kSub;
-    const int ip = lane % kPairsI, js = lane / kPairsI;
     int cur_sim = -1;
     double kfac = 0.0;
     PairConstQ kc;
@@ -361,31 +356,19 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
     };
     if (!kBatched) load_args(&a0);
 
-    for (;;) {
-        uint32_t unit = 0;
-        if (lane == 0) unit = atomicAdd(cursor, 1u);
-        unit = __shfl_sync(0xffffffffu, unit, 0);
-        if (unit >= n_units) break;
-        uint32_t item = kBatched ? order[unit / kSub] : unit / kSub;
-        if (kBatched) {
-            const int sim = (int)(item >> 24);
-            item &= 0xFFFFFFu;
-            if (sim != cur_sim) {
-                if (cur_sim >= 0) store_stat();
-                load_args(descs + sim);
-                cur_sim = sim;
-            }
-        }
+    // the group of up to kN particles of `cell` from slot `first` on
+    auto group = [&](auto size, uint32_t cell, uint32_t first, uint32_t cend) {
+        constexpr int kN = decltype(size)::value;
+        constexpr int kPairsI = kN / 2;              // lanes that share one list entry
+        constexpr int kStride = 2 * (32 / kPairsI);  // list entries per warp step
+        constexpr int kFlushChunks = kFlushTerms * kStride / kChunk < 1 ? 1 : kFlushTerms * kStride / kChunk;
+        static_assert(kChunk % kStride == 0, "whole steps per chunk");
         const P3MGeom &g = A.g;
         const int64_t n = g.n;
         const int nc = g.n_c;
-        const uint32_t cell = A.work[2 * (size_t)item];
-        const uint32_t first = A.work[2 * (size_t)item + 1] + (unit % kSub) * kG;
-        const uint32_t cend = A.cell_start[cell + 1];
-        if (first >= cend) continue;
+        const int ip = lane % kPairsI, js = lane / kPairsI;
         const int cx = (int)(cell % nc), cy = (int)((cell / nc) % nc), cz = (int)(cell / (nc * nc));
-
-        const GroupFrame fr = group_frame<kG>(A.relq, first, cend, cx, cy, cz, A.fac.lambda, A.fac.cell);
+        const GroupFrame fr = group_frame<kN>(A.relq, first, cend, cx, cy, cz, A.fac.lambda, A.fac.cell);
         const uint2 blocks = group_ranges(seg, A.cell_start, g, cx, cy, cz, fr, A.fac.cell);
         const float hx = fr.half[0], hy = fr.half[1], hz = fr.half[2];
 #pragma unroll
@@ -557,8 +540,8 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
         const double *__restrict__ acc_in = A.acc_in;
         double *__restrict__ acc_out = A.acc_out;
         double *__restrict__ mom = A.mom;
-        for (int t = lane; t < 3 * kG; t += 32) {
-            const int d = t / kG, k = t % kG;
+        for (int t = lane; t < 3 * kN; t += 32) {
+            const int d = t / kN, k = t % kN;
             const uint32_t i = first + k;
             if (i >= cend) continue;
             double s = 0.0;
@@ -573,12 +556,45 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
         const uint32_t pairs = __reduce_add_sync(0xffffffffu, my);
         if (lane == 0) {
             stat[0] += pairs;
-            stat[1] += (n_live * kG);              // j's tested against the group's box, in slots of 32
-            stat[2] += (n_list * kG + 16) / 32;    // list entries evaluated, the same
+            stat[1] += (n_live * kN);              // j's tested against the group's box, in slots of 32
+            stat[2] += (n_list * kN + 16) / 32;    // list entries evaluated, the same
             stat[3] += blocks.y - n_live;
             stat[4] += n_chunks + 2;
         }
         __syncwarp();
+    };
+
+    for (;;) {
+        uint32_t unit = 0;
+        if (lane == 0) unit = atomicAdd(cursor, 1u);
+        unit = __shfl_sync(0xffffffffu, unit, 0);
+        if (unit >= n_units) break;
+        uint32_t item = kBatched ? order[unit / kSub] : unit / kSub;
+        if (kBatched) {
+            const int sim = (int)(item >> 24);
+            item &= 0xFFFFFFu;
+            if (sim != cur_sim) {
+                if (cur_sim >= 0) store_stat();
+                load_args(descs + sim);
+                cur_sim = sim;
+            }
+        }
+        const uint32_t cell = A.work[2 * (size_t)item];
+        const uint32_t first = A.work[2 * (size_t)item + 1] + (unit % kSub) * kG;
+        const uint32_t cend = A.cell_start[cell + 1];
+        if (first >= cend) continue;
+        if (!kBatched) {
+            group(std::integral_constant<int, kG>{}, cell, first, cend);
+            continue;
+        }
+        // each context's own group size, so that its sums are those of a launch of its own
+        const uint32_t end = min(first + kG, cend);
+        if (A.group == 4)
+            for (uint32_t f = first; f < end; f += 4) group(std::integral_constant<int, 4>{}, cell, f, cend);
+        else if (A.group == 8)
+            for (uint32_t f = first; f < end; f += 8) group(std::integral_constant<int, 8>{}, cell, f, cend);
+        else
+            group(std::integral_constant<int, kG>{}, cell, first, cend);
     }
     if (!kBatched || cur_sim >= 0) store_stat();
 }
@@ -606,12 +622,12 @@ cudaError_t pairs64_impl(p3m_ctx *c, const double *acc_in, double *acc_out, doub
 }
 
 // The FP32 kernel for one context or (batched) several.
-template <bool kBatched, int kForm, int kChunkBlocks>
+template <bool kBatched, int kForm, int kChunkBlocks, int kG>
 cudaError_t launch_list(const PairArgs &a, const PairArgs *descs, const uint32_t *order,
                         const uint32_t *n_work, uint32_t *cursor, int num_sms, cudaStream_t s)
 {
     int per_sm = 0;
-    auto kern = k_pairs_list<kBatched, kForm, kChunkBlocks, kGroup>;
+    auto kern = k_pairs_list<kBatched, kForm, kChunkBlocks, kG>;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32, 0);
     if (e != cudaSuccess) return e;
     kern<<<num_sms * (per_sm < 1 ? 1 : per_sm), 32, 0, s>>>(a, descs, order, n_work, cursor);
@@ -626,8 +642,12 @@ cudaError_t pairs_list_impl(p3m_ctx *c, const double *acc_in, double *acc_out, d
     c->launches += 1;
     const PairArgs a = pair_args(c, acc_in, acc_out, kfac, kfac_dev);
     const bool add = c->pair_factor.additive != 0;
-    auto launch = c->tile_blocks == kShortChunk ? (add ? launch_list<false, 1, kShortChunk> : launch_list<false, 0, kShortChunk>)
-                                                : (add ? launch_list<false, 1, kLongChunk> : launch_list<false, 0, kLongChunk>);
+    const int group = pair_group(c);
+    auto launch = group == 4   ? (add ? launch_list<false, 1, kLongChunk, 4> : launch_list<false, 0, kLongChunk, 4>)
+                  : group == 8 ? (add ? launch_list<false, 1, kLongChunk, 8> : launch_list<false, 0, kLongChunk, 8>)
+                  : c->tile_blocks == kShortChunk
+                      ? (add ? launch_list<false, 1, kShortChunk, 16> : launch_list<false, 0, kShortChunk, 16>)
+                      : (add ? launch_list<false, 1, kLongChunk, 16> : launch_list<false, 0, kLongChunk, 16>);
     return launch(a, nullptr, nullptr, c->n_work, c->counters, c->num_sms, c->stream);
 }
 
@@ -674,6 +694,7 @@ PairArgs pair_args(const p3m_ctx *c, const double *acc_in, double *acc_out, doub
     // box size
     const double rcull = c->g.r_c * (1.0 + 1e-4) + c->g.box * 1e-6;
     a.rcull2 = (float)(rcull * rcull);
+    a.group = pair_group(c);
     return a;
 }
 
@@ -685,7 +706,7 @@ cudaError_t launch_pairs_batched(const PairArgs *descs, const uint32_t *order,
     if (e != cudaSuccess) return e;
     PairArgs unused;
     memset(&unused, 0, sizeof(unused));
-    return launch_list<true, 2, kLongChunk>(unused, descs, order, n_total, cursor, num_sms, s);
+    return launch_list<true, 2, kLongChunk, 16>(unused, descs, order, n_total, cursor, num_sms, s);
 }
 
 cudaError_t launch_store_pair_args(PairArgs *dst, const PairArgs &a, cudaStream_t s)

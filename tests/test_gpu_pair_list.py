@@ -154,3 +154,61 @@ def test_cutoff_decided_exactly(box, mesh, cutoff, softening, off):
     assert got["mixed"][2] == got["fp64"][2] == 2 * int((side < 0).sum())
     for a, b in zip(got["mixed"][:2], got["fp64"][:2]):
         assert np.abs(a - b).max() <= 1e-4 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("fraction", [0.499, 0.5, 0.51, 0.999, 1.0, 1.1])
+@pytest.mark.parametrize("kind,softening", [("uniform", 0.02), ("cell", 0.3)])
+def test_list_group_sizes(fraction, kind, softening):
+    """Lists of 4, 8 and 16 particles on both sides of the particle numbers where they change (as fractions of
+    16 particles per resident warp), against the FP64 kernel: 1e-5 relative RMS of the short-range force and
+    2e-5 of the VJP, the FP32 bars, and the same pairs (their coordinates' rounding, 1e-9 of the cutoff, may
+    move one in 10^8)."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1510_07621_gb300 import P3M, build
+    build.build()
+    n = int(16 * 18 * torch.cuda.get_device_properties(0).multi_processor_count * fraction)
+    box, mesh = 60.0, 40
+    x = np.mod(S.uniform_random(n, box, 17), box)
+    if kind == "cell":
+        m = n // 40
+        x[:, :m] = 0.45 * box + 0.02 * box * S.uniform_random(m, 1.0, 18)
+    v = np.random.default_rng(1).normal(size=x.shape)
+    got = {}
+    for precision in ("mixed", "fp64"):
+        with P3M(box, n, mesh, softening=softening, precision=precision) as sim:
+            sim.set_particles(x, np.zeros_like(x), a=1.0)
+            _, sr = sim.forces_split()
+            got[precision] = sr, sim.diagnostics()["pairs"], sim.force_vjp(v)
+    (a, na, va), (b, nb, vb) = got["mixed"], got["fp64"]
+    assert abs(na - nb) <= max(4, 2e-8 * nb)
+    assert math.sqrt(float(np.sum((a - b) ** 2))) <= 1e-5 * math.sqrt(float(np.sum(b ** 2)))
+    assert math.sqrt(float(np.sum((va - vb) ** 2))) <= 2e-5 * math.sqrt(float(np.sum(vb ** 2)))
+
+
+def test_ensemble_members_keep_their_group_size():
+    """Simulations whose lists have 4, 8 and 16 particles, advanced together and alone: the same bits."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1510_07621_gb300 import P3M, Ensemble, build
+    build.build()
+    a = S.log_spaced_steps(0.05, 0.08, 3)
+    sets = [(p, *S.zeldovich(p, 60.0, a[0], 5 + p)) for p in (17, 30, 40, 21)]
+    alone = []
+    for p, pos, mom in sets:
+        with P3M(60.0, p ** 3, max(20, p + p % 2), softening=0.02, stream=0) as sim:
+            sim.set_particles(pos, mom, a=a[0])
+            for k in range(3):
+                sim.step(a[k], a[k + 1] - a[k])
+            alone.append(sim.get_particles())
+    sims = [P3M(60.0, p ** 3, max(20, p + p % 2), softening=0.02, stream=0) for p, _, _ in sets]
+    for sim, (_, pos, mom) in zip(sims, sets):
+        sim.set_particles(pos, mom, a=a[0])
+    with Ensemble(sims) as ens:
+        ens.run(a)
+    for sim, (pos, mom) in zip(sims, alone):
+        got = sim.get_particles()
+        assert np.array_equal(got[0], pos) and np.array_equal(got[1], mom)
+        sim.close()
