@@ -233,8 +233,9 @@ struct PairArgs {
     double kfac;
     P3MGeom g;
     PairFactor fac;
-    float rcull2;
+    float rcull2, rin2;
     int group;  // particles per list (pair_group)
+    int pad;
 };
 
 #define P3M_FLAG_NONFINITE 2u

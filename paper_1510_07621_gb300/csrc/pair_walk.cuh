@@ -105,7 +105,7 @@ __device__ __forceinline__ uint2 group_ranges(PairSeg *seg, const uint32_t *cell
 }
 
 // A surviving block: (range << 26) | block, the group's centre in its image, and its slots that belong
-// to the range.
+// to the range.  kDeepBlock in the word: all 32 slots do, and all are within the cutoff of all of the group.
 struct __align__(16) LiveBlock {
     uint32_t word, cx, cy, cz;
 };
@@ -113,15 +113,16 @@ struct LiveBlocks {
     LiveBlock at[32];
     uint32_t slots[32];
 };
-constexpr uint32_t kBlockMask = 0x3FFFFFFu;
+constexpr uint32_t kBlockMask = 0x3FFFFFFu, kDeepBlock = 0x80000000u;
 
 // Tests block t of the ranges in sequence (t >= t1: none) against the group's box; the survivors of
 // the warp's 32 blocks go to live[0 ..] in order.  Returns their number.
+// rin2: the squared cutoff less the same margins (no deep blocks if negative).
 // length: one scaled length (as in f.half); rcull2: the squared cutoff, padded by more than the FP32
 // rounding of absolute coordinates.
 __device__ __forceinline__ int live_blocks(uint32_t t, uint32_t t1, const PairSeg *seg,
                                            const float4 *block_box, const GroupFrame &f, float length,
-                                           float rcull2, LiveBlocks &live)
+                                           float rcull2, LiveBlocks &live, float rin2 = -1.0f)
 {
     const int lane = threadIdx.x & 31;
     bool keep = false;
@@ -142,6 +143,10 @@ __device__ __forceinline__ int live_blocks(uint32_t t, uint32_t t1, const PairSe
         const uint32_t j0 = max(b * 32, S.start) - b * 32, j1 = min(S.end - b * 32, 32u);
         slots = (0xffffffffu << j0) & (0xffffffffu >> (32 - j1));  // (0 <= j0 < j1 <= 32)
         q = {((uint32_t)s << 26) | b, S.cx, S.cy, S.cz};
+        const float mx = fmaxf(hi.x - S.ax, S.ax - lo.x) + f.half[0] * length,
+                    my = fmaxf(hi.y - S.ay, S.ay - lo.y) + f.half[1] * length,
+                    mz = fmaxf(hi.z - S.az, S.az - lo.z) + f.half[2] * length;
+        if (slots == 0xffffffffu && mx * mx + my * my + mz * mz < rin2) q.word |= kDeepBlock;
     }
     const uint32_t m = __ballot_sync(0xffffffffu, keep);
     __syncwarp();  // every lane is done with the previous survivors
