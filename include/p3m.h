@@ -217,14 +217,15 @@ int p3m_ensemble_create(p3m_ensemble **ens, p3m_ctx *const *ctxs, int n_ctx, int
 int p3m_ensemble_run(p3m_ensemble *ens, const double *a_list, int n_steps, int use_graph);
 void p3m_ensemble_free(p3m_ensemble *ens);
 /*
- * Batched pair launch (off by default; enable != 0 turns it on when at least one context is an
- * FP32 P3M context): each step runs the contexts' phases up to the mesh force as parallel
- * branches, then merges their pair work lists into one list sorted by estimated cost and
- * evaluates every such context's pair sum in one persistent kernel launch (the contexts'
+ * Batched pair launch (off by default; enable != 0 turns it on when at least one context
+ * qualifies: FP32 P3M, a softening small against r_s, and as many particles per list as most of
+ * the ensemble's particles have): each step runs the contexts' phases up to the mesh force as
+ * parallel branches, then merges the pair work lists of those that qualify into one list sorted
+ * by estimated cost and evaluates their pair sums in one persistent kernel launch (the contexts'
  * arguments read from a device table).  Other contexts step as before.  Results equal the
  * per-context launches bit for bit.  Every step then waits for all contexts' mesh phases
- * before the pair launch; on the 48-simulation ensemble of 48^3..96^3 particles the two are
- * within 1 % of each other with graphs.  enable = 0 returns to per-context pair launches.
+ * before the pair launch; on the 48-simulation ensemble of 48^3..96^3 particles it is 5 %
+ * slower than per-context launches with graphs.  enable = 0 returns to per-context pair launches.
  */
 int p3m_ensemble_set_batched(p3m_ensemble *ens, int enable);
 /*

@@ -234,8 +234,6 @@ struct PairArgs {
     P3MGeom g;
     PairFactor fac;
     float rcull2, rin2;
-    int group;  // particles per list (pair_group)
-    int pad;
 };
 
 #define P3M_FLAG_NONFINITE 2u
@@ -273,8 +271,9 @@ PairArgs pair_args(const p3m_ctx *c, const double *acc_in, double *acc_out, doub
                    const double *kfac_dev);
 // One pair launch over the work items of several FP32 contexts: order[k] = (sim << 24) | item,
 // sorted by cost; *n_total items; descs[sim] the contexts' arguments; cursor zeroed here.
+// group: the contexts' common group size; all have the additive factor.
 cudaError_t launch_pairs_batched(const PairArgs *descs, const uint32_t *order,
-                                 const uint32_t *n_total, uint32_t *cursor, int num_sms,
+                                 const uint32_t *n_total, uint32_t *cursor, int group, int num_sms,
                                  cudaStream_t s);
 // dst (device) = a, as one kernel (so that captured graphs write the current pointers).
 cudaError_t launch_store_pair_args(PairArgs *dst, const PairArgs &a, cudaStream_t s);

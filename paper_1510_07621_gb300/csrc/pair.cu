@@ -308,8 +308,8 @@ __device__ __forceinline__ f2 pair_factor_q(f2 w, const PairConstQ &k)
     return f2_mul(f2_mul(gv, s), f2_mul(s, s));
 }
 
-// kForm: 1 the additive factor, 0 the general one, 2 each context's own (batched launches)
-template <bool kBatched, int kForm, int kChunkBlocks, int kG>
+// kAdditive: the form of the pair factor; kG: particles of a group
+template <bool kBatched, bool kAdditive, int kChunkBlocks, int kG>
 __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
     k_pairs_list(PairArgs a0, const PairArgs *__restrict__ descs, const uint32_t *__restrict__ order,
                  const uint32_t *__restrict__ n_work_ptr, uint32_t *__restrict__ cursor)
@@ -317,7 +317,11 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
     constexpr int kArgWords = sizeof(PairArgs) / 8;
     static_assert(sizeof(PairArgs) % 8 == 0, "PairArgs is copied in 8-byte words");
     constexpr int kChunk = 32 * kChunkBlocks, kCap = kChunk + 32;
+    constexpr int kPairsI = kG / 2;              // lanes that share one list entry
+    constexpr int kStride = 2 * (32 / kPairsI);  // list entries per warp step
     constexpr int kSub = P3M_PAIR_TI / kG;
+    constexpr int kFlushChunks = kFlushTerms * kStride / kChunk < 1 ? 1 : kFlushTerms * kStride / kChunk;
+    static_assert(kChunk % kStride == 0, "whole steps per chunk");
     __shared__ __align__(16) float list[3][kCap];
     __shared__ uint32_t slot[kCap];  // the sorted slot of each list entry
     __shared__ __align__(16) float deep[3][kChunk];  // entries within the cutoff of the whole group
@@ -331,6 +335,7 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
     const int lane = threadIdx.x;
     const uint32_t lt = (1u << lane) - 1u;
     const uint32_t n_units = *n_work_ptr * kSub;
+    const int ip = lane % kPairsI, js = lane / kPairsI;
     int cur_sim = -1;
     double kfac = 0.0;
     PairConstQ kc;
@@ -360,19 +365,31 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
     };
     if (!kBatched) load_args(&a0);
 
-    // the group of up to kN particles of `cell` from slot `first` on
-    auto group = [&](auto size, uint32_t cell, uint32_t first, uint32_t cend) {
-        constexpr int kN = decltype(size)::value;
-        constexpr int kPairsI = kN / 2;              // lanes that share one list entry
-        constexpr int kStride = 2 * (32 / kPairsI);  // list entries per warp step
-        constexpr int kFlushChunks = kFlushTerms * kStride / kChunk < 1 ? 1 : kFlushTerms * kStride / kChunk;
-        static_assert(kChunk % kStride == 0, "whole steps per chunk");
+    for (;;) {
+        uint32_t unit = 0;
+        if (lane == 0) unit = atomicAdd(cursor, 1u);
+        unit = __shfl_sync(0xffffffffu, unit, 0);
+        if (unit >= n_units) break;
+        uint32_t item = kBatched ? order[unit / kSub] : unit / kSub;
+        if (kBatched) {
+            const int sim = (int)(item >> 24);
+            item &= 0xFFFFFFu;
+            if (sim != cur_sim) {
+                if (cur_sim >= 0) store_stat();
+                load_args(descs + sim);
+                cur_sim = sim;
+            }
+        }
         const P3MGeom &g = A.g;
         const int64_t n = g.n;
         const int nc = g.n_c;
-        const int ip = lane % kPairsI, js = lane / kPairsI;
+        const uint32_t cell = A.work[2 * (size_t)item];
+        const uint32_t first = A.work[2 * (size_t)item + 1] + (unit % kSub) * kG;
+        const uint32_t cend = A.cell_start[cell + 1];
+        if (first >= cend) continue;
         const int cx = (int)(cell % nc), cy = (int)((cell / nc) % nc), cz = (int)(cell / (nc * nc));
-        const GroupFrame fr = group_frame<kN>(A.relq, first, cend, cx, cy, cz, A.fac.lambda, A.fac.cell);
+
+        const GroupFrame fr = group_frame<kG>(A.relq, first, cend, cx, cy, cz, A.fac.lambda, A.fac.cell);
         const uint2 blocks = group_ranges(seg, A.cell_start, g, cx, cy, cz, fr, A.fac.cell);
         const float hx = fr.half[0], hy = fr.half[1], hz = fr.half[2];
 #pragma unroll
@@ -498,18 +515,8 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
                 cnt[1] += 2 * count / kStride;
             }
         };
-        auto eval = [&](auto own, int count) {
-            if (kForm == 1 || (kForm == 2 && A.fac.additive))
-                eval_form(std::true_type{}, own, count);
-            else
-                eval_form(std::false_type{}, own, count);
-        };
-        auto eval_deep = [&](auto own, int count) {
-            if (kForm == 1 || (kForm == 2 && A.fac.additive))
-                deep_form(std::true_type{}, own, count);
-            else
-                deep_form(std::false_type{}, own, count);
-        };
+        auto eval = [&](auto own, int count) { eval_form(std::bool_constant<kAdditive>{}, own, count); };
+        auto eval_deep = [&](auto own, int count) { deep_form(std::bool_constant<kAdditive>{}, own, count); };
 
         uint32_t n_list = 0, n_live = 0, n_chunks = 0;
         int fill = 0, fill_deep = 0;
@@ -596,8 +603,8 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
         const double *__restrict__ acc_in = A.acc_in;
         double *__restrict__ acc_out = A.acc_out;
         double *__restrict__ mom = A.mom;
-        for (int t = lane; t < 3 * kN; t += 32) {
-            const int d = t / kN, k = t % kN;
+        for (int t = lane; t < 3 * kG; t += 32) {
+            const int d = t / kG, k = t % kG;
             const uint32_t i = first + k;
             if (i >= cend) continue;
             double s = 0.0;
@@ -612,45 +619,12 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
         const uint32_t pairs = __reduce_add_sync(0xffffffffu, my);
         if (lane == 0) {
             stat[0] += pairs;
-            stat[1] += (n_live * kN);              // j's tested against the group's box, in slots of 32
-            stat[2] += (n_list * kN + 16) / 32;    // list entries evaluated, the same
+            stat[1] += (n_live * kG);              // j's tested against the group's box, in slots of 32
+            stat[2] += (n_list * kG + 16) / 32;    // list entries evaluated, the same
             stat[3] += blocks.y - n_live;
             stat[4] += n_chunks + 2;
         }
         __syncwarp();
-    };
-
-    for (;;) {
-        uint32_t unit = 0;
-        if (lane == 0) unit = atomicAdd(cursor, 1u);
-        unit = __shfl_sync(0xffffffffu, unit, 0);
-        if (unit >= n_units) break;
-        uint32_t item = kBatched ? order[unit / kSub] : unit / kSub;
-        if (kBatched) {
-            const int sim = (int)(item >> 24);
-            item &= 0xFFFFFFu;
-            if (sim != cur_sim) {
-                if (cur_sim >= 0) store_stat();
-                load_args(descs + sim);
-                cur_sim = sim;
-            }
-        }
-        const uint32_t cell = A.work[2 * (size_t)item];
-        const uint32_t first = A.work[2 * (size_t)item + 1] + (unit % kSub) * kG;
-        const uint32_t cend = A.cell_start[cell + 1];
-        if (first >= cend) continue;
-        if (!kBatched) {
-            group(std::integral_constant<int, kG>{}, cell, first, cend);
-            continue;
-        }
-        // each context's own group size, so that its sums are those of a launch of its own
-        const uint32_t end = min(first + kG, cend);
-        if (A.group == 4)
-            for (uint32_t f = first; f < end; f += 4) group(std::integral_constant<int, 4>{}, cell, f, cend);
-        else if (A.group == 8)
-            for (uint32_t f = first; f < end; f += 8) group(std::integral_constant<int, 8>{}, cell, f, cend);
-        else
-            group(std::integral_constant<int, kG>{}, cell, first, cend);
     }
     if (!kBatched || cur_sim >= 0) store_stat();
 }
@@ -678,12 +652,12 @@ cudaError_t pairs64_impl(p3m_ctx *c, const double *acc_in, double *acc_out, doub
 }
 
 // The FP32 kernel for one context or (batched) several.
-template <bool kBatched, int kForm, int kChunkBlocks, int kG>
+template <bool kBatched, bool kAdditive, int kChunkBlocks, int kG>
 cudaError_t launch_list(const PairArgs &a, const PairArgs *descs, const uint32_t *order,
                         const uint32_t *n_work, uint32_t *cursor, int num_sms, cudaStream_t s)
 {
     int per_sm = 0;
-    auto kern = k_pairs_list<kBatched, kForm, kChunkBlocks, kG>;
+    auto kern = k_pairs_list<kBatched, kAdditive, kChunkBlocks, kG>;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32, 0);
     if (e != cudaSuccess) return e;
     kern<<<num_sms * (per_sm < 1 ? 1 : per_sm), 32, 0, s>>>(a, descs, order, n_work, cursor);
@@ -699,11 +673,11 @@ cudaError_t pairs_list_impl(p3m_ctx *c, const double *acc_in, double *acc_out, d
     const PairArgs a = pair_args(c, acc_in, acc_out, kfac, kfac_dev);
     const bool add = c->pair_factor.additive != 0;
     const int group = pair_group(c);
-    auto launch = group == 4   ? (add ? launch_list<false, 1, kLongChunk, 4> : launch_list<false, 0, kLongChunk, 4>)
-                  : group == 8 ? (add ? launch_list<false, 1, kLongChunk, 8> : launch_list<false, 0, kLongChunk, 8>)
+    auto launch = group == 4   ? (add ? launch_list<false, true, kLongChunk, 4> : launch_list<false, false, kLongChunk, 4>)
+                  : group == 8 ? (add ? launch_list<false, true, kLongChunk, 8> : launch_list<false, false, kLongChunk, 8>)
                   : c->tile_blocks == kShortChunk
-                      ? (add ? launch_list<false, 1, kShortChunk, 16> : launch_list<false, 0, kShortChunk, 16>)
-                      : (add ? launch_list<false, 1, kLongChunk, 16> : launch_list<false, 0, kLongChunk, 16>);
+                      ? (add ? launch_list<false, true, kShortChunk, 16> : launch_list<false, false, kShortChunk, 16>)
+                      : (add ? launch_list<false, true, kLongChunk, 16> : launch_list<false, false, kLongChunk, 16>);
     return launch(a, nullptr, nullptr, c->n_work, c->counters, c->num_sms, c->stream);
 }
 
@@ -752,20 +726,22 @@ PairArgs pair_args(const p3m_ctx *c, const double *acc_in, double *acc_out, doub
     a.rcull2 = (float)(rcull * rcull);
     const double rin = c->g.r_c * (1.0 - 1e-4) - c->g.box * 1e-6;
     a.rin2 = rin > 0.0 ? (float)(rin * rin) : -1.0f;
-    a.group = pair_group(c);
-    a.pad = 0;
+
     return a;
 }
 
 cudaError_t launch_pairs_batched(const PairArgs *descs, const uint32_t *order,
-                                 const uint32_t *n_total, uint32_t *cursor, int num_sms,
+                                 const uint32_t *n_total, uint32_t *cursor, int group, int num_sms,
                                  cudaStream_t s)
 {
     cudaError_t e = cudaMemsetAsync(cursor, 0, sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
     PairArgs unused;
     memset(&unused, 0, sizeof(unused));
-    return launch_list<true, 2, kLongChunk, 16>(unused, descs, order, n_total, cursor, num_sms, s);
+    auto launch = group == 16  ? launch_list<true, true, kLongChunk, 16>
+                  : group == 8 ? launch_list<true, true, kLongChunk, 8>
+                               : launch_list<true, true, kLongChunk, 4>;
+    return launch(unused, descs, order, n_total, cursor, num_sms, s);
 }
 
 cudaError_t launch_store_pair_args(PairArgs *dst, const PairArgs &a, cudaStream_t s)

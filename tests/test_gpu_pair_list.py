@@ -187,8 +187,11 @@ def test_list_group_sizes(fraction, kind, softening):
     assert math.sqrt(float(np.sum((va - vb) ** 2))) <= 2e-5 * math.sqrt(float(np.sum(vb ** 2)))
 
 
-def test_ensemble_members_keep_their_group_size():
-    """Simulations whose lists have 4, 8 and 16 particles, advanced together and alone: the same bits."""
+@pytest.mark.parametrize("batched", [False, True])
+@pytest.mark.parametrize("softening", [0.02, 1.0])
+def test_ensemble_members_keep_their_group_size(batched, softening):
+    """Simulations whose lists have 4, 8 and 16 particles, advanced together (the pair sums of those of one
+    group size and the additive factor in one launch, or all of them alone) and alone: the same bits."""
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
@@ -198,15 +201,15 @@ def test_ensemble_members_keep_their_group_size():
     sets = [(p, *S.zeldovich(p, 60.0, a[0], 5 + p)) for p in (17, 30, 40, 21)]
     alone = []
     for p, pos, mom in sets:
-        with P3M(60.0, p ** 3, max(20, p + p % 2), softening=0.02, stream=0) as sim:
+        with P3M(60.0, p ** 3, max(20, p + p % 2), softening=softening, stream=0) as sim:
             sim.set_particles(pos, mom, a=a[0])
             for k in range(3):
                 sim.step(a[k], a[k + 1] - a[k])
             alone.append(sim.get_particles())
-    sims = [P3M(60.0, p ** 3, max(20, p + p % 2), softening=0.02, stream=0) for p, _, _ in sets]
+    sims = [P3M(60.0, p ** 3, max(20, p + p % 2), softening=softening, stream=0) for p, _, _ in sets]
     for sim, (_, pos, mom) in zip(sims, sets):
         sim.set_particles(pos, mom, a=a[0])
-    with Ensemble(sims) as ens:
+    with Ensemble(sims, batched=batched) as ens:
         ens.run(a)
     for sim, (pos, mom) in zip(sims, alone):
         got = sim.get_particles()
