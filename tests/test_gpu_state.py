@@ -98,3 +98,27 @@ def test_results_in_the_callers_order(n, where):
         torch.cuda.synchronize()
     assert torch.equal(p.cpu(), pos) and torch.equal(m.cpu(), mom) and torch.equal(only.cpu(), mom)
     assert torch.equal(a.cpu(), alone.cpu())
+
+
+def test_sort_timeout_with_many_particles():
+    """The injected sort timeout also reaches a context whose sort has no look-back of its own (more than 2^18
+    particles): P3M_ETIMEOUT, unchanged positions, and the same forces once the injection is cleared."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1510_07621_gb300 import P3M, P3MError, _lib, build
+    build.build()
+    lib = _lib.load()
+    n, box = 300007, 100.0
+    x = np.mod(S.uniform_random(n, box, 23), box)
+    with P3M(box, n, 64, short_range=False) as sim:
+        sim.set_particles(x, np.zeros_like(x), a=1.0)
+        first = sim.forces(1.0)
+        sim.set_particles(x, np.zeros_like(x), a=1.0)
+        assert lib.p3m_inject_fault(sim._ctx, _lib.P3M_INJECT_SORT_TIMEOUT, 2000) == _lib.P3M_OK
+        with pytest.raises(P3MError) as e:
+            sim.forces(1.0)
+        assert e.value.code == _lib.P3M_ETIMEOUT
+        assert np.array_equal(sim.get_particles()[0], x)
+        assert lib.p3m_inject_fault(sim._ctx, _lib.P3M_INJECT_NONE, 0) == _lib.P3M_OK
+        assert np.array_equal(sim.forces(1.0), first)
