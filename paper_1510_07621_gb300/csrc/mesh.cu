@@ -13,6 +13,7 @@
 #include <mutex>
 
 #include "p3m_internal.cuh"
+#include "state.cuh"
 
 namespace {
 
@@ -26,10 +27,9 @@ __device__ __forceinline__ int wrap_index(int i, int M)
 template <typename T>
 __device__ __forceinline__ void cic_stencil(double x, double inv_h, int &i0, T &f)
 {
-    const double u = __dmul_rn(x, inv_h);
-    const double fl = floor(u);
-    i0 = (int)fl;
-    f = (T)(u - fl);
+    double r;
+    split_floor(__dmul_rn(x, inv_h), i0, r);
+    f = (T)r;
 }
 
 // CIC stencil of a sorted particle in FP32 from its cell-relative coordinates (FP32 mode).  The
