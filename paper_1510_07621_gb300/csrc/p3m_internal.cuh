@@ -243,7 +243,8 @@ struct PairArgs {
 // dfac = D / m).  vals are not touched.
 cudaError_t launch_kick_drift_keys(p3m_ctx *c, bool kick_drift, double kfac, double dfac,
                                    bool from_table = false);
-// Stable LSD radix sort of (keys, identity) -> c->keys (sorted), c->vals (source slots).
+// Stable LSD radix sort of (keys, identity) -> c->keys (sorted), c->vals (source slots); follows
+// launch_kick_drift_keys, which prepares its digit counts.
 cudaError_t launch_radix_sort(p3m_ctx *c);
 // Permutes pos/mom/pid by c->vals, writes the relative coordinates, cell_start, work list.
 cudaError_t launch_permute_and_cells(p3m_ctx *c);

@@ -16,6 +16,7 @@
 #include <string.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "p3m_internal.cuh"
 #include "state.cuh"
@@ -91,43 +92,74 @@ __device__ __forceinline__ uint32_t make_key(uint32_t fx, uint32_t fy, uint32_t 
     return (cell << (3 * b)) | code;
 }
 
+// hist[d] += 1 of every valid lane.  A warp whose digits agree (the upper digits of a set that is nearly
+// sorted) adds once, the others one by one in shared memory.
+__device__ __forceinline__ void count_digit(uint32_t *hist, uint32_t d, bool valid, int lane)
+{
+    const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
+    if (__all_sync(0xffffffffu, valid && d == d0)) {
+        if (lane == 0) atomicAdd(&hist[d0], 32u);
+    } else if (valid) {
+        atomicAdd(&hist[d], 1u);
+    }
+}
+
 // Half kick + drift (optional), periodic wrap, key.  Kick and drift are one FMA each (a single
 // rounding): p += (m K) a; x += p (D / m).  With fac_dev the two factors are read from
 // fac_dev[0], fac_dev[1] (graph-replayed steps).
 // Bound by memory (28 bytes per particle, 124 with the kick) once the FP64 compares are out of the way
 // and the Hilbert index is unrolled: 256^3 without a kick 0.381 -> 0.159 ms.  A position that is inside the
 // box already is not written again.
-template <int kBits, bool kKick>
+// kHist (the sort by look-back follows): hist[p 256 + d] += keys whose digit p is d, p < passes, by shared-memory
+// atomics; a kernel of its own took 4 to 5 us of a small set's evaluation.
+template <int kBits, bool kKick, bool kHist>
 __global__ void __launch_bounds__(256, 6)
     k_kick_drift_keys(double *__restrict__ pos, double *__restrict__ mom, const double *__restrict__ acc,
                       P3MGeom g, double kfac, double dfac, uint32_t *__restrict__ keys,
-                      const double *__restrict__ fac_dev)
+                      const double *__restrict__ fac_dev, int passes, uint32_t *__restrict__ hist)
 {
+    __shared__ uint32_t h[kHist ? 4 * kRadix : 1];
+    if (kHist) {
+        for (int i = threadIdx.x; i < passes * kRadix; i += kThreads) h[i] = 0;
+        __syncthreads();
+    }
+    const int lane = threadIdx.x & 31;
     const int64_t n = g.n;
     if (kKick && fac_dev) {
         kfac = fac_dev[0];
         dfac = fac_dev[1];
     }
     const float inv_f = (float)g.inv_fine, tol = (float)g.n_fine * 0x1p-21f;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t f[3];
+    for (int64_t i0 = blockIdx.x * (int64_t)kThreads; i0 < n; i0 += (int64_t)gridDim.x * kThreads) {
+        const int64_t i = i0 + threadIdx.x;
+        uint32_t key = 0;
+        if (i < n) {
+            uint32_t f[3];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            double x = pos[d * n + i];
-            const double x0 = x;
-            if (kKick) {
-                const double p = __fma_rn(kfac, acc[d * n + i], mom[d * n + i]);
-                mom[d * n + i] = p;
-                x = __fma_rn(p, dfac, x);
+            for (int d = 0; d < 3; ++d) {
+                double x = pos[d * n + i];
+                const double x0 = x;
+                if (kKick) {
+                    const double p = __fma_rn(kfac, acc[d * n + i], mom[d * n + i]);
+                    mom[d * n + i] = p;
+                    x = __fma_rn(p, dfac, x);
+                }
+                x = wrap_box(x, g.box);
+                if (__double_as_longlong(x) != __double_as_longlong(x0)) pos[d * n + i] = x;
+                f[d] = fine_index_fast(x, g.inv_fine, inv_f, tol, g.n_fine);
             }
-            x = wrap_box(x, g.box);
-            if (__double_as_longlong(x) != __double_as_longlong(x0)) pos[d * n + i] = x;
-            f[d] = fine_index_fast(x, g.inv_fine, inv_f, tol, g.n_fine);
+            key = make_key<kBits>(f[0], f[1], f[2], g);
+            p3m_in_bounds((key >> (3 * g.sub_bits)) < (uint32_t)g.n_cells, g.flags);
+            keys[i] = key;
         }
-        const uint32_t key = make_key<kBits>(f[0], f[1], f[2], g);
-        p3m_in_bounds((key >> (3 * g.sub_bits)) < (uint32_t)g.n_cells, g.flags);
-        keys[i] = key;
+        if (kHist)
+            for (int p = 0; p < passes; ++p)
+                count_digit(h + p * kRadix, (key >> (p * kRadixBits)) & (kRadix - 1), i < n, lane);
+    }
+    if (kHist) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < passes * kRadix; i += kThreads)
+            if (h[i]) atomicAdd(hist + i, h[i]);
     }
 }
 
@@ -150,18 +182,6 @@ __device__ __forceinline__ uint32_t match_digit(uint32_t d, bool valid, int bits
 // Tile t holds keys [t*4096, (t+1)*4096), visited in 16 rounds of 256 consecutive keys;
 // within a round warp w holds keys [w*32, w*32+32).  That visiting order is the input order,
 // so ranks assigned round by round, warp by warp, lane by lane make each pass stable.
-
-// hist[d] += 1 of every valid lane.  A warp whose digits agree (the upper digits of a set that is nearly
-// sorted) adds once, the others one by one in shared memory.
-__device__ __forceinline__ void count_digit(uint32_t *hist, uint32_t d, bool valid, int lane)
-{
-    const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
-    if (__all_sync(0xffffffffu, valid && d == d0)) {
-        if (lane == 0) atomicAdd(&hist[d0], 32u);
-    } else if (valid) {
-        atomicAdd(&hist[d], 1u);
-    }
-}
 
 __global__ void __launch_bounds__(kThreads)
     k_radix_upsweep(const uint32_t *__restrict__ keys, int64_t n, int shift,
@@ -234,10 +254,10 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // ------------------------------------------------------------------ one-sweep LSD radix sort
-// The particle sort of few keys: one histogram kernel for all passes, then one kernel per 8-bit pass.  A
-// pass's CTAs take tiles (4096 keys, fewer for few particles) in launch order from an atomic counter; each ranks its tile
-// (warp w its w-th eighth, round by round and lane by lane, so ranks are
-// stable), publishes its per-digit counts, and finds the count of each digit in all earlier
+// The particle sort of few keys: the digit counts of all passes from the keys' kernel, then one
+// kernel per 8-bit pass.  A pass's CTAs take tiles (4096 keys, fewer for few particles) in launch
+// order from an atomic counter; each ranks its tile (warp w its w-th eighth, round by round and lane
+// by lane, so ranks are stable), publishes its per-digit counts, and finds the count of each digit in all earlier
 // tiles by walking back over their published values (decoupled look-back: an entry holds a
 // tile's own count, flag kAgg, or the running total through that tile, flag kInc).  A tile
 // publishes kAgg before it waits for anything, and waits only on tiles taken before it, so
@@ -249,43 +269,12 @@ __global__ void __launch_bounds__(kThreads)
 // hundreds of tiles in flight a tile looks back over hundreds of entries of 256 digits, and that traffic
 // took more time than reading the keys twice.  Sort phase, before / now: 256^3 0.75 / 0.54 ms (look-back
 // with eight entries at once: 0.63), 128^3 0.165 / 0.123, 48^3 (look-back, tiles of 1024; counting: 87 us)
-// 50 / 35 us, 5003 keys 43 / 22 us.  What bounds a pass now is the ranking: 26 ballots per key and their
+// 50 / 35 us, 5003 keys 43 / 22 us (with the digit counts, which the keys' kernel has since taken over).  What bounds a pass now is the ranking: 26 ballots per key and their
 // integer operations keep the ALU pipe 75 % busy.
 
 constexpr int kWarps = kThreads / 32;
 constexpr int kLookBack = 8;  // earlier tiles whose entries are read at once (a chain of single reads before)
 constexpr uint32_t kAgg = 1u << 30, kInc = 2u << 30, kCountMask = kAgg - 1;  // (fewer than 2^30 keys)
-
-// hist[p * 256 + d] += number of keys whose digit p is d, for p < passes (<= 4).   (Counted by
-// shared-memory atomics: matching equal digits first kept the vote pipe 73 % busy, 256^3 0.118 -> 0.050 ms;
-// 5003 keys, in blocks of 1024 instead of 4096: 8 -> 3.6 us.)
-constexpr int kHistItems = 4;
-__global__ void __launch_bounds__(kThreads)
-    k_digit_hist(const uint32_t *__restrict__ keys, int64_t n, int passes, uint32_t *__restrict__ hist)
-{
-    __shared__ uint32_t h[4 * kRadix];
-    for (int i = threadIdx.x; i < 4 * kRadix; i += kThreads) h[i] = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * kThreads * kHistItems;
-    for (int64_t i0 = (int64_t)blockIdx.x * kThreads * kHistItems; i0 < n; i0 += stride) {
-        uint32_t k[kHistItems];
-#pragma unroll
-        for (int r = 0; r < kHistItems; ++r) {
-            const int64_t i = i0 + r * kThreads + threadIdx.x;
-            k[r] = i < n ? keys[i] : 0u;
-        }
-#pragma unroll
-        for (int r = 0; r < kHistItems; ++r) {
-            const bool valid = i0 + r * kThreads + threadIdx.x < n;
-            for (int p = 0; p < passes; ++p)
-                count_digit(h + p * kRadix, (k[r] >> (p * kRadixBits)) & (kRadix - 1), valid, lane);
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < passes * kRadix; i += kThreads)
-        if (h[i]) atomicAdd(hist + i, h[i]);
-}
 
 __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *total);
 
@@ -311,6 +300,7 @@ __global__ void __launch_bounds__(kThreads, 3)
     for (int w = 0; w < kWarps; ++w) s_wcnt[w][tid] = 0;
     __syncthreads();
     const uint32_t tile = s_tile;
+    if (tile >= gridDim.x) return;  // (never: the counter starts at zero)
     const int64_t wbase = (int64_t)tile * kTile + (int64_t)warp * kWarpItems;
     const uint32_t lt = (1u << lane) - 1u;
 
@@ -768,15 +758,52 @@ inline int grid_for(int64_t n, int threads, int num_sms)
 
 }  // namespace
 
+namespace {
+
+// How the particle sort of a context runs: by look-back (few particles; an injected timeout needs a look-back
+// to wait in) or counted passes.  The keys' kernel clears and fills the look-back's digit counts, so
+// every look-back sort follows one.
+struct SortPlan {
+    bool small, chain;
+    int passes;
+    unsigned n_tiles;
+    size_t status_words;  // look-back entries of a pass
+};
+
+SortPlan sort_plan(const p3m_ctx *c)
+{
+    SortPlan p;
+    p.small = c->g.n <= P3M_SORT_SMALL;
+    p.chain = p.small || c->sort_probe;
+    p.passes = (c->key_bits + kRadixBits - 1) / kRadixBits;
+    const int64_t tile = p.small ? 4 * kThreads : P3M_SORT_TILE;
+    p.n_tiles = (unsigned)((c->g.n + tile - 1) / tile);
+    p.status_words = (size_t)kRadix * p.n_tiles;
+    return p;
+}
+
+}  // namespace
+
 cudaError_t launch_kick_drift_keys(p3m_ctx *c, bool kick_drift, double kfac, double dfac,
                                    bool from_table)
 {
+    const SortPlan sp = sort_plan(c);
+    if (sp.chain) {
+        // sort_hist: 4 x 256 digit counts, then one tile counter per pass; sort_status follows it.  Few
+        // particles have a status array per pass, cleared together.
+        const cudaError_t e = cudaMemsetAsync(
+            c->sort_hist, 0, P3M_SORT_HIST_BYTES + 4 * sp.status_words * (sp.small ? sp.passes : 1), c->stream);
+        if (e != cudaSuccess) return e;
+    }
     c->launches += 1;
-    auto kern = c->g.sub_bits != 3 ? (kick_drift ? k_kick_drift_keys<-1, true> : k_kick_drift_keys<-1, false>)
-                                   : (kick_drift ? k_kick_drift_keys<3, true> : k_kick_drift_keys<3, false>);
-    kern<<<grid_for(c->g.n, 256, c->num_sms), 256, 0, c->stream>>>(
-        c->pos, c->mom, c->acc, c->g, kfac, dfac, c->keys,
-        from_table ? c->cur_fac : nullptr);
+    auto pick = [&](auto bits) {
+        constexpr int kB = decltype(bits)::value;
+        return kick_drift ? (sp.chain ? k_kick_drift_keys<kB, true, true> : k_kick_drift_keys<kB, true, false>)
+                          : (sp.chain ? k_kick_drift_keys<kB, false, true> : k_kick_drift_keys<kB, false, false>);
+    };
+    auto kern = c->g.sub_bits == 3 ? pick(std::integral_constant<int, 3>{}) : pick(std::integral_constant<int, -1>{});
+    kern<<<grid_for(c->g.n, kThreads, c->num_sms), kThreads, 0, c->stream>>>(
+        c->pos, c->mom, c->acc, c->g, kfac, dfac, c->keys, from_table ? c->cur_fac : nullptr, sp.passes, c->sort_hist);
     return cudaGetLastError();
 }
 
@@ -832,25 +859,13 @@ cudaError_t radix_sort_pairs(uint32_t **k, uint32_t **v, bool identity_vals, int
 cudaError_t launch_radix_sort(p3m_ctx *c)
 {
     const int64_t n = c->g.n;
-    const int passes = (c->key_bits + kRadixBits - 1) / kRadixBits;
-    const bool small = n <= P3M_SORT_SMALL;
-    const int64_t tile = small ? 4 * kThreads : P3M_SORT_TILE;
-    const unsigned n_tiles = (unsigned)((n + tile - 1) / tile);
-    // (an injected timeout needs a look-back to wait in)
-    const bool chain = small || c->sort_probe;
-    const size_t status_words = (size_t)kRadix * n_tiles;
+    const SortPlan sp = sort_plan(c);
+    const bool small = sp.small, chain = sp.chain;
+    const int passes = sp.passes;
+    const unsigned n_tiles = sp.n_tiles;
+    const size_t status_words = sp.status_words;
     cudaStream_t s = c->stream;
     cudaError_t e = cudaSuccess;
-    if (chain) {
-        // sort_hist: 4 x 256 digit counts, then one tile counter per pass; sort_status follows it.  Few
-        // particles have a status array per pass, cleared together.
-        e = cudaMemsetAsync(c->sort_hist, 0, P3M_SORT_HIST_BYTES + 4 * status_words * (small ? passes : 1), s);
-        if (e != cudaSuccess) return e;
-        const unsigned hist_grid = (unsigned)min((n + kHistItems * kThreads - 1) / (kHistItems * kThreads),
-                                                 (int64_t)c->num_sms * 8);
-        k_digit_hist<<<hist_grid, kThreads, 0, s>>>(c->keys, n, passes, c->sort_hist);
-        c->launches += 1;
-    }
     for (int p = 0; p < passes; ++p) {
         const int shift = p * kRadixBits, bits = min(kRadixBits, c->key_bits - shift);
         const uint32_t *vin = p ? c->vals : nullptr;  // the first pass's values are the slots
