@@ -484,7 +484,7 @@ __device__ __forceinline__ f2 pair_jac2(f2 w, f2 dw, const VjpConst2 &k, f2 *c)
 
 template <bool kAdditive, int kG>
 __global__ void __launch_bounds__(32, 16)
-    k_pairs_vjp_list(const uint32_t *__restrict__ relq, const float *__restrict__ vfx,
+    k_pairs_vjp_list(const uint32_t *__restrict__ relq, CutState cut, const float *__restrict__ vfx,
                      const float4 *__restrict__ block_box, const uint32_t *__restrict__ cell_start,
                      const uint32_t *__restrict__ work,
                      const uint32_t *__restrict__ n_work_ptr, P3MGeom g, PairFactor fac, double scale,
@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(32, 16)
                     if (part == rintf(part)) continue;
                     const float dw = fmaf(dx[2], wv[2], fmaf(dx[1], wv[1], dx[0] * wv[0]));
                     const uint32_t i = min(first + ip + u * kPairsI, cend - 1);
-                    const float t = (cut_inside(relq, i, slot[p], dx[0], dx[1], dx[2], fac) ? 1.0f : 0.0f) - part;
+                    const float t = (cut_inside<true>(relq, cut, g, i, slot[p], dx[0], dx[1], dx[2], fac) ? 1.0f : 0.0f) - part;
                     f2 c, h = pair_jac2<kAdditive>(f2_pack(w, w), f2_pack(dw, dw), kc, &c);
 #pragma unroll
                     for (int d = 0; d < 3; ++d) o[u][d].x = fmaf(t * h.x, wv[d], fmaf(t * c.x, dx[d], o[u][d].x));
@@ -1004,7 +1004,7 @@ cudaError_t vjp_pairs(p3m_ctx *c, const double *v_slots, double *out_slots)
     if (fp32) {
         const double len = ldexp(c->g.cs, -kFixBits) / (double)c->pair_factor.lambda;
         list<<<c->num_sms * per_sm, 32, 0, c->stream>>>(
-            c->relq, c->adj_vfx, c->block_box, c->cell_start, c->work,
+            c->relq, CutState{(const float4 *)c->rel, c->keys}, c->adj_vfx, c->block_box, c->cell_start, c->work,
             c->n_work, c->g, c->pair_factor, c->g.gm / (len * len * len), rcull2,
             c->counters + 3, out_slots);
     } else {

@@ -237,7 +237,8 @@ PairFactor fit_pair_factor(double cutoff_in_rs, const P3MGeom &g)
     p.cut_m = (float)(-0.5 / (kCutBand * rc2));
     p.cut_b = (float)(0.5 - (double)p.cut_m * (double)p.rc2);  // (half at the cutoff)
     const double fix_rc = ldexp(g.r_c / g.cs, kFixBits);        // (at most 2^29: cells are no smaller than r_c)
-    p.fix_rc2 = (long long)ceil(fix_rc * fix_rc);
+    p.fix_rc2 = g.n < g.n_cells ? (long long)ceil(fix_rc * fix_rc) : 0;
+    p.fp32_rc2 = (float)(g.r_c * g.r_c);
     p.length = (float)(g.r_s / rho);
     p.lambda = (float)(ldexp(g.cs, -kFixBits) * rho / g.r_s);
     p.cell = (float)g.cs;

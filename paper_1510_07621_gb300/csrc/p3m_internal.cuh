@@ -15,8 +15,8 @@ constexpr int kSplitTab64 = 64, kSplitRow64 = 10;
 // (8 cells), so that differences of particles in neighbouring cells are exact integers.
 constexpr int kFixBits = 29;
 constexpr float kFixUnit = 0x1p-29f;
-// The FP32 pair kernels decide on the cutoff by the FP32 r^2 outside a band of this relative half
-// width (six times its rms error there), by the fixed-point coordinates inside it.
+// The FP32 pair kernels decide on the cutoff by their lists' FP32 r^2 outside a band of this relative half
+// width (six times its rms error there), one by one inside it (see cut_inside).
 constexpr double kCutBand = 5e-7;
 
 // The FP32 pair factor f(r) = g(r/r_s) (r^2 + eps^2)^-3/2 in scaled lengths (see fit_pair_factor):
@@ -32,7 +32,8 @@ struct PairFactor {
     float lambda;        // scaled lengths per fixed-point unit
     float cell, length;  // side of a chaining cell; one scaled length
     double scale;        // accelerations = scale * sum f d
-    long long fix_rc2;   // a pair is inside if its squared distance in fixed-point units is below this
+    long long fix_rc2;   // a pair is inside if its squared distance in fixed-point units is below this; 0: not used
+    float fp32_rc2;      // the squared cutoff of the FP32 decision, in lengths
     float grad[3];       // general form of f'(r)/r: exponent of exp(-r^2/(4 r_s^2)) over t's,
                          // -1/(2 sqrt(pi)) in scaled lengths, and -3
     int additive;
@@ -221,6 +222,8 @@ inline int pair_group(const p3m_ctx *c)
 // indexed by simulation in the batched ensemble launch.
 struct PairArgs {
     const uint32_t *relq;
+    const float4 *rel;
+    const uint32_t *keys;
     const float4 *block_box;
     const uint32_t *cell_start;
     const uint32_t *work;

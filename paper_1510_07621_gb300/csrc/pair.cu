@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(32)
 // at 20.5), 19 the candidate tests and 6 the set-up of groups.  16 particles per group
 // and 18 CTAs per SM: 8, 32 and 16, 20, 24 are within 6 % or slower on both sets.  Two lists of 16 (or
 // four of 8) filled by one pass over the candidates save a third of the tests but cost as much in
-// registers and reloads (3.18 and 4.8 ms, against 3.06 without the exact cutoff).
+// registers and reloads (3.18 and 4.8 ms, against 3.06 without the decisions at the cutoff).
 //
 // Coordinates are 32-bit fixed point, 2^-29 of a chaining cell, modulo 8 cells (relq): differences
 // of particles in neighbouring cells, periodic images included, are exact integers, and only the
@@ -438,7 +438,7 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
                     const float part = cut_part(w, cut_m, cut_b);
                     if (part == rintf(part)) continue;
                     const uint32_t i = min(first + ip + u * kPairsI, cend - 1);
-                    const float t = (cut_inside(A.relq, i, slot[p], dx, dy, dz, A.fac) ? 1.0f : 0.0f) - part;
+                    const float t = (cut_inside<false>(A.relq, {A.rel, A.keys}, g, i, slot[p], dx, dy, dz, A.fac) ? 1.0f : 0.0f) - part;
                     const float f = t * pair_factor_q<kAdd>(f2_pack(w, w), kc).x;
                     px[u].x = fmaf(f, dx, px[u].x);
                     py[u].x = fmaf(f, dy, py[u].x);
@@ -708,6 +708,8 @@ PairArgs pair_args(const p3m_ctx *c, const double *acc_in, double *acc_out, doub
     PairArgs a;
     memset(&a, 0, sizeof(a));
     a.relq = c->relq;
+    a.rel = (const float4 *)c->rel;
+    a.keys = c->keys;
     a.block_box = c->block_box;
     a.cell_start = c->cell_start;
     a.work = c->work;

@@ -160,14 +160,18 @@ __device__ __forceinline__ int live_blocks(uint32_t t, uint32_t t1, const PairSe
 }
 
 // ------------------------------------------------------------------ the cutoff
-// FP32 r^2 has an rms error of 8e-8 at the cutoff, which would put about one pair in 10^7 on the wrong
-// side of it: the force jumps there, and for nearly uniform sets those few pairs were the largest part
-// of the error (2e-6 against 4e-7 of the rest; any FP32 evaluation has its own).  So the kernels
-// evaluate with a factor that is 1 inside, 0 outside and a fraction within kCutBand, sum it per lane
-// (it also counts the pairs), and where a sum has a fraction (one list of 160 in 600) look at the list
-// again and decide by the exact fixed-point distance.  (Two clamped FMAs, a product and a sum per two
-// pairs take 4 % of the force kernel's time; compares, selects and counts beside a minimum of
-// |w - rc2| took 9 %.)
+// Which pairs interact must not depend on a kernel's layout: the force jumps at the cutoff, and one pair on
+// the other side moves a component of a nearly uniform set by up to 3e-3 of the rms force.  The FP32 mode
+// decides r < r_c by the FP32 r^2 of the cell-relative coordinates, of x_j and of x_i shifted into j's
+// cell (cut_inside), which is within 8e-8 (rms) of the exact one at the cutoff: about one pair in 10^7
+// falls on the other side of it.  A set with fewer particles than chaining cells, where a pair may be all of a
+// particle's force, is decided by the fixed-point coordinates instead (PairFactor::fix_rc2).
+// The lists' own r^2 is rounded differently, so the kernels evaluate with a factor that is 1 inside, 0
+// outside and a fraction within kCutBand, sum it per lane (it also counts the pairs), and where a sum has a
+// fraction (one list of 160 in 600) look at the list again and decide its pairs in the band.  (Two fractions
+// of one lane whose sum is a whole number to 2^-18 would hide each other.)  Two clamped FMAs, a product and a sum
+// per two pairs take 4 % of the force kernel's time; compares, selects and counts beside a minimum of
+// |w - rc2| took 9 %.
 
 // 1 inside the cutoff, 0 outside
 __device__ __forceinline__ float cut_part(float w, float cut_m, float cut_b)
@@ -175,10 +179,50 @@ __device__ __forceinline__ float cut_part(float w, float cut_m, float cut_b)
     return __saturatef(fmaf(w, cut_m, cut_b));
 }
 
-// Whether i and j, whose scaled FP32 difference is (dx, dy, dz), are closer than the cutoff.
-__device__ __forceinline__ bool cut_inside(const uint32_t *relq, uint32_t i, uint32_t j, float dx, float dy,
-                                           float dz, const PairFactor &f)
+// r < r_c by FP32, i and j in neighbouring chaining cells (n_c >= 3: the two cells give the periodic image).
+__device__ __forceinline__ bool cut_inside_fp32(const float4 *rel, const uint32_t *keys, int sub_bits, int nc, double cs,
+                                                double box, float rc2, uint32_t i, uint32_t j)
 {
+    uint32_t ci = keys[i] >> (3 * sub_bits), cj = keys[j] >> (3 * sub_bits);
+    const float4 a = rel[i], b = rel[j];
+    const float xi[3] = {a.x, a.y, a.z}, xj[3] = {b.x, b.y, b.z};
+    float r2 = 1e-20f;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const int c = (int)(ci % (uint32_t)nc), w = (int)(cj % (uint32_t)nc);
+        ci /= (uint32_t)nc;
+        cj /= (uint32_t)nc;
+        const double image = w - c > 1 ? -box : (w - c < -1 ? box : 0.0);
+        // the two cells' origins differ by s, an FP32 value and its FP32 residual
+        const double s = ((double)w * cs + image) - (double)c * cs;
+        const float hi = (float)s, lo = (float)(s - (double)hi);
+        const float x = xj[d] - ((xi[d] - hi) - lo);
+        r2 = fmaf(x, x, r2);
+    }
+    return r2 < rc2;
+}
+
+// (A call in the force kernel, one in thousands of pairs: its registers are at their limit.  The VJP kernel
+// has some to spare and is 1.5 % faster with the function inlined.)
+__device__ __noinline__ bool cut_inside_fp32_call(const float4 *rel, const uint32_t *keys, int sub_bits, int nc, double cs,
+                                                  double box, float rc2, uint32_t i, uint32_t j)
+{
+    return cut_inside_fp32(rel, keys, sub_bits, nc, cs, box, rc2, i, j);
+}
+
+// What the decision on a pair in the band reads beside the fixed-point coordinates.
+struct CutState {
+    const float4 *rel;     // relative to the cells' origins, sorted order
+    const uint32_t *keys;  // sorted
+};
+
+// Whether i and j, whose scaled FP32 difference is (dx, dy, dz), are closer than the cutoff.
+template <bool kInline>
+__device__ __forceinline__ bool cut_inside(const uint32_t *relq, const CutState &st, const P3MGeom &g, uint32_t i,
+                                           uint32_t j, float dx, float dy, float dz, const PairFactor &f)
+{
+    if (f.fix_rc2 == 0)
+        return (kInline ? cut_inside_fp32 : cut_inside_fp32_call)(st.rel, st.keys, g.sub_bits, g.n_c, g.cs, g.box, f.fp32_rc2, i, j);
     const uint32_t *qi = fix_coords(relq, i), *qj = fix_coords(relq, j);
     const float d3[3] = {dx, dy, dz};
     long long r2 = 0;
