@@ -433,11 +433,11 @@ __global__ void __launch_bounds__(32)
 // and two list entries per lane in packed f32x2 arithmetic), here with v beside the coordinates, for
 //   out_k += Gm sum_j [h w + (h'/r) (d.w) d],  w = v_j - v_k,
 // where h is the force kernel's fitted factor and h'/r, in the additive form, twice the derivative of
-// that fit with respect to w = r^2 + eps^2 (scaled lengths, q = s + ab + na t, k = ln 2):
-//   h = q s^2 + P(t),  h'/r = t (2 k (-na) s^2 - 2 k P'(t)) - (2 q + s) s^4,
+// that fit with respect to w = r^2 + eps^2 (scaled lengths, q = s + ab + na t + e s^2, e = c[4], k = ln 2):
+//   h = q s^2 + P(t),  h'/r = t (2 k (-na) s^2 - 2 k P'(t)) - (2 (q + e s^2) + s) s^4,
 // as accurate as the closed form (1.9e-7 against 3.8e-7 of the force derivative at the cutoff 4.5) and
 // without a second exponential.  The general form takes g' = -x^2 exp(-x^2/4)/(2 sqrt(pi)) closed.
-// s^4 is never formed: (2 q + s) s^2 times s^2 (d.w) stays finite for close pairs without softening.
+// s^4 is never formed: (2 q + ..) s^2 times s^2 (d.w) stays finite for close pairs without softening.
 // r = 0 pairs are selected out (their w need not vanish for coincident particles); only the row of the
 // own cell can hold them.  Before, all 32 lanes met every j of a tested block with 40 FP32 operations
 // and three 8-cycle MUFU operations per pair (34 and one here).  128^3 near-uniform, one call with the
@@ -462,11 +462,11 @@ __device__ __forceinline__ f2 pair_jac2(f2 w, f2 dw, const VjpConst2 &k, f2 *c)
     p = f2_fma(p, t, k.c[2]);
     p = f2_fma(p, t, k.c[1]);
     if (kAdditive) {
-        const f2 q = f2_add(rw, f2_fma(k.na, t, k.ab)), s2 = f2_mul(rw, rw);
+        const f2 s2 = f2_mul(rw, rw), q = f2_fma(k.c[4], s2, f2_add(rw, f2_fma(k.na, t, k.ab)));
         const f2 h = f2_fma(p, t, f2_fma(q, s2, k.c[0]));
         const f2 dp = f2_fma(f2_fma(k.d[2], t, k.d[1]), t, k.d[0]);
         const f2 inner = f2_mul(t, f2_fma(k.na2, s2, dp));
-        const f2 m = f2_mul(f2_fma(k.two, q, rw), s2);
+        const f2 m = f2_mul(f2_fma(k.two, f2_fma(k.c[4], s2, q), rw), s2);
         *c = f2_fma(inner, dw, f2_neg(f2_mul(m, f2_mul(s2, dw))));
         return h;
     }

@@ -143,26 +143,31 @@ void fit_split_table(double cutoff_in_rs, double *tab)
 // itself counts.  Least squares with the weights raised where the error is largest; a few kappa
 // around the quoted ones are tried, the best kept.
 // Additive form: with w = u + eps^2 in place of u,
-//   g w^-3/2 = w^-3/2 + b/w + alpha (1 - t)/w + c0 + c1 t + c2 t^2 + c3 t^3,
-// b/w = -3/2 eps^2 Q(0)/w the leading softening term of Q(u) (u/w)^3/2.  What it leaves out, of
-// order eps^4/w^2, is a relative error of f of at most 0.046 (eps/r_s)^3, reached at r ~ eps.
+//   g w^-3/2 = w^-3/2 + b/w + e/w^2 + alpha (1 - t)/w + c0 + c1 t + c2 t^2 + c3 t^3,
+// b = -3/2 eps^2 Q(0) and e = 0.44 eps^4 Q(0) from Q(u) (u/w)^3/2, whose factor (1 - x)^3/2, x = eps^2/w, is
+// followed by 1 - 3/2 x + 0.44 x^2 on [0, 1] (0.44, not 3/8: the relative error of f stays below
+// 0.0031 (eps/r_s)^3 and changes sign).  Without e it is 0.046 (eps/r_s)^3 of one sign, which a
+// halo's pairs at r ~ eps do not average out: at eps = 0.032 r_s, r from 0.3 to 4 eps, 1.7e-6 at most and
+// 8.4e-7 on average, with e 5.7e-7 (rounding) and -0.8e-7; of h'/r 2.8e-6 and 1.2e-6, now 1e-6 and 0.1e-7.
+// e costs one operation of 17 per pair (48^3, 8 steps: 2.84 -> 2.90 ms; clustered 128^3 20.9 -> 21.3).
 PairFactor fit_pair_factor(double cutoff_in_rs, const P3MGeom &g)
 {
     constexpr int kMax = 6, kN = 48;
     const double xc = cutoff_in_rs, r0 = xc < 1.0 ? 0.1 * xc : 0.4;
     const double eps = g.eps / g.r_s;
-    // 0.046 eps^3 <= 1.6e-6: at r ~ eps the FP32 rounding of the pair distance is larger
+    // 0.0031 eps^3 <= 1.1e-7, one FP32 rounding
     const bool additive = eps <= 0.0326 && xc >= 2.0;  // (shorter cutoffs leave the fit ill-conditioned)
     const int kM = additive ? 5 : 6;  // alpha, c0 .. c3 (general form: .. c4)
     const double soft = additive ? eps * eps : 0.0;
-    const double bw = 1.5 * soft * 0.094031597257959381;  // Q(0) = -1/(6 sqrt(pi))
+    const double q0 = -0.094031597257959381;  // Q(0) = -1/(6 sqrt(pi))
+    const double bw = -1.5 * soft * q0, s4 = 0.44 * soft * soft * q0;
     double w[kN], tgt[kN], wt[kN], best[kMax] = {}, best_err = 1e300, kappa = 0.0;
     for (int i = 0; i < kN; ++i) {
         const double r = r0 + 0.5 * (xc - r0) * (1.0 - cos(M_PI * (i + 0.5) / kN)), u = r * r;
         const double q = split_q(u), g = 1.0 + u * r * q;
         w[i] = u + soft;
         const double ratio = u / w[i];
-        tgt[i] = q * ratio * sqrt(ratio) - bw / w[i];
+        tgt[i] = q * ratio * sqrt(ratio) - bw / w[i] - s4 / (w[i] * w[i]);
         // (general form: df = dQ r^3 s^3, which a large softening damps at small r)
         const double s2 = u + eps * eps, rs = sqrt(u / s2);
         wt[i] = (additive ? 1.0 : rs * rs * rs) / (1.0 / r + 2.0 * g / (s2 * sqrt(s2)));
@@ -228,6 +233,7 @@ PairFactor fit_pair_factor(double cutoff_in_rs, const P3MGeom &g)
     PairFactor p;
     memset(&p, 0, sizeof(p));
     for (int k = 0; k + 1 < kM; ++k) p.c[k] = (float)(best[k + 1] / (rho * rho * rho));
+    if (additive) p.c[4] = (float)(s4 * rho);
     p.na = (float)(-best[0] / rho);
     p.ab = (float)((best[0] + bw) / rho);
     const double e2 = eps * eps * rho * rho, rc2 = xc * xc * rho * rho;

@@ -22,7 +22,7 @@ constexpr double kCutBand = 5e-7;
 // The FP32 pair factor f(r) = g(r/r_s) (r^2 + eps^2)^-3/2 in scaled lengths (see fit_pair_factor):
 // one unit is `length`, chosen so that t = 2^-w is the exponential of the fit, w the squared
 // scaled distance.  With s = (w + softening)^-1/2 and P(t) = c[0] + c[1] t + c[2] t^2 + c[3] t^3:
-//   additive:  w includes the softening (e2): f = s^3 + (ab + na t) s^2 + P(t); rc2 is the cutoff's w
+//   additive:  w includes the softening (e2): f = s^3 + (ab + na t) s^2 + c[4] s^4 + P(t); rc2 is the cutoff's w
 //   otherwise: f = s^3 (1 + r (ab + na t + r^2 P(t))), r without the softening; rc2 the cutoff's r^2
 struct PairFactor {
     float c[5];

@@ -283,7 +283,7 @@ struct PairConstQ {
 // The factor g(r/r_s) (r^2 + eps^2)^-3/2 of both halves of w (see PairFactor and fit_pair_factor).
 // The MUFU pipe takes 8 cycles per warp for a reciprocal or a square root, so that the former
 // rsqrt, rcp and sqrt per pair cost as much as 24 FP32 operations; here it is one rsqrt and one
-// ex2.  kAdditive (softening small against r_s): 16 FP32 operations per pair with the distance
+// ex2.  kAdditive (softening small against r_s): 17 FP32 operations per pair with the distance
 // and the accumulation; otherwise 21 and one more rsqrt.
 template <bool kAdditive>
 __device__ __forceinline__ f2 pair_factor_q(f2 w, const PairConstQ &k)
@@ -296,8 +296,8 @@ __device__ __forceinline__ f2 pair_factor_q(f2 w, const PairConstQ &k)
     p = f2_fma(p, t, k.c[2]);
     p = f2_fma(p, t, k.c[1]);
     if (kAdditive) {
-        const f2 q = f2_fma(k.na, t, f2_add(rw, k.ab));
-        return f2_fma(p, t, f2_fma(q, f2_mul(rw, rw), k.c[0]));
+        const f2 s2 = f2_mul(rw, rw), q = f2_fma(k.c[4], s2, f2_fma(k.na, t, f2_add(rw, k.ab)));
+        return f2_fma(p, t, f2_fma(q, s2, k.c[0]));
     }
     p = f2_fma(p, t, k.c[0]);
     float sl, sh;
