@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "p3m.h"
+#include "work_list.h"
 
 // The FP64 pair kernel's table of g (fit_split_table): intervals of [0, r_c], and doubles per row
 // (8 coefficients, the interval's centre, one of padding against bank conflicts).
@@ -201,7 +202,7 @@ enum {
 // against 84; 128^3: 123 us counted, 133 by look-back.
 #define P3M_SORT_SMALL 262144
 #define P3M_SORT_HIST_BYTES (4 * (4 * 256 + 4))
-#define P3M_PAIR_TI 32       // i-particles per pair work item (one per lane of a warp)
+#define P3M_PAIR_TI ((int)kWorkItem)  // i-particles per pair work item (one per lane of a warp)
 #define P3M_PAIR_CTAS 18     // one-warp CTAs per SM that the FP32 kernel's registers leave room for
 #define P3M_COUNTERS (4 + 256 + 1 + 256)  // 32-bit words of counters
 #define P3M_FLAG_TIMEOUT 1u  // counters[1] bit: a bounded wait gave up

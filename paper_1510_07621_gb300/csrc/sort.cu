@@ -20,6 +20,7 @@
 
 #include "p3m_internal.cuh"
 #include "state.cuh"
+#include "work_list.h"
 
 namespace {
 
@@ -525,18 +526,6 @@ __device__ __forceinline__ double4_16a rel_coords<double4_16a>(double x, double 
     return make_double4_16a(x, y, z, 0.0);
 }
 
-// cell_start[c] = first sorted slot whose cell is >= c, the part that slot k (of cell `cell`) writes:
-// the cells after the previous slot's up to its own, and the last slot also the cells after its own.
-__device__ __forceinline__ void first_slots(const uint32_t *keys, int64_t k, uint32_t cell, const P3MGeom &g,
-                                            uint32_t *cell_start)
-{
-    const int64_t prev = k > 0 ? (int64_t)(keys[k - 1] >> (3 * g.sub_bits)) : -1;
-    if (!p3m_in_bounds(cell < (uint32_t)g.n_cells, g.flags)) return;
-    for (int64_t c = prev + 1; c <= (int64_t)cell; ++c) cell_start[c] = (uint32_t)k;
-    if (k == g.n - 1)
-        for (int64_t c = (int64_t)cell + 1; c <= (int64_t)g.n_cells; ++c) cell_start[c] = (uint32_t)g.n;
-}
-
 // One warp per 32-slot block of the sorted order; with kPairs (a context with the short-range force)
 // the warp also writes the block's fixed-point coordinates and its bounding box (FP32, absolute
 // coordinates, within the margins of the culling radii).
@@ -577,8 +566,9 @@ __global__ void __launch_bounds__(256, 6) k_permute(const uint32_t *__restrict__
             mom_out[n + k] = mom[n + j];
             mom_out[2 * n + k] = mom[2 * n + j];
             pid_out[k] = pid[j];
-            const uint32_t cell = keys[k] >> (3 * g.sub_bits);
-            first_slots(keys, k, cell, g, cell_start);
+            const uint32_t cell = cell_of_key(keys[k], g.sub_bits, g.n_cells);
+            p3m_in_bounds((keys[k] >> (3 * g.sub_bits)) < (uint32_t)g.n_cells, g.flags);
+            first_slots(keys, k, cell, n, g.sub_bits, g.n_cells, cell_start);
             const uint32_t cx = cell % g.n_c, cy = (cell / g.n_c) % g.n_c,
                            cz = cell / (g.n_c * g.n_c);
             rv = rel_coords<R4>(x, y, z, cx, cy, cz, origin);
@@ -628,56 +618,17 @@ __global__ void k_cell_start(const uint32_t *__restrict__ keys, P3MGeom g,
     const int64_t n = g.n;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
          k += (int64_t)gridDim.x * blockDim.x)
-        first_slots(keys, k, keys[k] >> (3 * g.sub_bits), g, cell_start);
+        first_slots(keys, k, cell_of_key(keys[k], g.sub_bits, g.n_cells), n, g.sub_bits, g.n_cells, cell_start);
 }
 
-// The pair work list: items of up to 32 particles of one cell, work[2w] = cell, work[2w + 1] = first slot,
-// the most expensive first.  An item's cost estimate is (its particles) x (particles in the 27 neighbour
+// The pair work list (work_list.h): items of up to 32 particles of one cell, work[2w] = cell, work[2w + 1] =
+// first slot, the most expensive first.  An item's cost estimate is (its particles) x (particles in the 27 neighbour
 // cells); its key is the class log2(cost) to 1/8 octave (the FP32 exponent and top 3 mantissa bits, 8 bits),
 // inverted.  k_work_count counts the items of every class, k_work_place scans the 256 counts and gives each
 // item a place in its class (their order within a class is arbitrary: results do not depend on it).  Two
 // kernels instead of a count, a scan, a fill and a radix pass with its memsets (ten launches and memsets):
 // 5003 particles 23 -> 8 us of kernels, clustered 128^3 (a thread wrote all items of a dense cell; now its
 // warp does) 55 -> 12 us.
-
-struct WorkItems {
-    uint32_t first, full, rest;  // first slot, items of 32, particles of the last item
-    uint32_t key_full, key_rest;
-};
-
-// the items of cell c (the ranges are ordered unless a sort gave up)
-__device__ __forceinline__ WorkItems work_items(const uint32_t *__restrict__ cell_start, int n_c, int c)
-{
-    WorkItems w = {cell_start[c], 0u, 0u, 255u, 255u};
-    const uint32_t end = cell_start[c + 1];
-    if (end <= w.first) return w;
-    const int cx = c % n_c, cy = (c / n_c) % n_c, cz = c / (n_c * n_c);
-    // rows of three cells along x are consecutive slots (a row that wraps: the rest of it)
-    uint32_t near = 0;
-#pragma unroll
-    for (int oz = -1; oz <= 1; ++oz) {
-        int z = cz + oz;
-        z += z < 0 ? n_c : (z >= n_c ? -n_c : 0);
-#pragma unroll
-        for (int oy = -1; oy <= 1; ++oy) {
-            int y = cy + oy;
-            y += y < 0 ? n_c : (y >= n_c ? -n_c : 0);
-            const uint32_t *row = cell_start + ((size_t)z * n_c + y) * n_c;
-            near += row[min(cx + 2, n_c)] - row[max(cx - 1, 0)];
-            if (cx == 0) near += row[n_c] - row[n_c - 1];
-            if (cx == n_c - 1) near += row[1] - row[0];
-        }
-    }
-    const float nb = (float)near;
-    auto key = [&](uint32_t particles) {  // cost >= 1
-        return 255u - min((__float_as_uint((float)particles * nb) >> 20) - (127u << 3), 255u);
-    };
-    w.full = (end - w.first) / P3M_PAIR_TI;
-    w.rest = (end - w.first) % P3M_PAIR_TI;
-    w.key_full = key(P3M_PAIR_TI);
-    if (w.rest) w.key_rest = key(w.rest);
-    return w;
-}
 
 // hist[key] += items (pairs), *max_count = max particles of a cell
 __global__ void __launch_bounds__(kThreads)
@@ -724,6 +675,7 @@ __global__ void __launch_bounds__(kThreads)
     uint32_t total;
     const uint32_t before = block_exclusive_scan(hist[tid], &total);
     base[tid] = before + (mine[tid] ? atomicAdd(next + tid, mine[tid]) : 0u);
+    total = work_length(total, max_work);
     if (blockIdx.x == 0 && tid == 0) *n_work = total;
     __syncthreads();
     at_full += base[w.key_full];
