@@ -218,8 +218,9 @@ int p3m_ensemble_run(p3m_ensemble *ens, const double *a_list, int n_steps, int u
 void p3m_ensemble_free(p3m_ensemble *ens);
 /*
  * Batched pair launch (off by default; enable != 0 turns it on when at least one context
- * qualifies: FP32 P3M, a softening small against r_s, and as many particles per list as most of
- * the ensemble's particles have): each step runs the contexts' phases up to the mesh force as
+ * qualifies: FP32 P3M, a softening small against r_s, as many particles per list as most of
+ * the ensemble's particles have, and lists of the default length; looked at again before every
+ * run): each step runs the contexts' phases up to the mesh force as
  * parallel branches, then merges the pair work lists of those that qualify into one list sorted
  * by estimated cost and evaluates their pair sums in one persistent kernel launch (the contexts'
  * arguments read from a device table).  Other contexts step as before.  Results equal the
@@ -406,6 +407,10 @@ int p3m_cell_sort_noalloc(const double *pos3n, int64_t n, double box, int n_c, i
  *                          force evaluations return P3M_ETIMEOUT right after the sort, before
  *                          any kernel reads the (unreliable) order; the particle state is kept.
  *                          Allocates a zeroed buffer the size of the sort's look-back status.
+ *   P3M_INJECT_PAIR_LISTS  no fault: on ctx, arg = 16 group + tile_blocks selects the FP32 pair kernels'
+ *                          lists, shared by group = 4, 8 or 16 particles (0: by the particle
+ *                          number) and evaluated every 32 tile_blocks entries (3 or 5), so that a
+ *                          small set reaches each kernel; the forces are evaluated again.
  *   P3M_INJECT_NONE        clears every injection (and, with ctx, frees that buffer and restores
  *                          the default wait limit of 2^31 cycles); the context is usable again.
  * Returns P3M_EINVAL for an unknown fault or argument.
@@ -414,6 +419,7 @@ int p3m_cell_sort_noalloc(const double *pos3n, int64_t n, double box, int n_c, i
 #define P3M_INJECT_ALLOC 1
 #define P3M_INJECT_FFT_PLAN 2
 #define P3M_INJECT_SORT_TIMEOUT 3
+#define P3M_INJECT_PAIR_LISTS 4
 int p3m_inject_fault(p3m_ctx *ctx, int what, int64_t arg);
 
 /*

@@ -29,6 +29,7 @@ P3M_INJECT_NONE = 0
 P3M_INJECT_ALLOC = 1
 P3M_INJECT_FFT_PLAN = 2
 P3M_INJECT_SORT_TIMEOUT = 3
+P3M_INJECT_PAIR_LISTS = 4
 
 # every symbol the header declares, with (restype, argtypes)
 _c = ctypes

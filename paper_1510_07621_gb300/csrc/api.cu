@@ -1164,6 +1164,8 @@ extern "C" int p3m_inject_fault(p3m_ctx *c, int what, int64_t arg)
             }
             c->sort_probe = nullptr;
             c->sort_wait_limit = 1ll << 31;
+            if (c->list_group) ++c->geom_version;
+            c->list_group = 0;
         }
         return P3M_OK;
     case P3M_INJECT_ALLOC:
@@ -1182,6 +1184,17 @@ extern "C" int p3m_inject_fault(p3m_ctx *c, int what, int64_t arg)
             CK(cudaMemset(c->sort_probe, 0, bytes));
         }
         c->sort_wait_limit = (long long)arg;
+        return P3M_OK;
+    }
+    case P3M_INJECT_PAIR_LISTS: {
+        if (!c) return fail(c, P3M_EINVAL, "p3m_inject_fault: the lists' sizes need a context");
+        const int64_t group = arg / 16, blocks = arg % 16;
+        if ((group != 0 && group != 4 && group != 8 && group != 16) || (blocks != 3 && blocks != 5))
+            return fail(c, P3M_EINVAL, "p3m_inject_fault: no lists of that size");
+        c->list_group = (int)group;
+        c->tile_blocks = (int)blocks;
+        ++c->geom_version;  // captured graphs bake the kernel choice
+        c->forces_valid = false;
         return P3M_OK;
     }
     default:

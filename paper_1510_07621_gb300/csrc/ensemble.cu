@@ -41,12 +41,13 @@ struct p3m_ensemble {
 
     // Batched pair launch: the FP32 P3M contexts' work items merged into one cost-sorted list
     // and evaluated by one persistent pair kernel per step.
-    bool batched;             // on (default when at least two contexts qualify)
+    bool batched;             // on (off by default; in effect while some context qualifies)
     int nb;                   // contexts that qualify for the batched pair launch
     int group;                // their group size (pair_group)
     int *slot;                // per context: its index among them, or -1
     size_t *base;             // per qualifying context: offset of its work list in gkey/gval
-    size_t cap;               // sum of the qualifying contexts' work-list capacities
+    size_t cap;               // sum of the qualifying contexts' work-list capacities (the arrays below hold
+                              // all contexts that any tuning makes qualify)
     PairArgs *descs;          // device: pair arguments per qualifying context
     const uint32_t **nwork;   // device: per qualifying context, its work-item count pointer
     uint32_t *gkey[2], *gval[2], *gcounts, *gaux, *gtotal, *gcursor;
@@ -81,6 +82,8 @@ constexpr int kChunkSteps = 8;  // steps per chunk graph (even: buffer roles hav
 int ens_step(p3m_ensemble *e, double a, double da, bool from_table);
 int ens_step_fft(p3m_ensemble *e, double a, double da, bool from_table);
 
+bool batching(const p3m_ensemble *e) { return e->batched && e->nb > 0; }
+
 int capture_steps(p3m_ensemble *e, int steps, cudaGraphExec_t *out)
 {
     p3m_ctx *c = nullptr;
@@ -89,10 +92,10 @@ int capture_steps(p3m_ensemble *e, int steps, cudaGraphExec_t *out)
     if (err != cudaSuccess)
         return p3m_fail_global(P3M_ECUDA, "graph capture: %s", cudaGetErrorString(err));
     int rc = P3M_OK;
-    if (e->batched || e->grouped) {  // the steps one after another, in lockstep
+    if (batching(e) || e->grouped) {  // the steps one after another, in lockstep
         for (int i = 0; i < e->n; ++i) e->c[i]->capturing = true;
         for (int k = 0; k < steps && rc == P3M_OK; ++k)
-            rc = e->batched ? ens_step(e, 0.0, 0.0, true) : ens_step_fft(e, 0.0, 0.0, true);
+            rc = batching(e) ? ens_step(e, 0.0, 0.0, true) : ens_step_fft(e, 0.0, 0.0, true);
         for (int i = 0; i < e->n; ++i) e->c[i]->capturing = false;
     } else {  // each context's steps as one branch
         err = cudaEventRecord(e->fork, e->parent);
@@ -362,6 +365,51 @@ void drop_graphs(p3m_ensemble *e)
     e->ready = false;
 }
 
+// The batched pair launch takes the FP32 P3M contexts with the additive pair factor, the group size that most
+// of their particles have and the list length of its kernel (work items coded (slot << 24) | item).  The others
+// launch their own: one kernel for any form and size holds six times the code and took 30 to 60 % longer than
+// the contexts' own launches (48 simulations of 48^3 to 96^3: 367 million particles a second against 498
+// with the kernel of their kind).
+bool batchable(const p3m_ctx *c)
+{
+    return c->precision == P3M_PREC_MIXED && c->short_range && c->max_work < (1u << 24) && c->pair_factor.additive;
+}
+
+// Chooses the contexts of the batched launch.  Their tuning may have changed since the last choice (lists of
+// another length or size add in another order): called before every run that batches.
+cudaError_t choose_batched(p3m_ensemble *e)
+{
+    auto tuned = [](const p3m_ctx *c) { return batchable(c) && (pair_group(c) != 16 || c->tile_blocks == 5); };
+    int64_t share[17] = {0};
+    for (int i = 0; i < e->n; ++i)
+        if (tuned(e->c[i])) share[pair_group(e->c[i])] += e->c[i]->g.n;
+    const int group = share[16] >= share[8] && share[16] >= share[4] ? 16 : share[8] >= share[4] ? 8 : 4;
+    bool same = group == e->group;
+    std::vector<int> slot(e->n);
+    std::vector<const uint32_t *> nw;
+    size_t cap = 0;
+    for (int i = 0; i < e->n; ++i) {
+        p3m_ctx *c = e->c[i];
+        const bool ok = tuned(c) && pair_group(c) == group && nw.size() < 255;
+        slot[i] = ok ? (int)nw.size() : -1;
+        same = same && slot[i] == e->slot[i];
+        if (!ok) continue;
+        e->base[nw.size()] = cap;
+        cap += c->max_work;
+        nw.push_back(c->n_work);
+    }
+    if (same) return cudaSuccess;
+    drop_graphs(e);
+    cudaError_t err = cudaStreamSynchronize(e->parent);
+    if (err == cudaSuccess && !nw.empty())
+        err = cudaMemcpy((void *)e->nwork, nw.data(), sizeof(uint32_t *) * nw.size(), cudaMemcpyHostToDevice);
+    e->group = group;
+    e->nb = (int)nw.size();
+    e->cap = cap;
+    memcpy(e->slot, slot.data(), sizeof(int) * e->n);
+    return err;
+}
+
 }  // namespace
 
 extern "C" int p3m_ensemble_create(p3m_ensemble **out, p3m_ctx *const *ctxs, int n, int own_streams)
@@ -397,49 +445,32 @@ extern "C" int p3m_ensemble_create(p3m_ensemble **out, p3m_ctx *const *ctxs, int
         p3m_ensemble_free(e);
         return p3m_fail_global(P3M_ECUDA, "p3m_ensemble_create: %s", cudaGetErrorString(err));
     }
-    // batched pair launch over the FP32 P3M contexts (work items coded (slot << 24) | item): those with the
-    // additive pair factor and the group size that most particles have.  The others launch their own: one
-    // kernel for any form and size holds six times the code and took 30 to 60 % longer than the
-    // contexts' own launches (48 simulations of 48^3 to 96^3: 367 million particles a second against
-    // 498 with the kernel of their kind).
-    auto batchable = [](const p3m_ctx *c) {
-        return c->precision == P3M_PREC_MIXED && c->short_range && c->max_work < (1u << 24) && c->pair_factor.additive;
-    };
-    int64_t share[17] = {0};
-    for (int i = 0; i < n; ++i)
-        if (batchable(ctxs[i])) share[pair_group(ctxs[i])] += ctxs[i]->g.n;
-    e->group = share[16] >= share[8] && share[16] >= share[4] ? 16 : share[8] >= share[4] ? 8 : 4;
     e->slot = (int *)malloc(sizeof(int) * n);
     e->base = (size_t *)calloc(n, sizeof(size_t));
     if (!e->slot || !e->base) err = cudaErrorMemoryAllocation;
-    std::vector<const uint32_t *> nw;
+    size_t cap = 0;
+    int nb = 0;
     for (int i = 0; i < n && err == cudaSuccess; ++i) {
-        p3m_ctx *c = ctxs[i];
-        const bool ok = batchable(c) && pair_group(c) == e->group && e->nb < 255;
-        e->slot[i] = ok ? e->nb : -1;
-        if (ok) {
-            e->base[e->nb] = e->cap;
-            e->cap += c->max_work;
-            nw.push_back(c->n_work);
-            ++e->nb;
-        }
+        e->slot[i] = -1;
+        if (!batchable(ctxs[i])) continue;
+        cap += ctxs[i]->max_work;
+        ++nb;
     }
-    if (err == cudaSuccess && e->nb > 0) {
-        const size_t tiles = (e->cap + P3M_SORT_TILE - 1) / P3M_SORT_TILE;
+    if (err == cudaSuccess && nb > 0) {
+        const size_t tiles = (cap + P3M_SORT_TILE - 1) / P3M_SORT_TILE;
         const size_t scan_n = 256 * tiles;
-        err = cudaMalloc((void **)&e->descs, sizeof(PairArgs) * e->nb);
-        if (err == cudaSuccess) err = cudaMalloc((void **)&e->nwork, sizeof(uint32_t *) * e->nb);
+        err = cudaMalloc((void **)&e->descs, sizeof(PairArgs) * nb);
+        if (err == cudaSuccess) err = cudaMalloc((void **)&e->nwork, sizeof(uint32_t *) * nb);
         for (int b = 0; b < 2 && err == cudaSuccess; ++b) {
-            err = cudaMalloc((void **)&e->gkey[b], 4 * e->cap);
-            if (err == cudaSuccess) err = cudaMalloc((void **)&e->gval[b], 4 * e->cap);
+            err = cudaMalloc((void **)&e->gkey[b], 4 * cap);
+            if (err == cudaSuccess) err = cudaMalloc((void **)&e->gval[b], 4 * cap);
         }
         if (err == cudaSuccess) err = cudaMalloc((void **)&e->gcounts, 4 * 256 * tiles);
         if (err == cudaSuccess) err = cudaMalloc((void **)&e->gaux, 4 * (scan_n / P3M_SORT_TILE + 4));
         if (err == cudaSuccess) err = cudaMalloc((void **)&e->gtotal, 16);
         if (err == cudaSuccess) err = cudaMalloc((void **)&e->gcursor, 16);
-        if (err == cudaSuccess)
-            err = cudaMemcpy((void *)e->nwork, nw.data(), sizeof(uint32_t *) * e->nb, cudaMemcpyHostToDevice);
         if (err == cudaSuccess) err = cudaEventCreateWithFlags(&e->after_pairs, cudaEventDisableTiming);
+        if (err == cudaSuccess) err = choose_batched(e);
     }
     e->batched = false;  // no faster than per-context branches on uneven ensembles, which
                          // keep the contexts independent
@@ -485,6 +516,8 @@ extern "C" int p3m_ensemble_set_fft_groups(p3m_ensemble *e, int enable)
 extern "C" int p3m_ensemble_set_batched(p3m_ensemble *e, int enable)
 {
     if (!e) return p3m_fail_global(P3M_EINVAL, "p3m_ensemble_set_batched: NULL ensemble");
+    const cudaError_t err = choose_batched(e);
+    if (err != cudaSuccess) return p3m_fail_global(P3M_ECUDA, "p3m_ensemble_set_batched: %s", cudaGetErrorString(err));
     const bool want = enable && e->nb >= 1;
     if (want != e->batched) drop_graphs(e);
     e->batched = want;
@@ -512,7 +545,11 @@ extern "C" int p3m_ensemble_run(p3m_ensemble *e, const double *a_list, int n_ste
             c->forces_valid = true;
         }
     }
-    if (!use_graph && e->batched) {
+    if (e->batched) {
+        const cudaError_t err = choose_batched(e);
+        if (err != cudaSuccess) return p3m_fail_global(P3M_ECUDA, "p3m_ensemble_run: %s", cudaGetErrorString(err));
+    }
+    if (!use_graph && batching(e)) {
         for (int k = 0; k < n_steps; ++k) {
             int rc = ens_step(e, a_list[k], a_list[k + 1] - a_list[k], false);
             if (rc) return rc;

@@ -95,6 +95,7 @@ struct p3m_ctx {
     float4 *block_box;  // per 32-slot block of the sorted order: lo, hi (FP32, absolute)
     uint32_t *relq;     // fixed-point coordinates (kFixBits), per 32-slot block x[32] y[32] z[32]
     int tile_blocks;    // FP32 pair kernel: its list is evaluated every 32 tile_blocks entries (3 or 5)
+    int list_group;     // particles that share a list; 0: by the particle number (pair_group)
 
     // sort
     uint32_t *keys, *keys_alt, *vals, *vals_alt;
@@ -213,6 +214,7 @@ enum {
 // 107 / 69 / 70, 32^3 109 / 95 / 119 (clustered 310 / 197 / 213), 40^3 143 / 150, 64^3 445 / 514.
 inline int pair_group(const p3m_ctx *c)
 {
+    if (c->list_group) return c->list_group;
     const int64_t warps = (int64_t)c->num_sms * P3M_PAIR_CTAS;
     return c->g.n >= 16 * warps ? 16 : c->g.n >= 8 * warps ? 8 : 4;
 }
