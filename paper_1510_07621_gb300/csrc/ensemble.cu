@@ -761,8 +761,8 @@ extern "C" int p3m_autotune(p3m_ctx *c, int *sub_bits_out, double *ms_out)
     int rc = key_current(c);
     if (!rc) rc = evaluate(c, 0.0, nullptr);
     if (rc) return rc;
-    // then the FP32 pair kernel's tile length at that key (3 or 5 blocks of 32 j particles)
-    if (c->precision == P3M_PREC_MIXED && c->short_range) {
+    // then the FP32 pair kernel's list length at that key (96 or 160 entries; lists of 4 and 8 have one length)
+    if (c->precision == P3M_PREC_MIXED && c->short_range && pair_group(c) == 16) {
         double best_t = 1e300;
         int best_tb = c->tile_blocks;
         CK(cudaEventCreate(&e0));
