@@ -100,10 +100,13 @@ typedef struct {
     uint64_t launches;    /* kernels this library launched on the stream since p3m_init
                              (cuFFT's own kernels not included)                             */
     uint64_t pair_warp_j[3]; /* pair kernel work since p3m_init, in warp-iterations over one
-                             j particle (32 pair slots each): [0] 0, [1] j's tested against a
-                             group of i's, [2] those evaluated (FP64 mode: steps of 32 pairs)    */
+                             j particle (32 pair slots each): [0] in blocks entirely inside
+                             r_c of a group of i's (evaluated untested; FP64 mode: 0), [1] j's
+                             tested against a group, [2] tested ones that were evaluated (FP64
+                             mode: steps of 32 pairs)                                          */
     uint64_t pair_blocks_culled; /* 32-particle j blocks skipped by the bounding-box test     */
-    uint64_t pair_tiles[2];  /* [0] j lists (FP64 mode: rounds of masks) evaluated, [1] 0      */
+    uint64_t pair_tiles[2];  /* batches of up to 32 j blocks tested against a group's bounding
+                                box; [1] of them entirely culled                             */
     int64_t n;            /* number of particles                                            */
     int32_t n_cells_side; /* chaining cells per side n_c                                    */
     int32_t max_cell_count; /* most particles in one chaining cell (last sort)              */

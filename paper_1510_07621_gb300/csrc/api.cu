@@ -1060,7 +1060,7 @@ extern "C" int p3m_diagnostics(p3m_ctx *c, p3m_diag *out)
     out->pairs = pc[0];
     out->pairs_total = pc[1];
     out->pair_warp_j[0] = pc[2];
-    out->pair_warp_j[1] = pc[3];
+    out->pair_warp_j[1] = pc[3] - pc[2];  // (near, less the ones that need no test)
     out->pair_warp_j[2] = pc[4];
     out->pair_blocks_culled = pc[5];
     out->pair_tiles[0] = pc[6];

@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(32)
     const float kscale = (float)(kSplitTab64 / g.r_c);
     const int nc = g.n_c;
     const float cell_f = (float)g.cs;
-    unsigned long long st_pairs = 0, st_tested = 0, st_steps = 0, st_culled = 0, st_rounds = 0;
+    unsigned long long st_pairs = 0, st_tested = 0, st_steps = 0, st_culled = 0, st_rounds = 0, st_empty = 0;
 
     for (;;) {
         uint32_t unit = 0;
@@ -125,13 +125,15 @@ __global__ void __launch_bounds__(32)
                     fz = (float)(int)(__ldg(qi + 64) - fr.ctr[2]) * kFixUnit;
         const double xi = pos[i], yi = pos[n + i], zi = pos[2 * n + i];
         double ax = 0.0, ay = 0.0, az = 0.0;
-        uint32_t pairs = 0, steps = 0, rounds = 0, n_live = 0;
+        uint32_t pairs = 0, steps = 0, rounds = 0, n_empty = 0, n_live = 0;
 
         for (uint32_t base = 0; base < blocks.y;) {
             int ne = 0;
             for (; base < blocks.y && ne + 32 <= kEntries64; base += 32) {
                 const int nl = live_blocks(base + lane, blocks.y, seg, block_box, fr, cell_f, rcull2, live);
                 n_live += nl;
+                ++rounds;
+                n_empty += nl == 0;
                 for (int k = 0; k < nl; ++k) {
                     const LiveBlock S = live.at[k];
                     const uint32_t w = S.word, in = live.slots[k];
@@ -198,7 +200,6 @@ __global__ void __launch_bounds__(32)
                 pairs += acc ? 1u : 0u;
                 ++steps;
             }
-            ++rounds;
             __syncwarp();  // the masks are rewritten by the next round
         }
         // the four lanes of a particle, always in the same order
@@ -220,6 +221,7 @@ __global__ void __launch_bounds__(32)
         st_steps += steps;
         st_culled += blocks.y - n_live;
         st_rounds += rounds;
+        st_empty += n_empty;
     }
     if (lane == 0) {
         if (st_pairs) {
@@ -230,6 +232,7 @@ __global__ void __launch_bounds__(32)
         if (st_steps) atomicAdd(pair_count + 4, st_steps);
         if (st_culled) atomicAdd(pair_count + 5, st_culled);
         if (st_rounds) atomicAdd(pair_count + 6, st_rounds);
+        if (st_empty) atomicAdd(pair_count + 7, st_empty);
     }
 }
 
@@ -328,7 +331,7 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
     __shared__ double sum[6][32];  // per lane: x, y, z of its first particle, then of its second
     __shared__ PairSeg seg[kPairSegs];
     __shared__ LiveBlocks live;
-    __shared__ unsigned long long stat[6];
+    __shared__ unsigned long long stat[7];  // pairs, tested, listed, culled, batches, empty batches, deep
     __shared__ __align__(16) PairArgs sA;  // the current work item's context
     const PairArgs &A = sA;
 
@@ -345,7 +348,7 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
         const uint64_t *from = (const uint64_t *)src;
         uint64_t *to = (uint64_t *)&sA;
         for (int w = lane; w < kArgWords; w += 32) to[w] = from[w];
-        if (lane < 6) stat[lane] = 0ull;
+        if (lane < 7) stat[lane] = 0ull;
         __syncwarp();
         kfac = A.kfac_dev ? *A.kfac_dev : A.kfac;
 #pragma unroll
@@ -358,8 +361,8 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
     // the counters gathered so far, into their context
     auto store_stat = [&]() {
         __syncwarp();
-        if (lane < 6 && stat[lane]) {
-            atomicAdd(A.pair_count + lane + (lane ? 2 : 1), stat[lane]);
+        if (lane < 7 && stat[lane]) {
+            atomicAdd(A.pair_count + (lane == 6 ? 2 : lane + (lane ? 2 : 1)), stat[lane]);
             if (lane == 0) atomicAdd(A.pair_count, stat[0]);
         }
     };
@@ -525,6 +528,7 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
             for (uint32_t base = t0; base < t1; base += 32) {
                 const int nl = live_blocks(base + lane, t1, seg, A.block_box, fr, A.fac.length, A.rcull2, live, A.rin2);
                 n_live += nl;
+                if (nl == 0 && lane == 0) ++stat[5];
                 // the next block's coordinates are loaded while the current one is tested
                 uint32_t xn = 0, yn = 0, zn = 0;
                 auto fetch = [&](int k) {
@@ -551,7 +555,7 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
                             eval_deep(own, kChunk);
                             __syncwarp();
                             fill_deep = 0;
-                            n_list += kChunk;
+                            if (lane == 0) stat[6] += kChunk / 32 * kG;
                             if (++n_chunks % kFlushChunks == 0) flush();
                         }
                         continue;
@@ -592,7 +596,8 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
             if (fill_deep) eval_deep(own, fill_deep);
             __syncwarp();
             flush();
-            n_list += fill + fill_deep;
+            n_list += fill;
+            if (fill_deep && lane == 0) stat[6] += fill_deep / 32 * kG;
             fill = fill_deep = 0;
         };
         walk(std::true_type{}, 0u, blocks.x);
@@ -619,10 +624,10 @@ __global__ void __launch_bounds__(32, P3M_PAIR_CTAS)
         const uint32_t pairs = __reduce_add_sync(0xffffffffu, my);
         if (lane == 0) {
             stat[0] += pairs;
-            stat[1] += (n_live * kG);              // j's tested against the group's box, in slots of 32
-            stat[2] += (n_list * kG + 16) / 32;    // list entries evaluated, the same
+            stat[1] += n_live * kG;              // j's of the blocks near the group (deep ones too), in slots of 32
+            stat[2] += (n_list * kG + 16) / 32;  // list entries evaluated after a test, the same
             stat[3] += blocks.y - n_live;
-            stat[4] += n_chunks + 2;
+            stat[4] += (blocks.x + 31) / 32 + (blocks.y - blocks.x + 31) / 32;
         }
         __syncwarp();
     }
