@@ -42,14 +42,15 @@ METRIC = "P3M particle-updates/s"
 UNIT = "particle-updates/s"
 # algorithmic FP32 flops per accepted pair of the short-range sum: the FP32 arithmetic of the
 # FP32 kernel's accepted-pair sequence, FMA = 2: d 3 FADD; r^2 + eps^2 3 FFMA; s + b FADD; the
-# (1 - t)/r^2 term FFMA; s^2 FMUL; its product and the constant FFMA; the cubic in t 3 FFMA;
-# a += f d 3 FFMA  ->  11 FFMA + 5 FADD/FMUL = 27 flops (rsqrt and ex2 run on the MUFU pipe and
-# are not counted)
-FLOPS_PER_PAIR = 27
-# the same for the FP64 kernel: d 6 DADD (difference plus image); r^2 DMUL + 2 DFMA; r^2 + eps^2
-# DADD; r^3 = r^2 (r^2 rsqrt(r^2)) 2 DMUL; tau DFMA; the degree-18 Horner chain 18 DFMA;
-# g DFMA; s^3 and g s^3 3 DMUL; a += f d 3 DFMA  ->  25 DFMA + 13 DADD/DMUL = 63 flops
-FLOPS_PER_PAIR_FP64 = 63
+# (1 - t)/r^2 term FFMA; s^2 FMUL; the next softening term FFMA; its product and the constant FFMA;
+# the cubic in t 3 FFMA; a += f d 3 FFMA  ->  12 FFMA + 5 FADD/FMUL = 29 flops (rsqrt and ex2 run on
+# the MUFU pipe and are not counted)
+FLOPS_PER_PAIR = 29
+# the same for the FP64 kernel: d 3 DADD (pairs that cross a face add 3); r^2 DMUL + 2 DFMA;
+# r^2 + eps^2 DADD; two reciprocal square roots from the hardware's approximation, each 2 DMUL + 3 DFMA;
+# r DMUL; t DFMA; the degree-7 Horner chain of g 7 DFMA; g s^3 3 DMUL; a += f d 3 DFMA
+# ->  19 DFMA + 13 DADD/DMUL = 51 flops
+FLOPS_PER_PAIR_FP64 = 51
 WORKLOAD = dict(n_p=128, mesh=128, box=200.0, r_s_cells=1.25, cutoff=4.5, softening=0.02,
                 a_begin=0.02, a_end=1.0, setup_steps=64, seed=1512)
 WORKLOAD_NAME = ("clustered_128: 128^3 particles, 128^3 mesh, box 200 Mpc/h, r_s 1.25 cells, "
