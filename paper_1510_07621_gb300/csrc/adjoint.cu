@@ -440,9 +440,9 @@ __global__ void __launch_bounds__(32)
 // s^4 is never formed: (2 q + ..) s^2 times s^2 (d.w) stays finite for close pairs without softening.
 // r = 0 pairs are selected out (their w need not vanish for coincident particles); only the row of the
 // own cell can hold them.  Before, all 32 lanes met every j of a tested block with 40 FP32 operations
-// and three 8-cycle MUFU operations per pair (34 and one here).  128^3 near-uniform, one call with the
-// mesh part: 9.35 -> 6.47 ms, the pair part 7.6 -> 5.3.  What bounds it: of 137 cycles per 32 accepted
-// pairs and scheduler, 111 are the evaluation (52 per 32 slots, 47 % of them accepted).  8 or 32
+// and three 8-cycle MUFU operations per pair (36 and one here).  128^3 near-uniform, one call with the
+// mesh part: 9.37 -> 6.71 ms, the pair part 7.6 -> 5.5.  What bounds it: of 143 cycles per 32 accepted
+// pairs and scheduler, 117 are the evaluation (55 per 32 slots, 47 % of them accepted).  8 or 32
 // particles per group, 18 or 20 CTAs per SM and lists of 192 are within 2 % or slower.
 constexpr int kVjpChunk = 128, kVjpTerms = 80;  // FP32 terms per partial sum before it joins the FP64 sum
 constexpr float kVjpTiny = 1e-24f, kVjpFar = 1e6f;

@@ -210,8 +210,9 @@ enum {
 
 // Particles that share one list of the FP32 pair kernels: the most of 16, 8 and 4 that gives every resident
 // warp a group (smaller lists cost more tests per pair, but a group is the least a warp can take: few
-// particles leave most warps without one).  Force kernel, 16 / 8 / 4: 17^3 particles 77 / 51 / 40 us, 24^3
-// 107 / 69 / 70, 32^3 109 / 95 / 119 (clustered 310 / 197 / 213), 40^3 143 / 150, 64^3 445 / 514.
+// particles leave most warps without one).  Pair phase, 16 / 8 / 4, about 180 particles per cell: 17^3 particles
+// 92 / 63 / 47 us, 24^3 113 / 72 / 78, 32^3 113 / 102 / 135 (clustered 324 / 197 / 250), 40^3 145 / 160 / 244,
+// 64^3 465 / 555 / 989.
 inline int pair_group(const p3m_ctx *c)
 {
     if (c->list_group) return c->list_group;

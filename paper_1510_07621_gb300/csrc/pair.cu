@@ -247,8 +247,8 @@ __global__ void __launch_bounds__(32)
 //      the group's box; the accepted ones are appended to a list in shared memory (ballot and
 //      prefix count), as coordinates relative to the group's centre.  A deep block (all its slots
 //      within the cutoff of the whole group: most of a halo's own pairs) goes untested into a list
-//      of its own, whose evaluation needs no cutoff (clustered 9.8 -> 8.8 ms; near-uniform sets
-//      have hardly any: 3.27 -> 3.28).
+//      of its own, whose evaluation needs no cutoff (by 10 % of the clustered set's time; near-uniform
+//      sets have hardly any).
 //   3. Every 32 kChunkBlocks entries the list is evaluated: a lane owns two particles i and takes
 //      every (64/kG)-th pair of consecutive entries, two entries at once in packed f32x2
 //      arithmetic, so that one 8-byte load per coordinate serves four pair slots.
@@ -257,10 +257,10 @@ __global__ void __launch_bounds__(32)
 // instructions were tests and votes.  The list holds 47 % accepted slots at kG = 16 (58 % at 8,
 // 39 % at 32: the union of the cutoff spheres grows with the group), there are no votes between
 // pairs, and a test sequence serves 32 candidates of the whole group.  Measured at 128^3 (one
-// evaluation, before / after): near-uniform 5.23 / 3.28 ms, clustered 12.3 / 8.8 ms.
-// What bounds it now: of 84 cycles per 32 accepted pairs and scheduler, 59 are the evaluation
-// (28 per 32 slots; two FP32 operations with three distinct registers already take three cycles
-// of register bandwidth, and the same mix of 16 packed operations, 2 rsqrt and 2 ex2 alone runs
+// evaluation, before / after): near-uniform 5.21 / 3.44 ms, clustered 13.0 / 10.1 ms.
+// What bounds it now: of 86 cycles per 32 accepted pairs and scheduler, 61 are the evaluation
+// (29 per 32 slots; two FP32 operations with three distinct registers already take three cycles
+// of register bandwidth, and a mix of 16 packed operations, 2 rsqrt and 2 ex2 alone runs
 // at 20.5), 19 the candidate tests and 6 the set-up of groups.  16 particles per group
 // and 18 CTAs per SM: 8, 32 and 16, 20, 24 are within 6 % or slower on both sets.  Two lists of 16 (or
 // four of 8) filled by one pass over the candidates save a third of the tests but cost as much in
